@@ -58,6 +58,7 @@ constexpr int kMinSpanParticles = 1024;
 constexpr int kMaxSpanParticles = 1 << 24;
 constexpr int kMaxInstances = 65535;  // grid y of the per-instance prefix pass
 constexpr int kGraphSteps = 16;       // steps per replay of the captured graph (even)
+constexpr int kResidentSteps = 512;   // steps per resident launch, at most
 
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
@@ -145,6 +146,10 @@ dsmc_status check_options(const dsmc_options* o) {
   return DSMC_OK;
 }
 
+bool names_partition(const dsmc_options& o) {
+  return o.span_particles || o.cta_warps || o.span_rows;
+}
+
 struct DeviceGuard {
   int prev = -1;
   explicit DeviceGuard(int dev) {
@@ -212,6 +217,7 @@ struct Inst {
   long long step = 0, n_samples = 0;
   int open_top = 0;  // y = 1 an open Chapman-Enskog interface
   float u_top = 0.0f, p_top = 0.0f;
+  int cut[kResidentMaxCluster + 1] = {};  // slot shares of the CTAs of a resident cluster
 };
 
 // Sizes of the device arrays of a handle.
@@ -336,6 +342,7 @@ void dsmc::set_last_error(const std::string& msg) { g_last_error = msg; }
 
 struct dsmc_sim {
   int device = 0;
+  int sms = 1;  // of the device
   bool pool = false;  // instances may be added and removed
   dsmc_options opt{};
   std::vector<Inst> inst;  // by id
@@ -369,6 +376,11 @@ struct dsmc_sim {
   std::vector<InstParams> tab, adm_tab;
   std::vector<int> span_inst, adm_span, span_order;
   bool tab_dirty = true, spans_dirty = true;
+  // Cluster-resident steps (dsmc_resident.cu): the launch's shape, or cl = 0 when the
+  // handle's steps take the span passes.
+  ResidentLaunch res{};
+  bool res_dirty = true;
+  bool span_passes = false;  // the caller's options name a partition, or it is being tuned
   // CUDA graph of kGraphSteps consecutive steps, replayed by dsmc_step when
   // options.graph is set.  Its kernels read the global step from gstep_dev, which the
   // last prefix kernel of each step advances.
@@ -508,7 +520,7 @@ void set_partition(dsmc_sim* h, int target) {
   h->max_spans = ms;
   h->part_total = np;
   set_span_order(h);
-  h->tab_dirty = h->spans_dirty = true;
+  h->tab_dirty = h->spans_dirty = h->res_dirty = true;
   h->graph_valid = false;
 }
 
@@ -550,6 +562,7 @@ InstParams instance_params(const dsmc_sim* h, int id, int span_base) {
   a.open_top = x.open_top;
   a.u_top = x.u_top;
   a.p_top = x.p_top;
+  std::copy(x.cut, x.cut + kResidentMaxCluster + 1, a.cut);
   return a;
 }
 
@@ -720,13 +733,14 @@ dsmc_status admit_fresh(dsmc_sim* h) {
   return DSMC_OK;
 }
 
-// Advances every active instance's counters for one step.
-void count_step(dsmc_sim* h) {
-  h->gstep += 1;
+// Advances every active instance's counters for n steps.
+void count_steps(dsmc_sim* h, int n) {
+  h->gstep += n;
   for (int id : h->order) {
     Inst& x = h->inst[id];
-    x.step += 1;
-    if (x.step >= h->opt.sample_start) x.n_samples += 1;
+    const long long from = std::max(x.step + 1, h->opt.sample_start);  // first sampled step
+    x.step += n;
+    x.n_samples += std::max(0LL, x.step - from + 1);
   }
 }
 
@@ -816,16 +830,136 @@ dsmc_status capture_graph(dsmc_sim* h) {
 }
 
 dsmc_status step_once(dsmc_sim* h) {
-  count_step(h);
+  count_steps(h, 1);
   dsmc_status s = upload_tables(h);
   if (s != DSMC_OK) return s;
   return run_pass(h, false);
+}
+
+// Shares of an instance's slots for the cl CTAs of its cluster, of about equal cost: a
+// particle at y costs 1 + 1.5 h(y), h its expected wall hits in the step (as in
+// set_span_order; 1.5 is the measured extra cost of a hit here, where a CTA's wall hits are
+// flown by all its warps).  With equal shares the CTAs next to the walls took 64,000 cycles
+// of a 67,000-cycle step of a 100,000-particle run and the others 46,000 (Kn = 0.5); with
+// these, 49,000 and 45,000 of 52,000.  The cost's integral is taken at 64 points and
+// inverted linearly.  Returns the largest share.
+int set_cuts(Inst& x, int cl) {
+  constexpr int kPoints = 64;
+  const double dt = x.p.dt, w = 1.5;
+  auto ierfc = [&](double y) {  // integral of erfc(t / dt) over [0, y]
+    const double u = y / dt;
+    return y * std::erfc(u) + dt * (1.0 - std::exp(-u * u)) / std::sqrt(M_PI);
+  };
+  const double whole = ierfc(1.0);
+  double cost[kPoints + 1];
+  for (int i = 0; i <= kPoints; ++i) {
+    const double y = (double)i / kPoints;
+    cost[i] = y + 0.5 * w * (ierfc(y) + whole - ierfc(1.0 - y));
+  }
+  int share = 0, i = 0;
+  x.cut[0] = 0;
+  for (int r = 1; r <= cl; ++r) {
+    const double target = cost[kPoints] * r / cl;
+    while (i < kPoints - 1 && cost[i + 1] < target) ++i;
+    const double y = (i + (target - cost[i]) / (cost[i + 1] - cost[i])) / kPoints;
+    const long long at = r == cl ? x.N : (long long)(y * (double)x.N);
+    x.cut[r] = (int)std::min(x.N, std::max<long long>(x.cut[r - 1], at));
+    share = std::max(share, x.cut[r] - x.cut[r - 1]);
+  }
+  return share;
+}
+
+// Decides whether the handle's steps run cluster-resident (dsmc_resident.cu) and with how
+// many CTAs per instance.  Options that name a partition of the span passes keep those, as
+// does profiling, which times their kernels; a pool's members come and go between calls.
+//
+// One run: 16 CTAs whenever its share fits a CTA's shared memory (up to ~110,000
+// particles; us per step against the span passes under graph replay: 2,250 particles 7.2 /
+// 20.5, 20,000 11.4 / 22.5, 100,000 24-26 / 26-34).
+// A batch: as many CTAs per instance as give shares of at most kResidentShare particles and
+// fill the SMs twice, as long as an instance then fits 16 CTAs and the launch is not many
+// waves long (64 x 2,250 particles: 11 us per step against 30; 64 x 10,000: 28 / 48;
+// 64 x 20,000: 45 / 70; 128 x 20,000, 1,024 CTAs: 87 / 95; beyond that the span passes,
+// which spread every instance over all SMs, are as fast: 256 x 20,000, 161 / 153;
+// 24 x 100,000, 137 / 85).
+constexpr int kResidentShare = 2600;
+
+void plan_resident(dsmc_sim* h) {
+  h->res = ResidentLaunch{};
+  h->res_dirty = false;
+  const dsmc_options& o = h->opt;
+  if (h->pool || o.profile || h->span_passes) return;
+  long long n_max = 0;
+  for (int id : h->order) n_max = std::max(n_max, h->inst[id].N);
+  ResidentLaunch R{};
+  R.n_inst = h->n_inst();
+  R.cl = kResidentMaxCluster;
+  if (R.n_inst > 1) {
+    R.cl = 2;
+    while (R.cl < kResidentMaxCluster &&
+           (n_max > (long long)kResidentShare * R.cl || R.n_inst * 2 * R.cl <= 2 * h->sms))
+      R.cl *= 2;
+    if (n_max > (long long)kResidentShare * R.cl) return;
+    if ((long long)R.n_inst * R.cl > (R.cl == 16 ? 512 : 1024)) return;
+  }
+  if (n_max / R.cl > 30000) return;  // local slots are 16-bit; a share this large never fits
+  R.max_cells = h->max_cells;
+  int share = 0;
+  for (int id : h->order) share = std::max(share, set_cuts(h->inst[id], R.cl));
+  R.range_cap = share + h->cap();
+  R.list_cap = R.range_cap / o.group_size + std::min(R.max_cells, R.range_cap) + 2;
+  R.own_cap = (R.max_cells + R.cl - 1) / R.cl;
+  const size_t smem = resident_smem_layout(R.max_cells, R.range_cap, R.list_cap, R.own_cap, R.cl,
+                                           resident_warps(R.n_inst > 1))
+                          .total;
+  if (smem > kResidentSmemMax) return;
+  int clusters = 0;
+  if (resident_clusters(R.cl, smem, R.n_inst > 1, o.accum == DSMC_ACCUM_FP64, &clusters) !=
+          cudaSuccess ||
+      clusters < 1) {
+    cudaGetLastError();
+    return;
+  }
+  h->res = R;
+  h->tab_dirty = true;  // the instance table carries the cuts
+}
+
+// n steps of a resident launch.
+dsmc_status step_resident(dsmc_sim* h, int n) {
+  ResidentLaunch R = h->res;
+  R.tab = h->tab_dev;
+  R.n_steps = n;
+  R.gstep = h->gstep + 1;
+  R.parity_rec = h->cur;
+  R.parity_off = h->ocur;
+  R.parity_smax = h->scur;
+  DSMC_CUDA(launch_resident(h->P[0], h->P[1], h->off[0], h->off[1], h->smax[0], h->smax[1],
+                            h->ncand, h->nacc, h->acc, h->tab[0], R,
+                            h->opt.accum == DSMC_ACCUM_FP64, h->err, h->stream()),
+            "resident steps");
+  h->cur ^= n & 1;
+  h->ocur ^= n & 1;
+  h->scur ^= n & 1;
+  count_steps(h, n);
+  return DSMC_OK;
 }
 
 dsmc_status step_n(dsmc_sim* h, int n_steps) {
   dsmc_status s;
   if ((s = admit_fresh(h)) != DSMC_OK) return s;
   int it = 0;
+  if (h->n_inst() > 0 && n_steps > 0) {
+    if (h->res_dirty) plan_resident(h);
+    if (h->res.cl > 0) {
+      if ((s = upload_tables(h)) != DSMC_OK) return s;
+      while (it < n_steps) {
+        const int n = std::min(n_steps - it, kResidentSteps);
+        if ((s = step_resident(h, n)) != DSMC_OK) return s;
+        it += n;
+      }
+      return DSMC_OK;
+    }
+  }
   if (h->opt.graph && !h->opt.profile && h->n_inst() > 0) {
     while (n_steps - it >= kGraphSteps) {
       if ((s = upload_tables(h)) != DSMC_OK) return s;
@@ -834,7 +968,7 @@ dsmc_status step_n(dsmc_sim* h, int n_steps) {
       // The graph's first step runs at global step gstep + 1.
       DSMC_CUDA(launch_set_counter(h->gstep_dev, h->gstep + 1, h->stream()), "set step");
       DSMC_CUDA(cudaGraphLaunch(h->graph, h->stream()), "graph launch");
-      for (int k = 0; k < kGraphSteps; ++k) count_step(h);
+      count_steps(h, kGraphSteps);
       it += kGraphSteps;
     }
   }
@@ -937,11 +1071,14 @@ dsmc_status new_handle(const Capacity& C, const dsmc_options& opt, bool pool, vo
   // than 8-warp CTAs in the request loop).
   h->cta_warps = opt.cta_warps ? opt.cta_warps : (pool ? kAWarpsSmall : kAWarps);
   h->span_rows = opt.span_rows ? opt.span_rows : 1;
+  h->span_passes = names_partition(opt);
   h->ex_slots.reset(C.slots);
   h->ex_cells.reset(C.cells);
   h->ex_offs.reset(C.offs);
   h->ex_hist.reset(C.hist_ints);
   cudaError_t ce = cudaGetDevice(&h->device);
+  if (ce == cudaSuccess)
+    ce = cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device);
   if (ce != cudaSuccess) {
     delete h;
     return cuda_fail(ce, "cudaGetDevice");
@@ -1257,11 +1394,12 @@ dsmc_status dsmc_set_options(dsmc_handle h, const dsmc_options* opt) {
     if (s != DSMC_OK) return s;
   }
   h->opt = *opt;
+  h->span_passes = names_partition(*opt);
   for (int id : h->order) h->inst[id].p = ps[id];
   h->cta_warps = warps_use;
   h->span_rows = rows_use;
   if (target_use != h->span_target) set_partition(h, target_use);
-  h->tab_dirty = true;
+  h->tab_dirty = h->res_dirty = true;
   drop_graph(h);  // launch shapes or the stream may have changed
   return DSMC_OK;
 }
@@ -1296,6 +1434,8 @@ dsmc_status dsmc_autotune(dsmc_handle h, int steps_per_trial, int* best_span_par
   int best = h->span_target, best_warps = h->cta_warps, best_rows = h->span_rows;
   double best_ms = -1.0;
   dsmc_status r = DSMC_OK;
+  const bool span_passes = h->span_passes;
+  h->span_passes = h->res_dirty = true;  // the trials are of the span passes
   const int shapes[4][2] = {{kAWarps, 1}, {kAWarps, 2}, {kAWarpsSmall, 1}, {kAWarpsSmall, 2}};
   for (const auto& shape : shapes) {
     const int w = shape[0], rows = shape[1];
@@ -1336,6 +1476,8 @@ dsmc_status dsmc_autotune(dsmc_handle h, int steps_per_trial, int* best_span_par
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
+  h->span_passes = span_passes;
+  h->res_dirty = true;
   if (r != DSMC_OK) return r;
   h->cta_warps = best_warps;
   h->span_rows = best_rows;

@@ -108,6 +108,9 @@ struct InstParams {
   float smax0;  // initial (sigma g)_max / sigma_ref of every cell
   int open_top;        // 1: y = 1 is an open Chapman-Enskog interface
   float u_top, p_top;  // its bulk velocity and shear stress
+  // cluster-resident steps: CTA r takes the groups that start in slots
+  // [part_base + cut[r], part_base + cut[r + 1])
+  int cut[17];
 };
 
 // Dynamic shared memory of one collide/move CTA (byte offsets).
@@ -154,6 +157,77 @@ __host__ __device__ inline StepSmem step_smem_layout(int n_cells, int cps, int c
   L.total = o;
   return L;
 }
+
+// Many steps of small runs in one launch (dsmc_resident.cu): a cluster of `cl` CTAs per
+// instance.
+constexpr int kResidentWarps = 20;       // warps per CTA, one instance
+constexpr int kResidentWarpsBatch = 12;  // several instances, two CTAs per SM
+constexpr int kResidentMaxCluster = 16;   // entries of InstParams::cut less one
+constexpr size_t kResidentSmemMax = 225 * 1024;
+
+inline int resident_warps(bool batch) { return batch ? kResidentWarpsBatch : kResidentWarps; }
+
+struct ResidentLaunch {
+  int n_inst;
+  const InstParams* tab;  // device, n_inst entries (batched launches)
+  int cl;                 // CTAs per cluster
+  int n_steps;
+  long long gstep;        // global step number of the first step
+  int parity_rec, parity_off, parity_smax;  // the buffers that hold the state now
+  int max_cells;          // largest n_cells of the instances
+  int range_cap;          // slots of a CTA, at most
+  int list_cap;           // collision groups of a CTA, at most
+  int own_cap;            // cells owned by a CTA, at most
+};
+
+// Dynamic shared memory of one CTA (byte offsets).
+struct ResidentSmem {
+  size_t rec, key, list, rows, tot, off, base, smax, cfix, csum, cgmax, total;
+  size_t rows_bytes;
+};
+
+__host__ __device__ inline ResidentSmem resident_smem_layout(int n_cells, int range_cap,
+                                                             int list_cap, int own_cap, int cl,
+                                                             int warps) {
+  ResidentSmem L;
+  size_t o = 0;
+  L.rec = o;
+  o += (size_t)range_cap * 16;
+  L.cfix = o;
+  o += (size_t)own_cap * 12 * 8;
+  L.csum = o;
+  o += (size_t)own_cap * kNMom * 8;
+  L.list = o;
+  o += (size_t)list_cap * 8;
+  L.cgmax = o;
+  o += (size_t)own_cap * 2 * 4;
+  L.key = o;
+  o += (size_t)range_cap * 4;
+  // counts per warp and cell; before them, the queue of wall hits (16-bit local slots),
+  // 4,096 of them if the counts are smaller than that
+  const size_t counts = (size_t)warps * n_cells * 4;
+  const size_t queue = range_cap < 4096 ? ((size_t)range_cap * 2 + 64) : 8192;
+  L.rows = o;
+  L.rows_bytes = step_align(counts > queue ? counts : queue, 4);
+  o += L.rows_bytes;
+  L.tot = o;
+  o += (size_t)cl * n_cells * 4;
+  L.off = o;
+  o += 2 * ((size_t)n_cells + 1) * 4;
+  L.base = o;
+  o += (size_t)n_cells * 4;
+  L.smax = o;
+  o += (size_t)n_cells * 4;
+  L.total = step_align(o, 128);
+  return L;
+}
+
+// Clusters of `cl` CTAs with `smem` bytes each that fit on the device at once (0: none).
+cudaError_t resident_clusters(int cl, size_t smem, bool batch, bool f64, int* clusters);
+cudaError_t launch_resident(float4* P0, float4* P1, int* off0, int* off1, float* smax0,
+                            float* smax1, unsigned long long* ncand, unsigned long long* nacc,
+                            double* acc, const InstParams& one, const ResidentLaunch& L,
+                            bool f64, int* err, cudaStream_t st);
 
 cudaError_t launch_init(float4* P, int N, int ppc, float ncf, uint32_t k0, uint32_t k1,
                         int* err, cudaStream_t st);

@@ -1,0 +1,515 @@
+// dsmc_resident.cu -- many steps of small runs in one launch.
+//
+// A small run's step is bound by launches and by the latency of its passes, not by work:
+// 20,000 particles through the span passes of dsmc_step.cu take 22 us per step (three
+// launches under graph replay, each a cold start of a CTA's worth of dependent phases),
+// against about 2 us of instruction issue on 16 SMs.  Here a thread-block cluster owns an
+// instance and runs all the steps of a call: particles, counters and prefixes pass between
+// its CTAs through L2 and distributed shared memory, with two hardware cluster barriers
+// per step instead of kernel boundaries.  Instances do not depend on one another, so a
+// batch is one cluster per instance.
+//
+// A step, for CTA r of the cluster (identical arithmetic, operation for operation, to the
+// span passes; only the place where it happens differs):
+//   A  load its slots -- the collision groups that start in [r N / CL, (r+1) N / CL) --
+//      into shared memory; its warps take the groups one after another (moments, NTC
+//      candidates, moments, flight) and update them in place; then every warp ranks a
+//      contiguous part of the slots by new cell (running counts per warp and cell), and
+//      the CTA publishes its particles per cell.
+//      [cluster barrier]
+//   B  every CTA reads the others' counts: exclusive prefix over CTAs and cells gives the
+//      new cell offsets and the CTA's base in every cell; the cell's owner CTA adds the
+//      step's moment sums to the run's; each record goes to its sorted place in the other
+//      record buffer (global memory, L2-resident at these sizes).
+//      [cluster barrier]
+// Cell results (fixed-point moment totals, counters, largest relative speed) are integer
+// adds and maxima in the owner CTA's shared memory, so they do not depend on the order.
+#include <type_traits>
+
+#include "dsmc_collide.cuh"
+#include "dsmc_device.cuh"
+#include "dsmc_internal.h"
+
+namespace dsmc {
+
+namespace {
+
+// --- cluster primitives ---------------------------------------------------------------
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+
+// Barrier of all threads of the cluster; memory operations before it (shared, distributed
+// shared and global) are visible to the cluster's threads after it.
+__device__ __forceinline__ void cluster_barrier() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// The address of this CTA's shared-memory location `p` in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t peer_addr(const void* p, uint32_t rank) {
+  uint32_t a;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  return a;
+}
+
+__device__ __forceinline__ uint32_t peer_load(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
+
+__device__ __forceinline__ void peer_store(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+
+__device__ __forceinline__ void peer_add(uint32_t addr, unsigned long long v) {
+  asm volatile("red.relaxed.cluster.shared::cluster.add.u64 [%0], %1;" ::"r"(addr), "l"(v)
+               : "memory");
+}
+
+__device__ __forceinline__ void peer_max(uint32_t addr, uint32_t v) {
+  asm volatile("red.relaxed.cluster.shared::cluster.max.u32 [%0], %1;" ::"r"(addr), "r"(v)
+               : "memory");
+}
+
+}  // namespace
+
+template <bool kBatch, int kWarps, bool kF64>
+__global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
+    k_resident(float4* P0, float4* P1, int* off0, int* off1, float* smax0, float* smax1,
+               unsigned long long* ncand_all, unsigned long long* nacc_all, double* acc_all,
+               const InstParams one, const ResidentLaunch RL, int* err) {
+  using Acc = typename std::conditional<kF64, double, float>::type;
+  constexpr int kThreads = kWarps * 32;
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ InstParams sh_inst;
+  __shared__ int wsum[2][32];
+  __shared__ int bnd_slot[2], bnd_cell[2], bnd_group[2];  // first group of this CTA, and the end
+  __shared__ int n_groups_sh, next_group, n_hits;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const unsigned lt = (1u << lane) - 1u;
+  const int CL = RL.cl;
+  const int rank = (int)cluster_rank();
+  if constexpr (kBatch) {
+    const int* src = reinterpret_cast<const int*>(&RL.tab[blockIdx.x / CL]);
+    int* dst = reinterpret_cast<int*>(&sh_inst);
+    for (int i = tid; i < (int)(sizeof(InstParams) / 4); i += kThreads) dst[i] = src[i];
+    __syncthreads();
+  }
+  const InstParams& a = kBatch ? sh_inst : one;
+  const ResidentSmem L = resident_smem_layout(RL.max_cells, RL.range_cap, RL.list_cap,
+                                              RL.own_cap, RL.cl, kWarps);
+  float4* rec = reinterpret_cast<float4*>(smem + L.rec);        // this CTA's records
+  unsigned* key = reinterpret_cast<unsigned*>(smem + L.key);    // candidate masks, then ranks
+  int2* list = reinterpret_cast<int2*>(smem + L.list);          // groups: (cell, gi << 10 | gn)
+  int* rows = reinterpret_cast<int*>(smem + L.rows);            // counts per warp and cell
+  int* tot = reinterpret_cast<int*>(smem + L.tot);              // counts per CTA and cell
+  int* base = reinterpret_cast<int*>(smem + L.base);            // this CTA's first slot per cell
+  float* csmax = reinterpret_cast<float*>(smem + L.smax);       // (sigma g)_max per cell
+  // of the cells this CTA owns: the step's fixed-point sums, the run's moment sums, and the
+  // largest relative speed of even and odd steps
+  unsigned long long* cfix = reinterpret_cast<unsigned long long*>(smem + L.cfix);
+  double* csum = reinterpret_cast<double*>(smem + L.csum);
+  unsigned* cgmax = reinterpret_cast<unsigned*>(smem + L.cgmax);
+
+  const int n_cells = a.n_cells, G = a.G, mode = a.mode;
+  const int own = (n_cells + CL - 1) / CL;          // cells per owner CTA
+  const int own0 = rank * own;                      // first cell this CTA owns
+  const int own_n = max(0, min(own, n_cells - own0));
+  const int lo = a.part_base, hi = a.part_base + a.n_part;
+  // slots at which this CTA's and the next CTA's groups may start
+  const int B0 = lo + a.cut[rank], B1 = lo + a.cut[rank + 1];
+  unsigned long long* ncand = ncand_all + a.cell_base;
+  unsigned long long* nacc = nacc_all + a.cell_base;
+  double* acc = acc_all + (size_t)a.cell_base * kNMom;
+  long long istep = RL.gstep - a.step0;
+
+  int* off = reinterpret_cast<int*>(smem + L.off);  // this step's cell offsets
+  int* off_next = off + RL.max_cells + 1;
+  {
+    const int* g = (RL.parity_off ? off1 : off0) + a.off_base;
+    const float* s = (RL.parity_smax ? smax1 : smax0) + a.cell_base;
+    for (int c = tid; c <= n_cells; c += kThreads) off[c] = g[c];
+    for (int c = tid; c < n_cells; c += kThreads) csmax[c] = s[c];
+    for (int i = tid; i < own * 12; i += kThreads) cfix[i] = 0ull;
+    for (int i = tid; i < own_n * kNMom; i += kThreads) csum[i] = acc[(size_t)own0 * kNMom + i];
+    for (int i = tid; i < 2 * own; i += kThreads) cgmax[i] = 0u;
+  }
+  // The group boundaries of this CTA from cell offsets: boundary B falls into the cell
+  // c with first <= B < first + n; the CTA's groups begin with the cell's first group
+  // that starts at or after B, or with the next cell.
+  auto set_bound = [&](int k, int B, int c, int first, int n) {
+    if (B < first || B >= first + n) return;
+    const int i = (B - first + G - 1) / G;
+    const int ng = group_count(n, G);
+    bnd_cell[k] = c;
+    bnd_group[k] = min(i, ng);
+    bnd_slot[k] = i < ng ? first + i * G : first + n;
+  };
+  unsigned short* queue = reinterpret_cast<unsigned short*>(rows);
+  const int qcap = (int)(L.rows_bytes / 2) & ~31;  // wall hits the queue holds
+  if (tid == 0) n_hits = 0;
+  if (tid == 0) {  // ends of the instance (the last CTA's end is past every cell)
+    bnd_slot[1] = hi;
+    bnd_cell[1] = n_cells;
+    bnd_group[1] = 0;
+  }
+  __syncthreads();
+  for (int c = tid; c < n_cells; c += kThreads) {
+    const int first = off[c], n = off[c + 1] - first;
+    set_bound(0, B0, c, first, n);
+    if (rank + 1 < CL) set_bound(1, B1, c, first, n);
+  }
+  const float4* Pin = RL.parity_rec ? P1 : P0;
+  float4* Pout = RL.parity_rec ? P0 : P1;
+  bool bad_bounce = false, cand_fail = false, inflow_fail = false, mom_range = false;
+  bool bad_sort = false;
+  cluster_barrier();  // every CTA's accumulators are cleared
+
+  for (int st = 0; st < RL.n_steps; ++st, ++istep) {
+    const uint32_t step = (uint32_t)istep;
+    const bool sample = istep >= a.sample_start;
+    const bool collide = a.collide != 0;
+    const int s0 = bnd_slot[0];
+    int len = bnd_slot[1] - s0;
+    if (len < 0 || len > RL.range_cap) {  // only corrupted offsets can do this
+      bad_sort = true;
+      len = 0;
+    }
+
+    // A. This CTA's records and groups.
+    if (w == 0) {
+      const int cb = bnd_cell[0], ce = bnd_cell[1];
+      const int gb = bnd_group[0], ge = bnd_group[1];
+      int run = 0;
+      const int cend = len > 0 ? min(ce, n_cells - 1) : cb - 1;
+      for (int c0 = cb; c0 <= cend; c0 += 32) {
+        const int c = c0 + lane;
+        int g0 = 0, g1 = 0, ng = 0, nc = 0;
+        if (c <= cend) {
+          nc = off[c + 1] - off[c];
+          ng = group_count(nc, G);
+          g0 = c == cb ? gb : 0;
+          g1 = max(g0, c == ce ? ge : ng);
+        }
+        const int cnt = g1 - g0;
+        int incl = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int t = __shfl_up_sync(kFull, incl, o);
+          if (lane >= o) incl += t;
+        }
+        if (c <= cend) {
+          int p = run + incl - cnt;
+          for (int g = g0; g < g1; ++g, ++p)
+            if (p < RL.list_cap)
+              list[p] = make_int2(c, (g << 10) | (g == ng - 1 ? nc - g * G : G));
+        }
+        run += __shfl_sync(kFull, incl, 31);
+      }
+      if (lane == 0) {
+        if (run > RL.list_cap) {
+          bad_sort = true;
+          run = 0;
+        }
+        n_groups_sh = run;
+        next_group = kWarps;  // every warp starts with the group of its own number
+      }
+    } else {
+      for (int i = tid - 32; i < len; i += kThreads - 32) rec[i] = __ldcg(Pin + s0 + i);
+      for (int i = tid - 32; i < len; i += kThreads - 32) key[i] = 0u;
+    }
+    __syncthreads();
+    const int n_groups = n_groups_sh;
+
+    for (int q = w; q < n_groups;) {
+      const int2 e = list[q];
+      const int c = e.x, gi = e.y >> 10, gn = e.y & 1023;
+      const int cs = off[c], nc = off[c + 1] - cs;
+      const int gl = cs + gi * G - s0;  // first local slot of the group
+      if (gl < 0 || gl + gn > len) {  // only corrupted offsets can do this
+        bad_sort = true;
+        break;
+      }
+      float4* rg = rec + gl;
+      unsigned* touch = key + gl;
+      const float smax = csmax[c];
+
+      // Moments before the collisions, candidates, moments after them.
+      float gmax = 0.0f;
+      unsigned laccn = 0;
+      uint32_t M = 0;
+      LaneSums<Acc> m;
+      m.zero();
+      if (sample)
+        for (int i = lane; i < gn; i += 32) {
+          const float4 r = rg[i];
+          m.add(r.y, r.z, r.w);
+        }
+      if (collide && gn >= 2)
+        ntc_collide(a, rg, touch, gn, nc, c, gi, step, smax, mode, lane, lt, gmax, M, laccn,
+                    cand_fail);
+      __syncwarp();
+      if (sample)
+        for (int i = lane; i < gn; i += 32) {
+          const float4 r = rg[i];
+          m.add(r.y, r.z, r.w);
+        }
+
+      // The group's results into the slots of the cell's owner.
+      const int oc = c / own, os = c - oc * own;
+      if (sample) {
+        const Acc total = group_total(m, lane);
+        const int k = moment_of_lane(lane);
+        if ((lane & 1) == 0 && k >= 1 && k <= 12) {
+          const int gexp = grid_exponent(nc);
+          const long long fx = fixed_of(total, gexp);
+          const long long lim = (long long)(2 * gn) << (20 + gexp);
+          if (fx > lim || fx < -lim) mom_range = true;
+          peer_add(peer_addr(cfix + os * 12 + (k - 1), oc), (unsigned long long)fx);
+        }
+      }
+      const unsigned gbits = __reduce_max_sync(kFull, __float_as_uint(gmax));  // gmax >= 0
+      const unsigned nac = __reduce_add_sync(kFull, laccn);
+      if (lane == 0) {
+        if (gbits) peer_max(peer_addr(cgmax + (st & 1) * own + os, oc), gbits);
+        if (M) atomicAdd(ncand + c, (unsigned long long)M);
+        if (nac) atomicAdd(nacc + c, (unsigned long long)nac);
+        q = atomicAdd(&next_group, 1);
+      }
+      q = __shfl_sync(kFull, q, 0);
+    }
+    __syncthreads();
+
+    // Flight.  Particles that reach a wall are queued and flown afterwards, shared evenly by
+    // all warps of the CTA (they come from the few cells next to a wall).  The queue lives
+    // in the space of the ranks' counts, as many slots at a time as it could ever need.
+    for (int c0 = 0; c0 < len; c0 += qcap) {
+      const int c1 = min(len, c0 + qcap);
+      for (int b = c0 + w * 32; b < c1; b += kThreads) {
+        const int i = b + lane;
+        bool hits = false;
+        if (i < c1) {
+          const float4 r = rec[i];
+          const float ynew = fadd(r.x, fmul(r.z, a.dt));
+          hits = (ynew < 0.0f) || (ynew > 1.0f);
+          if (!hits)
+            *reinterpret_cast<float2*>(&rec[i]) = make_float2(ynew, fadd(r.y, fmul(a.F, a.dt)));
+        }
+        const unsigned hm = __ballot_sync(kFull, hits);
+        if (hm) {
+          int at = 0;
+          if (lane == 0) at = atomicAdd(&n_hits, __popc(hm));
+          at = __shfl_sync(kFull, at, 0) + __popc(hm & lt);
+          if (hits) queue[at] = (unsigned short)i;
+        }
+      }
+      __syncthreads();
+      const int nq = n_hits;
+      for (int b = w * 32; b < nq; b += kThreads)
+        if (b + lane < nq) {
+          const int i = queue[b + lane];
+          const float4 r = rec[i];
+          float yy = r.x, xx = r.y, uy = r.z, zz = r.w;
+          if (!fly(yy, xx, uy, zz, a.dt, a.F, a.keys, step, (uint32_t)(s0 + i - lo), a.open_top,
+                   a.u_top, a.p_top, inflow_fail))
+            bad_bounce = true;
+          rec[i] = make_float4(yy, xx, uy, zz);
+        }
+      __syncthreads();
+      if (tid == 0) n_hits = 0;
+      if (c1 < len) __syncthreads();
+    }
+    int* row = rows + w * n_cells;
+    for (int c = lane; c < n_cells; c += 32) row[c] = 0;
+    __syncwarp();
+
+    // Rank of every record among the earlier ones of its warp's part bound for its cell.
+    const int part = ((len + kWarps - 1) / kWarps + 31) & ~31;
+    const int pb = w * part, pe = min(len, pb + part);
+    for (int b = pb; b < pe; b += 32) {
+      const int i = b + lane;
+      const bool act = i < pe;
+      const int cell = act ? cell_of(rec[i].x, n_cells, a.ncf) : -1;
+      const unsigned peers = __match_any_sync(kFull, cell);
+      int first = 0;
+      if (act) first = row[cell];
+      __syncwarp();
+      if (act) {
+        const int before = __popc(peers & lt);
+        if (before == 0) row[cell] = first + __popc(peers);
+        key[i] = ((unsigned)cell << 16) | (unsigned)(first + before);
+      }
+      __syncwarp();
+    }
+    __syncthreads();
+    for (int c = tid; c < n_cells; c += kThreads) {
+      int t[kWarps], run = 0;
+#pragma unroll
+      for (int v = 0; v < kWarps; ++v) t[v] = rows[v * n_cells + c];
+#pragma unroll
+      for (int v = 0; v < kWarps; ++v) {
+        rows[v * n_cells + c] = run;
+        run += t[v];
+      }
+      for (int v = 0; v < CL; ++v) peer_store(peer_addr(tot + rank * n_cells + c, v), run);
+    }
+    cluster_barrier();
+
+    // B. New offsets, the cells' results, and the sort.
+    int carry = lo;
+    for (int cb = 0, ph = 0; cb < n_cells; cb += kThreads, ph ^= 1) {
+      const int c = cb + tid;
+      int total = 0, pre = 0;
+      uint32_t gm = 0u;
+      if (c < n_cells) {
+        const int oc = c / own;  // the owner's largest relative speed, used below
+        gm = peer_load(peer_addr(cgmax + (st & 1) * own + (c - oc * own), oc));
+#pragma unroll 4
+        for (int v = 0; v < CL; ++v) {
+          const int t = tot[v * n_cells + c];
+          total += t;
+          pre += v < rank ? t : 0;
+        }
+      }
+      int incl = total;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += t;
+      }
+      if (lane == 31) wsum[ph][w] = incl;
+      __syncthreads();
+      const int ws = lane < kWarps ? wsum[ph][lane] : 0;
+      const int before = carry + __reduce_add_sync(kFull, lane < w ? ws : 0);
+      const int all = __reduce_add_sync(kFull, ws);
+      carry += all;
+      if (c < n_cells) {
+        const int first = before + incl - total;
+        off_next[c] = first;
+        base[c] = first + pre;
+        set_bound(0, B0, c, first, total);
+        if (rank + 1 < CL) set_bound(1, B1, c, first, total);
+        if (c == n_cells - 1) off_next[n_cells] = first + total;
+        // (sigma g)_max of the next step
+        const float g = __uint_as_float(gm);
+        const float sg = (mode == 0) ? g : fmul(a.cvhs, pow32(g, a.vexp));
+        csmax[c] = fmaxf(csmax[c], sg);
+      }
+    }
+    // (taken from the last threads down: the first ones are busy with the cells above)
+    for (int i = kThreads - 1 - tid; i < own_n * kNMom; i += kThreads) {
+      const int oc = i / kNMom, k = i - oc * kNMom, c = own0 + oc;
+      if (k == 0) cgmax[((st & 1) ^ 1) * own + oc] = 0u;
+      if (sample) {
+        const int nc = off[c + 1] - off[c];
+        if (k == 0) {
+          csum[i] += (double)nc;
+        } else {
+          const double grid =
+              __longlong_as_double((long long)(1023 - grid_exponent(nc > 0 ? nc : 1)) << 52);
+          csum[i] += 0.5 * grid * (double)(long long)cfix[oc * 12 + k - 1];
+          cfix[oc * 12 + k - 1] = 0ull;
+        }
+      }
+    }
+    __syncthreads();
+    for (int b = pb; b < pe; b += 32) {
+      const int i = b + lane;
+      if (i < pe) {
+        const unsigned kk = key[i];
+        const int cell = (int)(kk >> 16);
+        const int d = base[cell] + rows[w * n_cells + cell] + (int)(kk & 0xffffu);
+        if (d >= lo && d < hi)
+          Pout[d] = rec[i];
+        else
+          bad_sort = true;
+      }
+    }
+    cluster_barrier();
+    int* t0 = off;
+    off = off_next;
+    off_next = t0;
+    float4* t1 = const_cast<float4*>(Pin);
+    Pin = Pout;
+    Pout = t1;
+  }
+
+  for (int i = tid; i < own_n * kNMom; i += kThreads) acc[(size_t)own0 * kNMom + i] = csum[i];
+  // The run's state after the last step, where the next launch of either kind looks for it.
+  if (rank == 0) {
+    int* g = ((RL.parity_off ^ RL.n_steps) & 1 ? off1 : off0) + a.off_base;
+    float* s = ((RL.parity_smax ^ RL.n_steps) & 1 ? smax1 : smax0) + a.cell_base;
+    for (int c = tid; c <= n_cells; c += kThreads) g[c] = off[c];
+    for (int c = tid; c < n_cells; c += kThreads) s[c] = csmax[c];
+  }
+  if (bad_bounce) atomicOr(err, kErrBounces);
+  if (cand_fail && lane == 0) atomicOr(err, kErrCandidates);
+  if (inflow_fail) atomicOr(err, kErrInflow);
+  if (mom_range) atomicOr(err, kErrMoments);
+  if (bad_sort) atomicOr(err, kErrSort);
+}
+
+namespace {
+
+const void* resident_kernel(bool batch, bool f64) {
+  if (batch)
+    return f64 ? (const void*)k_resident<true, kResidentWarpsBatch, true>
+               : (const void*)k_resident<true, kResidentWarpsBatch, false>;
+  return f64 ? (const void*)k_resident<false, kResidentWarps, true>
+             : (const void*)k_resident<false, kResidentWarps, false>;
+}
+
+}  // namespace
+
+cudaError_t resident_clusters(int cl, size_t smem, bool batch, bool f64, int* clusters) {
+  const void* f = resident_kernel(batch, f64);
+  *clusters = 0;
+  cudaError_t e =
+      cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResidentSmemMax);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(cl);
+  cfg.blockDim = dim3(resident_warps(batch) * 32);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = cl;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaOccupancyMaxActiveClusters(clusters, f, &cfg);
+}
+
+cudaError_t launch_resident(float4* P0, float4* P1, int* off0, int* off1, float* smax0,
+                            float* smax1, unsigned long long* ncand, unsigned long long* nacc,
+                            double* acc, const InstParams& one, const ResidentLaunch& L,
+                            bool f64, int* err, cudaStream_t st) {
+  const ResidentSmem S =
+      resident_smem_layout(L.max_cells, L.range_cap, L.list_cap, L.own_cap, L.cl,
+                           resident_warps(L.n_inst > 1));
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(L.cl * L.n_inst));
+  cfg.blockDim = dim3(resident_warps(L.n_inst > 1) * 32);
+  cfg.dynamicSmemBytes = S.total;
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = L.cl;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  void* args[] = {&P0,   &P1,  &off0, &off1, &smax0, &smax1, &ncand, &nacc, &acc,
+                  const_cast<InstParams*>(&one), const_cast<ResidentLaunch*>(&L), &err};
+  const cudaError_t e = cudaLaunchKernelExC(&cfg, resident_kernel(L.n_inst > 1, f64), args);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+}  // namespace dsmc

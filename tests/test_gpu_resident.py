@@ -1,0 +1,96 @@
+"""Cluster-resident steps (csrc/dsmc_resident.cu) against the span passes, bit for bit.
+
+A handle with default options runs small problems cluster-resident; with profile=1 the
+same handle takes the span passes (whose parity with the oracle the other tests pin).  Both
+must give the same records, offsets, maxima, counters and moment sums at the sizes where the
+resident kernel's tables and partitions can go wrong.
+"""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _bits(a):
+    a = np.ascontiguousarray(a)
+    return a.view(np.uint8)
+
+
+def _snapshot(h, i=None):
+    args = () if i is None else (i,)
+    m, n = h.moments(*args)
+    return (*h.state(*args), *h.cells(*args), m, np.int64(n))
+
+
+def _assert_same(a, b):
+    for k, (x, y) in enumerate(zip(a, b)):
+        np.testing.assert_array_equal(_bits(x), _bits(y), err_msg=f"output {k}")
+
+
+CASES = [
+    dict(Kn=1.0, n_cells=100, ppc=200, omega=0.5),              # the small hard-sphere run
+    dict(Kn=0.1, n_cells=200, ppc=50, omega=0.5),               # the training run
+    dict(Kn=0.44, n_cells=45, ppc=50, omega=0.81),              # the hybrid's sub-domain
+    dict(Kn=0.5, n_cells=200, ppc=500, omega=0.5),              # largest shares
+    dict(Kn=1.0, n_cells=7, ppc=3, omega=1.0),                  # fewer particles than lanes
+    dict(Kn=1.0, n_cells=1, ppc=700, omega=0.5),                # one cell over all CTAs
+    dict(Kn=10.0, n_cells=37, ppc=533, omega=0.74),             # about one wall hit each
+    dict(Kn=0.5, n_cells=3, ppc=5, omega=0.5, group_size=2),    # groups of two
+    dict(Kn=0.1, n_cells=20, ppc=3000, omega=0.81, accum=1),    # many groups per cell
+    dict(Kn=0.1, n_cells=700, ppc=20, omega=0.5, group_size=8),  # more cells than threads
+    dict(Kn=0.3, n_cells=300, ppc=100, omega=0.5, collisions=False),
+    dict(Kn=0.3, n_cells=60, ppc=300, omega=0.81, group_size=512),
+]
+
+
+@pytest.mark.parametrize("case", CASES, ids=lambda c: f"{c['n_cells']}x{c['ppc']}")
+def test_resident_steps_match_the_span_passes(case):
+    from paper_2311_14140_gb300 import Dsmc
+    got = []
+    for profile in (False, True):
+        d = Dsmc(body_force=1e-2, seed=5, sample_start=4, profile=profile, **case)
+        for n in (1, 2, 7, 3):  # odd and even counts: every buffer parity
+            d.step(n)
+        got.append(_snapshot(d))
+        d.close()
+    _assert_same(*got)
+
+
+def test_resident_steps_of_an_uneven_state_and_open_boundary():
+    """A loaded state that fills only part of the channel (empty cells, dense cells), then
+    an open upper boundary; switching between the two step kinds on the way."""
+    from paper_2311_14140_gb300 import Dsmc
+    rng = np.random.default_rng(3)
+    n = 60 * 150
+    y = (0.35 * rng.random(n) ** 2 + 0.5).astype(np.float32)
+    v = [rng.normal(0, np.sqrt(0.5), n).astype(np.float32) for _ in range(3)]
+    got = []
+    for profile in (False, True):
+        d = Dsmc(0.3, 60, 150, omega=0.81, body_force=1e-2, seed=9, profile=profile)
+        d.load_state(y, *v, step=3)
+        d.step(4)
+        d.set_open_top(0.01, -0.02)
+        d.step(5)
+        d.set_options(profile=not profile)
+        d.step(2)
+        d.set_options(profile=profile)
+        d.step(3)
+        got.append(_snapshot(d))
+        d.close()
+    _assert_same(*got)
+
+
+@pytest.mark.parametrize("n,cells,ppc", [(2, 30, 41), (9, 0, 0), (40, 100, 100), (24, 200, 200)])
+def test_resident_batches_match_the_span_passes(n, cells, ppc):
+    from paper_2311_14140_gb300 import DsmcBatch
+    defs = [dict(Kn=0.2 + 0.3 * i, n_cells=cells or 30 + 7 * i, ppc=ppc or 40 + 11 * i,
+                 omega=(0.5, 0.81, 1.0)[i % 3], body_force=1e-3, seed=i) for i in range(n)]
+    got = []
+    for profile in (False, True):
+        b = DsmcBatch(defs, sample_start=3, profile=profile)
+        b.step(5)
+        b.step(6)
+        got.append([_snapshot(b, i) for i in range(n)])
+        b.close()
+    for a, b in zip(*got):
+        _assert_same(a, b)
