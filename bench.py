@@ -88,7 +88,7 @@ def ncu_traffic(kernel: str):
 
 
 # Sources of the step kernels the committed traffic figures were taken from.
-STEP_SOURCES = ("dsmc_step.cu", "dsmc_device.cuh", "dsmc_internal.h")
+STEP_SOURCES = ("dsmc_step.cu", "dsmc_collide.cuh", "dsmc_device.cuh", "dsmc_internal.h")
 
 
 def _code_only(text: str) -> str:

@@ -82,8 +82,15 @@ __device__ __forceinline__ void direction_of(uint32_t w0, uint32_t w1, float& nx
 // cell's particle number and needs no sum): v, v_i v_j (six), v_i |v|^2 (three).
 // LaneSums<float>: the products of the binary32 velocities summed in binary32, the
 // second and third moments by fused multiply-add (one rounding per term).
-// LaneSums<double>: every product rounded to binary32 exactly as the oracle forms it,
-// then added in binary64.
+// LaneSums<double> (DSMC_ACCUM_FP64): every product rounded to binary32 exactly as the
+// oracle forms it, then summed with its rounding errors kept, as pairs of binary32.  A
+// group's total, before it is rounded to its cell's grid (fixed_of), is then within 2^-40 of
+// the sum of |products| (48 terms per lane), against grid steps of 2^-27 at 25,000 particles
+// per cell and 2^-35 at 50: against exact sums of known velocities (50 to 25,000 particles
+// per cell) the results' error is that of binary64 additions to every digit compared
+// (rms 6.8e-14 to 1.7e-12 of the sum of |products|), because the grid makes it.  The GB300
+// makes 2 binary64 additions per clock and SM against 128 in binary32: a step of 5,000,000
+// particles took 0.678 ms with them and takes 0.161 ms (0.128 with LaneSums<float>).
 template <typename T>
 struct LaneSums;
 
@@ -126,29 +133,75 @@ struct LaneSums<float> {
   }
 };
 
-template <>
-struct LaneSums<double> {
-  double m[12];
-  __device__ __forceinline__ void zero() {
-#pragma unroll
-    for (int k = 0; k < 12; ++k) m[k] = 0.0;
-  }
-  __device__ __forceinline__ void add(float x, float y, float z) {
-    const float v2 = fadd(fadd(fmul(x, x), fmul(y, y)), fmul(z, z));
-    const float p[12] = {x,          y,          z,          fmul(x, x), fmul(y, y), fmul(z, z),
-                         fmul(x, y), fmul(x, z), fmul(y, z), fmul(x, v2), fmul(y, v2),
-                         fmul(z, v2)};
-#pragma unroll
-    for (int k = 0; k < 12; ++k) m[k] = __dadd_rn(m[k], (double)p[k]);
-  }
-  __device__ __forceinline__ double get(int k) const {
-    double r = 0.0;
-#pragma unroll
-    for (int j = 0; j < 12; ++j)
-      if (k == j + 1) r = m[j];
-    return r;
+// Exact sums of binary32 values as unevaluated pairs hi + lo, two sums at a time: Knuth's
+// two-sum gives the rounding error of every addition to hi exactly, and lo collects the
+// errors (in binary32: they are 2^-24 of hi, so the pair carries 48 bits).
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
+  float2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;"
+      : "=l"(reinterpret_cast<unsigned long long&>(r))
+      : "l"(reinterpret_cast<const unsigned long long&>(a)),
+        "l"(reinterpret_cast<const unsigned long long&>(b)));
+  return r;
+}
+
+struct Pair2 {
+  float2 hi, lo;
+  __device__ __forceinline__ void add(float2 p) {
+    const float2 s = __fadd2_rn(hi, p);
+    const float2 t = sub2(s, hi);
+    const float2 e = __fadd2_rn(sub2(hi, sub2(s, t)), sub2(p, t));
+    lo = __fadd2_rn(lo, e);
+    hi = s;
   }
 };
+
+template <>
+struct LaneSums<double> {
+  Pair2 a, b, c, d, e, f;  // the same places as in LaneSums<float>
+  __device__ __forceinline__ void zero() {
+    const float2 z = make_float2(0.0f, 0.0f);
+    a = b = c = d = e = f = Pair2{z, z};
+  }
+  // (the products by scalar multiplications: a packed product followed by a packed addition
+  // was contracted, which adds the exact product instead of the rounded one)
+  __device__ __forceinline__ void add(float x, float y, float z) {
+    const float xx = fmul(x, x), yy = fmul(y, y), zz = fmul(z, z);
+    const float v2 = fadd(fadd(xx, yy), zz);
+    a.add(make_float2(x, y));
+    b.add(make_float2(z, zz));
+    c.add(make_float2(xx, yy));
+    d.add(make_float2(fmul(x, y), fmul(x, z)));
+    e.add(make_float2(fmul(y, z), fmul(z, v2)));
+    f.add(make_float2(fmul(x, v2), fmul(y, v2)));
+  }
+  // moment k as its pair (hi, lo), in the order of LaneSums<float>::get
+  __device__ __forceinline__ float2 get(int k) const {
+    switch (k) {
+      case 1: return make_float2(a.hi.x, a.lo.x);
+      case 2: return make_float2(a.hi.y, a.lo.y);
+      case 3: return make_float2(b.hi.x, b.lo.x);
+      case 4: return make_float2(c.hi.x, c.lo.x);
+      case 5: return make_float2(c.hi.y, c.lo.y);
+      case 6: return make_float2(b.hi.y, b.lo.y);
+      case 7: return make_float2(d.hi.x, d.lo.x);
+      case 8: return make_float2(d.hi.y, d.lo.y);
+      case 9: return make_float2(e.hi.x, e.lo.x);
+      case 10: return make_float2(f.hi.x, f.lo.x);
+      case 11: return make_float2(f.hi.y, f.lo.y);
+      case 12: return make_float2(e.hi.y, e.lo.y);
+      default: return make_float2(0.0f, 0.0f);
+    }
+  }
+};
+
+// Sum of two pairs: two-sum of the high parts, the errors collected in the low part.
+__device__ __forceinline__ float2 pair_sum(float2 a, float2 b) {
+  const float s = fadd(a.x, b.x);
+  const float t = fsub(s, a.x);
+  const float e = fadd(fsub(a.x, fsub(s, t)), fsub(b.x, t));
+  return make_float2(s, fadd(fadd(a.y, b.y), e));
+}
 
 // Warp sum of a group's lane sums by a transposing butterfly over 16 slots (moments
 // 1..12 and zero padding): each exchange halves the values a lane carries, so 16
@@ -157,9 +210,8 @@ __device__ __forceinline__ int moment_of_lane(int lane) {
   return ((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
 }
 
-template <typename T>
-__device__ __forceinline__ T group_total(const LaneSums<T>& m, int lane) {
-  T v[16];
+__device__ __forceinline__ float group_total(const LaneSums<float>& m, int lane) {
+  float v[16];
 #pragma unroll
   for (int k = 0; k < 16; ++k) v[k] = m.get(k);
 #pragma unroll
@@ -167,12 +219,34 @@ __device__ __forceinline__ T group_total(const LaneSums<T>& m, int lane) {
     const bool upper = (lane & mask) != 0;
 #pragma unroll
     for (int k = 0; k < half; ++k) {
-      const T send = upper ? v[k] : v[k + half];
-      const T keep = upper ? v[k + half] : v[k];
+      const float send = upper ? v[k] : v[k + half];
+      const float keep = upper ? v[k + half] : v[k];
       v[k] = keep + __shfl_xor_sync(kFull, send, mask);
     }
   }
   return v[0] + __shfl_xor_sync(kFull, v[0], 1);
+}
+
+// The same for pairs; the pair's value in binary64.
+__device__ __forceinline__ double group_total(const LaneSums<double>& m, int lane) {
+  float2 v[16];
+#pragma unroll
+  for (int k = 0; k < 16; ++k) v[k] = m.get(k);
+  auto other = [](float2 x, int mask) {
+    return make_float2(__shfl_xor_sync(kFull, x.x, mask), __shfl_xor_sync(kFull, x.y, mask));
+  };
+#pragma unroll
+  for (int half = 8, mask = 16; half >= 1; half >>= 1, mask >>= 1) {
+    const bool upper = (lane & mask) != 0;
+#pragma unroll
+    for (int k = 0; k < half; ++k) {
+      const float2 send = upper ? v[k] : v[k + half];
+      const float2 keep = upper ? v[k + half] : v[k];
+      v[k] = pair_sum(keep, other(send, mask));
+    }
+  }
+  const float2 s = pair_sum(v[0], other(v[0], 1));
+  return (double)s.x + (double)s.y;
 }
 
 // Exact, order-independent combination of group totals.  A cell's group totals are

@@ -57,7 +57,7 @@ __device__ __forceinline__ bool add_group(const LaneSums<T>& m, bool sample, int
                                           unsigned long long* caccn, int lane) {
   bool ok = true;
   if (sample) {
-    const T tot = group_total(m, lane);
+    const auto tot = group_total(m, lane);
     const int k = moment_of_lane(lane);
     if ((lane & 1) == 0 && k >= 1 && k <= 12) {
       const int ge = grid_exponent(nc);
@@ -114,11 +114,11 @@ __device__ __forceinline__ const InstParams& stage_instance(const InstParams& on
 // (sigma g independent of g).  CTAs per SM the register budget is set for: 3 of 8 warps,
 // 6 of 4 warps; the batched 4-warp kernel reads its parameters from shared memory and
 // spills at 6 (85 registers), so it is given 5 (no spills, 10 % faster on the
-// 256-instance batch).  The binary64 moment sums (kF64) hold twelve binary64 values per
-// lane and get half the CTAs per SM.
+// 256-instance batch).  With the error-keeping moment sums (kF64: 24 binary32 values per
+// lane, 114 to 118 registers) two and four.
 template <bool kBatch, int kWarps, bool kF64>
 constexpr int collide_ctas_per_sm() {
-  return (kWarps == kAWarps ? 3 : (kBatch ? 5 : 6)) / (kF64 ? 2 : 1);
+  return kF64 ? (kWarps == kAWarps ? 2 : 4) : (kWarps == kAWarps ? 3 : (kBatch ? 5 : 6));
 }
 
 template <bool kBatch, int kWarps, bool kF64>

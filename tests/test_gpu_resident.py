@@ -94,3 +94,36 @@ def test_resident_batches_match_the_span_passes(n, cells, ppc):
         b.close()
     for a, b in zip(*got):
         _assert_same(a, b)
+
+
+@pytest.mark.parametrize("n_cells,ppc,group_size", [(60, 3, 256), (40, 50, 256), (30, 500, 512),
+                                                    (6, 25000, 256)])
+def test_error_keeping_sums_of_known_velocities(n_cells, ppc, group_size):
+    """accum=1 without collisions: the sums before and after the collisions are those of the
+    state before the step, so a step's moments are known exactly (math.fsum of the binary32
+    products).  Bound: every group total is rounded to its cell's grid (half a step of
+    2^-(41 - e) per group, e the bit length of the cell's count) after an addition error of at
+    most 2^-40 of the sum of |products|, halved and doubled again by the two samples."""
+    import math
+
+    from paper_2311_14140_gb300 import Dsmc
+    d = Dsmc(0.1, n_cells, ppc, omega=0.81, body_force=1e-3, seed=3, accum=1, collisions=False,
+             group_size=group_size, sample_start=2)
+    d.step(1)
+    _, x, y, z = d.state()
+    off = d.cells()[0]
+    d.step(1)
+    sums, n = d.moments()
+    d.close()
+    assert n == 1
+    xx, yy, zz = x * x, y * y, z * z
+    v2 = (xx + yy) + zz
+    prods = [x, y, z, xx, yy, zz, x * y, x * z, y * z, x * v2, y * v2, z * v2]
+    for c in range(n_cells):
+        nc = int(off[c + 1] - off[c])
+        groups = nc // group_size + 1
+        grid = 2.0 ** -(41 - nc.bit_length())
+        for k, p in enumerate(prods):
+            q = p[off[c]:off[c + 1]].astype(np.float64)
+            bound = 0.5 * grid * groups + 2.0 ** -40 * np.abs(q).sum()
+            assert abs(sums[c, k + 1] - math.fsum(q)) <= bound, (c, k)
