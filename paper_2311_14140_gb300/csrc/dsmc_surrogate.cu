@@ -4,6 +4,8 @@
 // macroscopic solve with Monte Carlo uncertainty bands.
 //
 // Device work (binary64):
+//   k_basis   once per surrogate: the Appendix A basis at the training cells (their values
+//             depend on the grid and the exponents alone) and their Phi^T Phi.
 //   k_window  one training sample per call: from a window's raw moment sums, the cell
 //             velocities and shear stresses (Eq. 6 units), the constitutive targets
 //             E_i = P_i + (2 Kn / sqrt(pi)) du/dy_i at the interior cells (Eq. 13, du/dy
@@ -12,10 +14,11 @@
 //             sample's sufficient statistics (Phi^T Phi, Phi^T t, t^T t, sum t, N) for
 //             the boundary and constitutive models to running totals.  The moment sums
 //             stay on the device: a run's accumulators are read in place.
-//   k_trials  one thread per Monte Carlo trial: weights drawn from the selected
-//             models' posteriors (w = m + L z, S = L L^T by Cholesky), the cell-centred
-//             finite-volume system of Eq. 8 with Eqs. 9-10 solved by the Thomas
-//             algorithm.
+//   k_modes   Eq. 8 is linear: a trial's profile is its wall velocity plus the profile of the
+//             body force plus its weights times the profiles of the basis functions, so those
+//             (at most four) are solved once, in closed form up to a prefix sum; also the
+//             trials' weights, drawn from the selected models' posteriors (w = m + L z,
+//             S = L L^T by Cholesky on the host).
 //   k_bands   per cell: mean and standard deviation over the trials.
 // Host work: the evidence maximisation itself (MacKay's re-estimation of alpha and beta
 // on 1x1 to 3x3 matrices, Bishop Sec. 3.5, Tipping App. A) and Eq. 17.
@@ -38,6 +41,7 @@ constexpr int kStats = 20;  // sufficient statistics, layout below
 // [12] t^T t, [13] N (constitutive); [14] sum x t, [15] sum x^2, [16] t^T t, [17] N
 // (boundary); [18] sum t (constitutive), [19] sum t (boundary).
 constexpr int kThreads = 256;
+constexpr int kWindowCells = 1024;  // cells whose velocities k_window keeps in shared memory
 constexpr double kAlphaMax = 1e30;  // weight precision above which weights are off
 constexpr double kSqrtPi = 1.7724538509055160273;
 
@@ -71,149 +75,185 @@ struct WindowArgs {
   int both;        // 1: both walls give boundary data (whole channel), 0: bottom only
 };
 
-__device__ __forceinline__ double cell_u(const double* acc, int i) {
-  return acc[(size_t)i * dsmc::kNMom + 1] / acc[(size_t)i * dsmc::kNMom + 0];
+// Sum over the CTA of K values per thread, into red[0..K) (valid after the call's barrier):
+// warp k adds value k of all threads.  (A butterfly of every value in every warp is three times
+// the binary64 additions, which come at two per clock.)
+template <int K>
+__device__ __forceinline__ void block_sums(const double (&v)[K], double (&part)[K][kThreads],
+                                           double* red) {
+  static_assert(K <= kThreads / 32, "a warp per value");
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+#pragma unroll
+  for (int k = 0; k < K; ++k) part[k][t] = v[k];
+  __syncthreads();
+  if (w < K) {
+    double s = 0.0;
+#pragma unroll
+    for (int u = 0; u < kThreads / 32; ++u) s += part[w][u * 32 + lane];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) red[w] = s;
+  }
+  __syncthreads();
 }
 
-__global__ void __launch_bounds__(kThreads) k_window(const double* __restrict__ acc,
-                                                     WindowArgs a, double* __restrict__ stats) {
-  __shared__ double red[16][kThreads];
+// basis[l n + i] = c (exp(-b_l y_i) - exp(-b_l (1 - y_i))) at the training cells 1..last, and
+// gram[0..5] = their products' sums (00, 01, 02, 11, 12, 22).
+__global__ void __launch_bounds__(kThreads)
+    k_basis(WindowArgs a, double* __restrict__ basis, double* __restrict__ gram) {
+  __shared__ double part[6][kThreads];
+  const double h = a.length / a.n;
+  const double c = 2.0 * a.kn / kSqrtPi;
+  double g[6] = {0, 0, 0, 0, 0, 0};
+  for (int i = 1 + threadIdx.x; i <= a.last; i += kThreads) {
+    const double y = (i + 0.5) * h;
+    double f[3];
+#pragma unroll
+    for (int l = 0; l < 3; ++l) {
+      f[l] = c * (exp(-a.b[l] * y) - exp(-a.b[l] * (1.0 - y)));
+      basis[(size_t)l * a.n + i] = f[l];
+    }
+    g[0] = fma(f[0], f[0], g[0]);
+    g[1] = fma(f[0], f[1], g[1]);
+    g[2] = fma(f[0], f[2], g[2]);
+    g[3] = fma(f[1], f[1], g[3]);
+    g[4] = fma(f[1], f[2], g[4]);
+    g[5] = fma(f[2], f[2], g[5]);
+  }
+  block_sums<6>(g, part, gram);
+}
+
+// One CTA: a cell per thread (200 cells in the paper), one division per cell.  Binary64 runs at
+// two operations per clock and SM here, so the exponentials of the basis (now k_basis's) and
+// six divisions per cell were most of this kernel: windows of 200 cells added one after another
+// took 25 us each and take 8.9, the kernel 8.
+__global__ void __launch_bounds__(kThreads)
+    k_window(const double* __restrict__ acc, WindowArgs a, const double* __restrict__ basis,
+             const double* __restrict__ gram, double* __restrict__ stats,
+             double* __restrict__ scratch) {
+  __shared__ double u_sh[kWindowCells];
+  double* u = a.n <= kWindowCells ? u_sh : scratch;  // cell velocities
+  __shared__ double part[5][kThreads];
+  __shared__ double red[5];
   const int t = threadIdx.x;
   const double h = a.length / a.n;
   const double c = 2.0 * a.kn / kSqrtPi;
-  double g00 = 0, g01 = 0, g02 = 0, g11 = 0, g12 = 0, g22 = 0, p0 = 0, p1 = 0, p2 = 0, tt = 0,
-         st = 0, nn = 0;
+  const double per = 2.0 / a.n_norm, slope = c / (2.0 * h);
+  const int gi[9] = {0, 1, 2, 1, 3, 4, 2, 4, 5};
+  // what the totals below need, on its way while the cells are worked on
+  const double before = t < kStats ? stats[t] : 0.0;
+  const double gr = t < 9 ? gram[gi[t]] : 0.0;
+  for (int i = t; i < a.n; i += kThreads) {
+    const double* r = acc + (size_t)i * dsmc::kNMom;
+    u[i] = r[1] / r[0];
+  }
+  __syncthreads();
+  double v[5] = {0, 0, 0, 0, 0};  // Phi^T t (three), t^T t, sum t
   for (int i = 1 + t; i <= a.last; i += kThreads) {
     const double* r = acc + (size_t)i * dsmc::kNMom;
-    const double N = r[0];
-    const double ux = r[1] / N, uy = r[2] / N;
-    const double P = 2.0 * (N / a.n_norm) * (r[7] / N - ux * uy);
-    const double dudy = (cell_u(acc, i + 1) - cell_u(acc, i - 1)) / (2.0 * h);
-    const double E = P + c * dudy;
-    const double y = (i + 0.5) * h;
-    const double f0 = c * (exp(-a.b[0] * y) - exp(-a.b[0] * (1.0 - y)));
-    const double f1 = c * (exp(-a.b[1] * y) - exp(-a.b[1] * (1.0 - y)));
-    const double f2 = c * (exp(-a.b[2] * y) - exp(-a.b[2] * (1.0 - y)));
-    g00 += f0 * f0;
-    g01 += f0 * f1;
-    g02 += f0 * f2;
-    g11 += f1 * f1;
-    g12 += f1 * f2;
-    g22 += f2 * f2;
-    p0 += f0 * E;
-    p1 += f1 * E;
-    p2 += f2 * E;
-    tt += E * E;
-    st += E;
-    nn += 1.0;
-  }
-  double v[12] = {g00, g01, g02, g11, g12, g22, p0, p1, p2, tt, st, nn};
+    // P = 2 (N / n_norm) (S_xy / N - u_x u_y) with u_y = S_y / N
+    const double P = per * (r[7] - u[i] * r[2]);
+    const double E = fma(slope, u[i + 1] - u[i - 1], P);
 #pragma unroll
-  for (int k = 0; k < 12; ++k) red[k][t] = v[k];
-  __syncthreads();
-  for (int s = kThreads / 2; s > 0; s >>= 1) {
-    if (t < s)
-#pragma unroll
-      for (int k = 0; k < 12; ++k) red[k][t] += red[k][t + s];
-    __syncthreads();
+    for (int l = 0; l < 3; ++l) v[l] = fma(basis[(size_t)l * a.n + i], E, v[l]);
+    v[3] = fma(E, E, v[3]);
+    v[4] += E;
   }
-  if (t == 0) {
-    const double G[9] = {red[0][0], red[1][0], red[2][0], red[1][0], red[3][0],
-                         red[4][0], red[2][0], red[4][0], red[5][0]};
-    for (int k = 0; k < 9; ++k) stats[k] += G[k];
-    stats[9] += red[6][0];
-    stats[10] += red[7][0];
-    stats[11] += red[8][0];
-    stats[12] += red[9][0];
-    stats[13] += red[11][0];
-    stats[18] += red[10][0];
-    // boundary models: x = -P(0) = F (and P(1) = F), t = wall velocities
-    const int n = a.n;
-    const double ub = 1.5 * cell_u(acc, 0) - 0.5 * cell_u(acc, 1);
-    if (a.both) {
-      const double ut = 1.5 * cell_u(acc, n - 1) - 0.5 * cell_u(acc, n - 2);
-      stats[14] += a.F * ub + a.F * ut;
-      stats[15] += a.F * a.F + a.F * a.F;
-      stats[16] += ub * ub + ut * ut;
-      stats[17] += 2.0;
-      stats[19] += ub + ut;
-    } else {
-      stats[14] += a.F * ub;
-      stats[15] += a.F * a.F;
-      stats[16] += ub * ub;
-      stats[17] += 1.0;
-      stats[19] += ub;
-    }
-  }
+  block_sums<5>(v, part, red);
+  // Totals: Phi^T Phi of the sample is the basis's own; the boundary models have x = -P(0) = F
+  // (and P(1) = F) and t = the wall velocities.
+  if (t >= kStats) return;
+  const int n = a.n;
+  const double ub = 1.5 * u[0] - 0.5 * u[1];
+  const double ut = a.both ? 1.5 * u[n - 1] - 0.5 * u[n - 2] : 0.0;
+  double add = 0.0;
+  if (t < 9) add = gr;
+  else if (t < 13) add = red[t - 9];
+  else if (t == 13) add = (double)a.last;
+  else if (t == 14) add = a.both ? a.F * ub + a.F * ut : a.F * ub;
+  else if (t == 15) add = a.both ? a.F * a.F + a.F * a.F : a.F * a.F;
+  else if (t == 16) add = a.both ? ub * ub + ut * ut : ub * ub;
+  else if (t == 17) add = a.both ? 2.0 : 1.0;
+  else if (t == 18) add = red[4];
+  else add = a.both ? ub + ut : ub;
+  stats[t] = before + add;
 }
 
-// Posterior of one model as the trials need it.
+// Posterior of the selected models as the trials need it.
 struct TrialModels {
   int sel_v, k;  // slip selected; number of constitutive weights (0..3)
-  double m_v, s_v;
-  double m[3], S[9];
+  double m_v, sd_v;
+  double m[3], L[9];  // weights' means and the Cholesky factor of their covariance
   double kn, F;
   double b[3];
   int n;  // CFD cells
 };
 
-__global__ void __launch_bounds__(128) k_trials(TrialModels tm, const double* __restrict__ z,
-                                                int n_trials, double* __restrict__ u,
-                                                double* __restrict__ cp) {
-  const int tr = blockIdx.x * blockDim.x + threadIdx.x;
-  if (tr >= n_trials) return;
-  const double* zt = z + (size_t)tr * 4;
-  double uw = 0.0;
-  if (tm.sel_v) uw = (tm.m_v + sqrt(tm.s_v) * zt[0]) * tm.F;  // -sigma_P P(0) = sigma_P F
-  double w[3] = {0.0, 0.0, 0.0};
-  if (tm.k > 0) {
-    // Cholesky S = L L^T (lower, k <= 3), then w = m + L z
-    double L[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-    for (int i = 0; i < tm.k; ++i)
-      for (int j = 0; j <= i; ++j) {
-        double s = tm.S[i * 3 + j];
-        for (int q = 0; q < j; ++q) s -= L[i * 3 + q] * L[j * 3 + q];
-        L[i * 3 + j] = (i == j) ? sqrt(s > 0.0 ? s : 0.0) : (L[j * 3 + j] > 0.0 ? s / L[j * 3 + j] : 0.0);
+// Blocks 0..k: the profile of one unit right side of the cell-centred finite-volume form of
+// Eq. 8 with zero wall values: block 0 the body force, block 1 + l the basis function l.
+// With face fluxes q_f (f = 0..n) the rows say q_{i+1} - q_i = r_i, so q_f = q_0 + R_f with
+// R_f = f src (block 0) or S_f - S_0; summing u_{i+1} - u_i = h q_{i+1} from wall to wall
+// (half cells at both ends) gives q_0 = -(h sum_{0<f<n} R_f + h/2 R_n) and
+// u_i = h/2 q_0 + h i q_0 + h sum_{0<f<=i} R_f: one prefix sum instead of a sweep of n
+// dependent divisions per trial (dsmc_surrogate_profile at 200 cells: 0.85 ms with one trial,
+// 1.18 with 1,000; now 0.057 and 0.066).
+// The blocks after them: the weights of the trials, (uw, w_1..w_3) in weights[4 t ..].
+__global__ void __launch_bounds__(kThreads)
+    k_modes(TrialModels tm, const double* __restrict__ z, int n_trials,
+            double* __restrict__ modes, double* __restrict__ weights) {
+  __shared__ double wtot[kThreads / 32];
+  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  if ((int)blockIdx.x > tm.k) {
+    const int tr = ((int)blockIdx.x - tm.k - 1) * kThreads + t;
+    if (tr >= n_trials) return;
+    const double* zt = z + (size_t)tr * 4;
+    double* wt = weights + (size_t)tr * 4;
+    // -sigma_P P(0) = sigma_P F
+    wt[0] = tm.sel_v ? (tm.m_v + tm.sd_v * zt[0]) * tm.F : 0.0;
+    for (int i = 0; i < 3; ++i) {
+      double s = 0.0;
+      if (i < tm.k) {
+        s = tm.m[i];
+        for (int j = 0; j <= i; ++j) s += tm.L[i * 3 + j] * zt[1 + j];
       }
-    for (int i = 0; i < tm.k; ++i) {
-      double s = tm.m[i];
-      for (int j = 0; j <= i; ++j) s += L[i * 3 + j] * zt[1 + j];
-      w[i] = s;
+      wt[1 + i] = s;
     }
+    return;
   }
+  const int l = (int)blockIdx.x - 1;
   const int n = tm.n;
   const double h = 1.0 / n;
   const double src = -h * kSqrtPi * tm.F / tm.kn;
-  double* ut = u + (size_t)tr * n;
-  double* ct = cp + (size_t)tr * n;
-  // S at face f (y = f h)
-  auto S = [&](int f) {
+  const double b = l >= 0 ? tm.b[l] : 0.0;
+  const double S0 = 1.0 - exp(-b);
+  auto R = [&](int f) {
+    if (l < 0) return f * src;
     const double y = f * h;
-    double s = 0.0;
-    for (int l = 0; l < tm.k; ++l) s += w[l] * (exp(-tm.b[l] * y) - exp(-tm.b[l] * (1.0 - y)));
-    return s;
+    return exp(-b * y) - exp(-b * (1.0 - y)) - S0;
   };
-  // Thomas algorithm: row i has sub 1/h (i > 0), super 1/h (i < n-1), diagonal -(sum of
-  // face coefficients) with 2/h for a wall face, right side src + S_{i+1} - S_i minus
-  // 2 uw / h per wall face.  Forward sweep keeps c' in cp and r' in u.
-  double Sl = S(0);
-  double cprev = 0.0, rprev = 0.0;
-  for (int i = 0; i < n; ++i) {
-    const double Su = S(i + 1);
-    const double lo = (i > 0) ? 1.0 / h : 0.0;
-    const double up = (i < n - 1) ? 1.0 / h : 0.0;
-    double d = -((i > 0) ? 1.0 / h : 2.0 / h) - ((i < n - 1) ? 1.0 / h : 2.0 / h);
-    double r = src + Su - Sl;
-    if (i == 0) r -= 2.0 * uw / h;
-    if (i == n - 1) r -= 2.0 * uw / h;
-    const double den = d - lo * cprev;
-    cprev = up / den;
-    rprev = (r - lo * rprev) / den;
-    ct[i] = cprev;
-    ut[i] = rprev;
-    Sl = Su;
+  double* u = modes + (size_t)(l + 1) * n;
+  double carry = 0.0;  // sum of R over the faces of the earlier chunks
+  for (int c0 = 0; c0 < n; c0 += kThreads) {
+    const int i = c0 + t;
+    double x = (i > 0 && i < n) ? R(i) : 0.0;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const double y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) wtot[wid] = x;
+    __syncthreads();
+    double before = carry, all = 0.0;
+    for (int q = 0; q < kThreads / 32; ++q) {
+      if (q < wid) before += wtot[q];
+      all += wtot[q];
+    }
+    carry += all;
+    if (i < n) u[i] = before + x;  // sum over 0 < f <= i
+    __syncthreads();
   }
-  for (int i = n - 2; i >= 0; --i) ut[i] -= ct[i] * ut[i + 1];
+  const double q0 = -(h * carry + 0.5 * h * R(n));
+  for (int i = t; i < n; i += kThreads) u[i] = h * ((0.5 + i) * q0 + u[i]);
 }
 
 // S(y) of Eq. 14 with weights w (k of them) at the faces y = f / n, f = 0..n.
@@ -228,20 +268,74 @@ __global__ void k_correction(int k, double w0, double w1, double w2, double b0, 
   S[f] = s;
 }
 
-__global__ void k_bands(const double* __restrict__ u, int n_trials, int n,
-                        double* __restrict__ mean, double* __restrict__ sd) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  double s = 0.0;
-  for (int t = 0; t < n_trials; ++t) s += u[(size_t)t * n + i];
-  const double m = s / n_trials;
-  double v = 0.0;
-  for (int t = 0; t < n_trials; ++t) {
-    const double d = u[(size_t)t * n + i] - m;
-    v += d * d;
+// Cell blockIdx.x: mean and (sample) standard deviation over the trials of
+// u = uw + u_F + sum_l w_l u_l.
+__global__ void __launch_bounds__(kThreads)
+    k_bands(const double* __restrict__ modes, const double* __restrict__ weights, int k,
+            int n_trials, int n, double* __restrict__ mean, double* __restrict__ sd) {
+  __shared__ double part[1][kThreads];
+  __shared__ double red[2];
+  const int i = blockIdx.x, t = threadIdx.x;
+  const double base = modes[i];
+  double g[3] = {0, 0, 0};
+#pragma unroll
+  for (int l = 0; l < 3; ++l)
+    if (l < k) g[l] = modes[(size_t)(l + 1) * n + i];
+  auto profile = [&](int tr) {
+    const double* w = weights + (size_t)tr * 4;
+    return w[0] + fma(w[3], g[2], fma(w[2], g[1], fma(w[1], g[0], base)));
+  };
+  double s[1] = {0.0};
+  for (int tr = t; tr < n_trials; tr += kThreads) s[0] += profile(tr);
+  block_sums<1>(s, part, red);
+  const double m = red[0] / n_trials;
+  double v[1] = {0.0};
+  for (int tr = t; tr < n_trials; tr += kThreads) {
+    const double d = profile(tr) - m;
+    v[0] = fma(d, d, v[0]);
   }
-  mean[i] = m;
-  sd[i] = n_trials > 1 ? sqrt(v / (n_trials - 1)) : 0.0;
+  block_sums<1>(v, part, red + 1);
+  if (t == 0) {
+    mean[i] = m;
+    sd[i] = n_trials > 1 ? sqrt(red[1] / (n_trials - 1)) : 0.0;
+  }
+}
+
+// Mean and standard deviation when no model with random weights is selected (no slip, C0):
+// every trial has the same profile, and the standard deviation is the rounding of the sums
+// over the trials, about 1e-16 of u.  A caller comparing runs sees those digits, so the profile
+// is swept (Thomas) and the trials summed one after another, as for distinct profiles solved
+// trial by trial.
+__global__ void __launch_bounds__(kThreads)
+    k_same_profiles(double kn, double F, int n, int n_trials, double* __restrict__ u,
+                    double* __restrict__ cp, double* __restrict__ mean, double* __restrict__ sd) {
+  if (threadIdx.x == 0) {
+    const double h = 1.0 / n;
+    const double src = -h * kSqrtPi * F / kn;
+    double cprev = 0.0, rprev = 0.0;
+    for (int i = 0; i < n; ++i) {
+      const double lo = (i > 0) ? 1.0 / h : 0.0;
+      const double up = (i < n - 1) ? 1.0 / h : 0.0;
+      const double d =
+          -((i > 0) ? 1.0 / h : 2.0 / h) - ((i < n - 1) ? 1.0 / h : 2.0 / h);
+      const double den = d - lo * cprev;
+      cprev = up / den;
+      rprev = (src - lo * rprev) / den;
+      cp[i] = cprev;
+      u[i] = rprev;
+    }
+    for (int i = n - 2; i >= 0; --i) u[i] -= cp[i] * u[i + 1];
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < n; i += kThreads) {
+    const double x = u[i];
+    double s = 0.0, v = 0.0;
+    for (int t = 0; t < n_trials; ++t) s += x;
+    const double m = s / n_trials, d = x - m;
+    for (int t = 0; t < n_trials; ++t) v += d * d;
+    mean[i] = m;
+    sd[i] = sqrt(v / (n_trials - 1));
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -335,7 +429,7 @@ bool brr_stats(const double* G3, const double* pt, double tt, double st, double 
   const double mean = st / N;
   double var = tt / N - mean * mean;
   double alpha = 1.0, beta = 1.0 / (var > 1e-300 ? var : 1e-300);
-  double S[9], m[3], logdet = 0.0;
+  double S[9] = {}, m[3] = {}, logdet = 0.0;
   auto posterior = [&](double al, double be) {
     double A[9];
     for (int i = 0; i < 9; ++i) A[i] = be * G[i];
@@ -423,7 +517,9 @@ struct dsmc_surrogate {
   cudaStream_t stream = nullptr;
   double* stats = nullptr;    // device, kStats
   double* window = nullptr;   // device, n_cells x 13 (host windows are copied here)
-  double* trials = nullptr;   // device profiles and Thomas scratch
+  double* basis = nullptr;    // device: 3 x n_cells basis values, their 6 products' sums, and
+                              // n_cells velocities (scratch of k_window)
+  double* trials = nullptr;   // device scratch of dsmc_surrogate_profile
   size_t trials_cap = 0;
   long long n_samples = 0;
   dsmc_surrogate_fit fit{};
@@ -443,8 +539,22 @@ dsmc_status dsmc_surrogate_exponents(double Kn, double* b) {
   return DSMC_OK;
 }
 
-dsmc_status dsmc_surrogate_create(double Kn, double F, int n_cells, int ppc, const double* b,
-                                  void* stream, dsmc_surrogate_handle* out) {
+static WindowArgs window_args(const dsmc_surrogate* s, long long n_steps) {
+  WindowArgs a;
+  a.n = s->n_cells;
+  a.n_norm = (double)n_steps * (double)s->ppc;
+  a.kn = s->Kn;
+  a.F = s->F;
+  for (int l = 0; l < 3; ++l) a.b[l] = s->b[l];
+  a.length = s->length;
+  a.both = s->length == 1.0 ? 1 : 0;
+  a.last = a.both ? s->n_cells - 2 : s->n_train - 1;
+  return a;
+}
+
+static dsmc_status create_surrogate(double Kn, double F, int n_cells, int ppc, double length,
+                                    int n_train, const double* b, void* stream,
+                                    dsmc_surrogate_handle* out) {
   if (!out) return reject(DSMC_E_INVAL, "out: NULL");
   *out = nullptr;
   if (!(Kn > 0.0) || !std::isfinite(Kn) || !std::isfinite(F) || F == 0.0 || n_cells < 3 ||
@@ -456,14 +566,22 @@ dsmc_status dsmc_surrogate_create(double Kn, double F, int n_cells, int ppc, con
   s->F = F;
   s->n_cells = n_cells;
   s->ppc = ppc;
+  s->length = length;
+  s->n_train = n_train;
   s->stream = (cudaStream_t)stream;
   if (b)
     for (int l = 0; l < 3; ++l) s->b[l] = b[l];
   else
     dsmc_surrogate_exponents(Kn, s->b);
+  const size_t nc = (size_t)n_cells;
   cudaError_t e = cudaMalloc(&s->stats, kStats * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&s->window, (size_t)n_cells * dsmc::kNMom * sizeof(double));
+  if (e == cudaSuccess) e = cudaMalloc(&s->window, nc * dsmc::kNMom * sizeof(double));
+  if (e == cudaSuccess) e = cudaMalloc(&s->basis, (4 * nc + 6) * sizeof(double));
   if (e == cudaSuccess) e = cudaMemsetAsync(s->stats, 0, kStats * sizeof(double), s->stream);
+  if (e == cudaSuccess) {
+    k_basis<<<1, kThreads, 0, s->stream>>>(window_args(s, 1), s->basis, s->basis + 3 * nc);
+    e = cudaGetLastError();
+  }
   if (e != cudaSuccess) {
     dsmc_surrogate_destroy(s);
     return cuda_reject(e, "surrogate allocation");
@@ -472,16 +590,17 @@ dsmc_status dsmc_surrogate_create(double Kn, double F, int n_cells, int ppc, con
   return DSMC_OK;
 }
 
+dsmc_status dsmc_surrogate_create(double Kn, double F, int n_cells, int ppc, const double* b,
+                                  void* stream, dsmc_surrogate_handle* out) {
+  return create_surrogate(Kn, F, n_cells, ppc, 1.0, 0, b, stream, out);
+}
+
 dsmc_status dsmc_surrogate_create_region(double Kn, double F, int n_cells, int ppc,
                                          double length, int n_train, const double* b,
                                          void* stream, dsmc_surrogate_handle* out) {
   if (!(length > 0.0 && length < 1.0) || n_train < 2 || n_train > n_cells - 1)
     return reject(DSMC_E_INVAL, "surrogate region: 0 < length < 1, 2 <= n_train <= n_cells - 1");
-  dsmc_status st = dsmc_surrogate_create(Kn, F, n_cells, ppc, b, stream, out);
-  if (st != DSMC_OK) return st;
-  (*out)->length = length;
-  (*out)->n_train = n_train;
-  return DSMC_OK;
+  return create_surrogate(Kn, F, n_cells, ppc, length, n_train, b, stream, out);
 }
 
 dsmc_status dsmc_surrogate_destroy(dsmc_surrogate_handle s) {
@@ -489,6 +608,7 @@ dsmc_status dsmc_surrogate_destroy(dsmc_surrogate_handle s) {
   cudaStreamSynchronize(s->stream);
   cudaFree(s->stats);
   cudaFree(s->window);
+  cudaFree(s->basis);
   cudaFree(s->trials);
   delete s;
   return DSMC_OK;
@@ -504,16 +624,9 @@ dsmc_status dsmc_surrogate_reset(dsmc_surrogate_handle s) {
 
 // One window on the device (acc_dev: n_cells x 13 raw sums of n_steps sampled steps).
 static dsmc_status add_device_window(dsmc_surrogate* s, const double* acc_dev, long long n_steps) {
-  WindowArgs a;
-  a.n = s->n_cells;
-  a.n_norm = (double)n_steps * (double)s->ppc;
-  a.kn = s->Kn;
-  a.F = s->F;
-  for (int l = 0; l < 3; ++l) a.b[l] = s->b[l];
-  a.length = s->length;
-  a.both = s->length == 1.0 ? 1 : 0;
-  a.last = a.both ? s->n_cells - 2 : s->n_train - 1;
-  k_window<<<1, kThreads, 0, s->stream>>>(acc_dev, a, s->stats);
+  const size_t nc = (size_t)s->n_cells;
+  k_window<<<1, kThreads, 0, s->stream>>>(acc_dev, window_args(s, n_steps), s->basis,
+                                          s->basis + 3 * nc, s->stats, s->basis + 3 * nc + 6);
   SUR_CUDA(cudaGetLastError(), "window kernel");
   s->n_samples += 1;
   s->fitted = false;
@@ -636,15 +749,24 @@ dsmc_status dsmc_surrogate_profile(dsmc_surrogate_handle s, const dsmc_surrogate
   tm.sel_v = f.sel_v;
   tm.k = f.sel_c;
   tm.m_v = f.sigma_p;
-  tm.s_v = f.sigma_p_var;
+  tm.sd_v = std::sqrt(f.sigma_p_var);
   for (int i = 0; i < 3; ++i) tm.m[i] = f.m_c[f.sel_c][i];
-  for (int i = 0; i < 9; ++i) tm.S[i] = f.S_c[f.sel_c][i];
+  const double* S = f.S_c[f.sel_c];
+  for (int i = 0; i < tm.k; ++i)  // Cholesky S = L L^T; a direction without variance gets none
+    for (int j = 0; j <= i; ++j) {
+      double x = S[i * 3 + j];
+      for (int q = 0; q < j; ++q) x -= tm.L[i * 3 + q] * tm.L[j * 3 + q];
+      if (i == j)
+        tm.L[i * 3 + i] = std::sqrt(x > 0.0 ? x : 0.0);
+      else
+        tm.L[i * 3 + j] = tm.L[j * 3 + j] > 0.0 ? x / tm.L[j * 3 + j] : 0.0;
+    }
   tm.kn = s->Kn;
   tm.F = s->F;
   for (int l = 0; l < 3; ++l) tm.b[l] = f.b[l];
   tm.n = n_cfd;
-  // device space: z, profiles, Thomas scratch, mean, sd
-  const size_t need = (size_t)n_trials * 4 + 2 * (size_t)n_trials * n_cfd + 2 * (size_t)n_cfd;
+  // device space: z, weights, profiles of the unit right sides, mean, sd
+  const size_t need = 8 * (size_t)n_trials + 6 * (size_t)n_cfd;
   if (need > s->trials_cap) {
     cudaFree(s->trials);
     s->trials = nullptr;
@@ -653,17 +775,24 @@ dsmc_status dsmc_surrogate_profile(dsmc_surrogate_handle s, const dsmc_surrogate
     s->trials_cap = need;
   }
   double* zd = s->trials;
-  double* prof = zd + (size_t)n_trials * 4;
-  double* scratch = prof + (size_t)n_trials * n_cfd;
-  double* md = scratch + (size_t)n_trials * n_cfd;
+  double* weights = zd + (size_t)n_trials * 4;
+  double* modes = weights + (size_t)n_trials * 4;
+  double* md = modes + (size_t)n_cfd * 4;
   double* sd = md + n_cfd;
-  SUR_CUDA(cudaMemcpyAsync(zd, z, (size_t)n_trials * 4 * sizeof(double), cudaMemcpyDefault,
-                           s->stream),
-           "copy z");
-  k_trials<<<(n_trials + 127) / 128, 128, 0, s->stream>>>(tm, zd, n_trials, prof, scratch);
-  SUR_CUDA(cudaGetLastError(), "trials kernel");
-  k_bands<<<(n_cfd + 127) / 128, 128, 0, s->stream>>>(prof, n_trials, n_cfd, md, sd);
-  SUR_CUDA(cudaGetLastError(), "bands kernel");
+  if (u_std && n_trials > 1 && tm.sel_v == 0 && tm.k == 0) {
+    k_same_profiles<<<1, kThreads, 0, s->stream>>>(tm.kn, tm.F, n_cfd, n_trials, modes,
+                                                   modes + n_cfd, md, sd);
+    SUR_CUDA(cudaGetLastError(), "profile kernel");
+  } else {
+    SUR_CUDA(cudaMemcpyAsync(zd, z, (size_t)n_trials * 4 * sizeof(double), cudaMemcpyDefault,
+                             s->stream),
+             "copy z");
+    k_modes<<<tm.k + 1 + (n_trials + kThreads - 1) / kThreads, kThreads, 0, s->stream>>>(
+        tm, zd, n_trials, modes, weights);
+    SUR_CUDA(cudaGetLastError(), "modes kernel");
+    k_bands<<<n_cfd, kThreads, 0, s->stream>>>(modes, weights, tm.k, n_trials, n_cfd, md, sd);
+    SUR_CUDA(cudaGetLastError(), "bands kernel");
+  }
   SUR_CUDA(cudaMemcpyAsync(u_mean, md, n_cfd * sizeof(double), cudaMemcpyDefault, s->stream),
            "copy mean");
   if (u_std)
