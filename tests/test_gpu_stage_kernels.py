@@ -1,13 +1,26 @@
 """The surrogate stage's kernels at the edges of their chunks and tiles, against the oracle.
 
 Tolerances: the CFD profiles are sums of n terms of one sign pattern in binary64 (rounding of
-about n 2^-53 of the largest value, bounded here by 1e-11)."""
+about n 2^-53 of the largest value, bounded here by 1e-11); the GP's marginal likelihoods and
+predictions as in the tests of the larger designs."""
 import numpy as np
 import pytest
 
+from oracle import gp as GP
 from oracle import surrogate as S
 
 pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 33, 255, 256, 257, 1000])
+def test_face_cfd_sizes(n):
+    from paper_2311_14140_gb300 import cfd_faces
+    Kn, F = 0.3, 5e-3
+    Sf = S.stress_correction(np.arange(n + 1) / n, (0.3, -0.1), S.exponents(Kn)[:2])
+    for sp in (None, 1.1):
+        want = GP.cfd_faces(Kn, F, n, sp, Sf)
+        np.testing.assert_allclose(cfd_faces(Kn, F, n, sp, Sf), want, rtol=0,
+                                   atol=1e-11 * np.abs(want).max())
 
 
 @pytest.mark.parametrize("n_cfd,trials", [(1, 2), (2, 1), (33, 255), (256, 257), (257, 256),
@@ -41,3 +54,33 @@ def test_bands_of_a_given_fit(n_cfd, trials, k):
     np.testing.assert_allclose(mean, prof.mean(axis=0), rtol=0, atol=1e-11 * scale)
     want = prof.std(axis=0, ddof=1) if trials > 1 else np.zeros(n_cfd)
     np.testing.assert_allclose(sd, want, rtol=0, atol=1e-11 * scale)
+
+
+@pytest.mark.parametrize("n,m", [(2, 1), (3, 7), (17, 8), (33, 9), (127, 3), (128, 40)])
+def test_gp_sizes(n, m):
+    from paper_2311_14140_gb300 import GaussianProcess
+    rng = np.random.default_rng(n)
+    X = rng.uniform(size=(n, 2))
+    Y = np.sin(3 * X[:, :1]) * np.linspace(0.5, 2, m) + 0.1 * rng.normal(size=(n, m))
+    g = GaussianProcess(X, Y, GP.GRID)
+    o = GP.fit(X, Y)
+    np.testing.assert_allclose(g.lml, o["lml"], rtol=1e-9, atol=1e-9 * n * m)
+    assert g.best == o["best"]
+    Xs = rng.uniform(size=(5, 2))
+    np.testing.assert_allclose(g.predict(Xs), GP.predict(o, Xs), rtol=1e-8,
+                               atol=1e-10 * np.abs(Y).max())
+
+
+def test_gp_grid_larger_than_one_chunk():
+    """6,001 hyperparameter points of 64-point factors take more than one chunk; the chosen
+    point lies in the first, so its factor is formed again."""
+    from paper_2311_14140_gb300 import GaussianProcess
+    rng = np.random.default_rng(1)
+    X = rng.uniform(size=(64, 2))
+    Y = np.sin(3 * X[:, :1]) + 0.1 * rng.normal(size=(64, 2))
+    grid = [(0.4, 1.0, 1e-2)] + [(0.05, 0.05, 0.3 + 1e-4 * i) for i in range(6000)]
+    g = GaussianProcess(X, Y, grid)
+    o = GP.fit(X, Y, grid[:3])
+    assert g.best == o["best"]
+    Xs = rng.uniform(size=(5, 2))
+    np.testing.assert_allclose(g.predict(Xs), GP.predict(o, Xs), rtol=1e-8, atol=1e-10)
