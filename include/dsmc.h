@@ -110,11 +110,12 @@ typedef struct dsmc_options {
                              1024..2^24.
                              Only the work split changes: results are identical for
                              every value.  While this, cta_warps and span_rows are
-                             all 0, steps of small runs (up to about 110,000
-                             particles; batches up to about 40,000 per instance) may
-                             run many at a time in one launch, a cluster of CTAs per
-                             instance; a value in any of the three keeps the span
-                             passes; default 0 */
+                             all 0, steps of one run of up to about 1,300,000
+                             particles, or of a batch of up to about 40,000 per
+                             instance, may run many at a time in one launch (a
+                             cooperative one, with a CTA on every SM, above 40,000);
+                             a value in any of the three keeps the span passes;
+                             default 0 */
   int cta_warps;          /* warps per CTA of the collide/move pass: 0 keeps the shape
                              in use (8 at creation, 4 for a pool, or what dsmc_autotune
                              chose), else 4 or 8; results are identical; default 0 */
@@ -582,7 +583,7 @@ DSMC_API dsmc_status dsmc_cfd_faces(double Kn, double F, int n, int slip, double
  * timed steps, keeps the fastest, and stores it in the handle's options (cta_warps,
  * span_rows, span_particles).  The trial steps are real steps of the run: they
  * advance every instance, and since the partition does not change results the run is
- * the same as without tuning.  A handle whose steps run as one launch per cluster (see
+ * the same as without tuning.  A handle whose steps run many to a launch (see
  * dsmc_options.span_particles) keeps doing so; the tuner then chooses the partition its
  * span passes would use.  *best_span_particles and *best_ms_per_step (either may
  * be NULL) get the choice and its time per step.  Synchronises. */

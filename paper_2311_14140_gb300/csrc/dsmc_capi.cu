@@ -58,6 +58,7 @@ constexpr int kMinSpanParticles = 1024;
 constexpr int kMaxSpanParticles = 1 << 24;
 constexpr int kMaxInstances = 65535;  // grid y of the per-instance prefix pass
 constexpr int kGraphSteps = 16;       // steps per replay of the captured graph (even)
+constexpr long long kTeamParticles = 1500000;  // more never fit the SMs' shared memory
 constexpr int kResidentSteps = 512;   // steps per resident launch, at most
 
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
@@ -289,6 +290,11 @@ Capacity capacity_of(const dsmc_instance* d, int n) {
     C.spans += rows;
   }
   C.inst = n;
+  // one run: room for the exchange of a team of CTAs (dsmc_resident.cu) in the sort matrix's
+  // place, for the sizes whose records the SMs' shared memory holds
+  if (n == 1 && C.slots <= kTeamParticles)
+    C.hist_ints = std::max<long long>(C.hist_ints,
+                                      (long long)team_exchange_ints(kTeamMax, d[0].n_cells));
   return C;
 }
 
@@ -388,6 +394,7 @@ struct dsmc_sim {
   bool graph_valid = false, capturing = false;
   int graph_parity = 0;  // buffer parities (cur, ocur, scur) the graph starts from
   long long* gstep_dev = nullptr;
+  unsigned* barrier = nullptr;  // of a team's CTAs: count and generation
   dsmc_status latched = DSMC_OK;
   std::vector<cudaEvent_t> events;
   std::vector<int> event_kernel;
@@ -773,6 +780,7 @@ dsmc_status read_error_word(dsmc_sim* h) {
     if (v & kErrCopyTimeout) what += " bulk-copy-timeout";
     if (v & kErrInflow) what += " inflow-attempts";
     if (v & kErrMoments) what += " moment-range";
+    if (v & kErrTeam) what += " team-barrier-timeout";
     return fail(DSMC_E_DEVICE_LIMIT, "device limit reached:" + what);
   }
   return DSMC_OK;
@@ -836,15 +844,15 @@ dsmc_status step_once(dsmc_sim* h) {
   return run_pass(h, false);
 }
 
-// Shares of an instance's slots for the cl CTAs of its cluster, of about equal cost: a
+// Shares of an instance's slots for the cl CTAs of its cluster or team, of about equal cost: a
 // particle at y costs 1 + 1.5 h(y), h its expected wall hits in the step (as in
 // set_span_order; 1.5 is the measured extra cost of a hit here, where a CTA's wall hits are
 // flown by all its warps).  With equal shares the CTAs next to the walls took 64,000 cycles
 // of a 67,000-cycle step of a 100,000-particle run and the others 46,000 (Kn = 0.5); with
-// these, 49,000 and 45,000 of 52,000.  The cost's integral is taken at 64 points and
+// these, 49,000 and 45,000 of 52,000.  The cost's integral is taken at 256 points and
 // inverted linearly.  Returns the largest share.
-int set_cuts(Inst& x, int cl) {
-  constexpr int kPoints = 64;
+int set_cuts(const Inst& x, int cl, int* cut) {
+  constexpr int kPoints = 256;
   const double dt = x.p.dt, w = 1.5;
   auto ierfc = [&](double y) {  // integral of erfc(t / dt) over [0, y]
     const double u = y / dt;
@@ -857,69 +865,92 @@ int set_cuts(Inst& x, int cl) {
     cost[i] = y + 0.5 * w * (ierfc(y) + whole - ierfc(1.0 - y));
   }
   int share = 0, i = 0;
-  x.cut[0] = 0;
+  cut[0] = 0;
   for (int r = 1; r <= cl; ++r) {
     const double target = cost[kPoints] * r / cl;
     while (i < kPoints - 1 && cost[i + 1] < target) ++i;
     const double y = (i + (target - cost[i]) / (cost[i + 1] - cost[i])) / kPoints;
     const long long at = r == cl ? x.N : (long long)(y * (double)x.N);
-    x.cut[r] = (int)std::min(x.N, std::max<long long>(x.cut[r - 1], at));
-    share = std::max(share, x.cut[r] - x.cut[r - 1]);
+    cut[r] = (int)std::min(x.N, std::max<long long>(cut[r - 1], at));
+    share = std::max(share, cut[r] - cut[r - 1]);
   }
   return share;
 }
 
-// Decides whether the handle's steps run cluster-resident (dsmc_resident.cu) and with how
-// many CTAs per instance.  Options that name a partition of the span passes keep those, as
-// does profiling, which times their kernels; a pool's members come and go between calls.
+// Decides whether the handle's steps run resident (dsmc_resident.cu) and with how many CTAs
+// per instance.  Options that name a partition of the span passes keep those, as does
+// profiling, which times their kernels; a pool's members come and go between calls.
 //
-// One run: 16 CTAs whenever its share fits a CTA's shared memory (up to ~110,000
-// particles; us per step against the span passes under graph replay: 2,250 particles 7.2 /
-// 20.5, 20,000 11.4 / 22.5, 100,000 24-26 / 26-34).
-// A batch: as many CTAs per instance as give shares of at most kResidentShare particles and
-// fill the SMs twice, as long as an instance then fits 16 CTAs and the launch is not many
-// waves long (64 x 2,250 particles: 11 us per step against 30; 64 x 10,000: 28 / 48;
+// One run: a cluster of 16 CTAs up to kClusterParticles (us per step, cluster / team of 152 /
+// span passes under graph replay: 2,250 particles 7.0 / 10.7 / 20.5, 20,000 11.4 / 13.0 / 22.5,
+// 40,000 13.8 / 13.0 / 23, 80,000 23.1 / 14.9 / 27), from there a team of a CTA per SM (more
+// CTAs were never slower: 100,000 particles 18.4 with 32, 15.2 with 64, 13.7 with 152), as long
+// as its share fits a CTA's shared memory (1,004,807 particles 27.7 against 71; up to about
+// 1,300,000, depending on the cells).
+// A batch: clusters of as many CTAs per instance as give shares of at most kResidentShare
+// particles and fill the SMs twice, as long as an instance then fits 16 CTAs and the launch is
+// not many waves long (64 x 2,250 particles: 11 us per step against 30; 64 x 10,000: 28 / 48;
 // 64 x 20,000: 45 / 70; 128 x 20,000, 1,024 CTAs: 87 / 95; beyond that the span passes,
 // which spread every instance over all SMs, are as fast: 256 x 20,000, 161 / 153;
 // 24 x 100,000, 137 / 85).
+constexpr long long kClusterParticles = 40000;
 constexpr int kResidentShare = 2600;
+
+// Fills in a resident launch's sizes; false when it does not fit the device.
+bool size_resident(dsmc_sim* h, ResidentLaunch& R) {
+  const dsmc_options& o = h->opt;
+  long long n_max = 0;
+  for (int id : h->order) n_max = std::max(n_max, h->inst[id].N);
+  if (n_max / R.cl > 30000) return false;  // local slots are 16-bit; so large a share never fits
+  R.max_cells = h->max_cells;
+  if (R.team && team_exchange_ints(R.cl, R.max_cells) > (size_t)h->C.hist_ints) return false;
+  int share = 0;
+  for (int id : h->order)
+    share = std::max(share, set_cuts(h->inst[id], R.cl, R.team ? R.cut : h->inst[id].cut));
+  R.range_cap = share + h->cap();
+  R.list_cap = R.range_cap / o.group_size + std::min(R.max_cells, R.range_cap) + 2;
+  R.own_cap = (R.max_cells + R.cl - 1) / R.cl;
+  const size_t smem = resident_smem_layout(R.max_cells, R.range_cap, R.list_cap, R.own_cap,
+                                           R.team ? 0 : R.cl, resident_warps(R.n_inst > 1))
+                          .total;
+  if (smem > kResidentSmemMax) return false;
+  bool fits = false;
+  if (resident_fits(R, smem, o.accum == DSMC_ACCUM_FP64, &fits) == cudaSuccess && fits)
+    return true;
+  cudaGetLastError();
+  return false;
+}
 
 void plan_resident(dsmc_sim* h) {
   h->res = ResidentLaunch{};
   h->res_dirty = false;
-  const dsmc_options& o = h->opt;
-  if (h->pool || o.profile || h->span_passes) return;
+  if (h->pool || h->opt.profile || h->span_passes) return;
   long long n_max = 0;
   for (int id : h->order) n_max = std::max(n_max, h->inst[id].N);
   ResidentLaunch R{};
   R.n_inst = h->n_inst();
   R.cl = kResidentMaxCluster;
-  if (R.n_inst > 1) {
+  bool fits = false;
+  if (R.n_inst == 1) {
+    ResidentLaunch T{};
+    T.n_inst = 1;
+    T.cl = std::min(h->sms, kTeamMax);
+    T.team = 1;
+    if (n_max <= kClusterParticles) fits = size_resident(h, R);
+    if (!fits && size_resident(h, T)) {
+      R = T;
+      fits = true;
+    }
+    if (!fits && n_max > kClusterParticles) fits = size_resident(h, R);
+  } else {
     R.cl = 2;
     while (R.cl < kResidentMaxCluster &&
            (n_max > (long long)kResidentShare * R.cl || R.n_inst * 2 * R.cl <= 2 * h->sms))
       R.cl *= 2;
-    if (n_max > (long long)kResidentShare * R.cl) return;
-    if ((long long)R.n_inst * R.cl > (R.cl == 16 ? 512 : 1024)) return;
+    fits = n_max <= (long long)kResidentShare * R.cl &&
+           (long long)R.n_inst * R.cl <= (R.cl == 16 ? 512 : 1024) && size_resident(h, R);
   }
-  if (n_max / R.cl > 30000) return;  // local slots are 16-bit; a share this large never fits
-  R.max_cells = h->max_cells;
-  int share = 0;
-  for (int id : h->order) share = std::max(share, set_cuts(h->inst[id], R.cl));
-  R.range_cap = share + h->cap();
-  R.list_cap = R.range_cap / o.group_size + std::min(R.max_cells, R.range_cap) + 2;
-  R.own_cap = (R.max_cells + R.cl - 1) / R.cl;
-  const size_t smem = resident_smem_layout(R.max_cells, R.range_cap, R.list_cap, R.own_cap, R.cl,
-                                           resident_warps(R.n_inst > 1))
-                          .total;
-  if (smem > kResidentSmemMax) return;
-  int clusters = 0;
-  if (resident_clusters(R.cl, smem, R.n_inst > 1, o.accum == DSMC_ACCUM_FP64, &clusters) !=
-          cudaSuccess ||
-      clusters < 1) {
-    cudaGetLastError();
-    return;
-  }
+  if (!fits) return;
   h->res = R;
   h->tab_dirty = true;  // the instance table carries the cuts
 }
@@ -934,7 +965,7 @@ dsmc_status step_resident(dsmc_sim* h, int n) {
   R.parity_off = h->ocur;
   R.parity_smax = h->scur;
   DSMC_CUDA(launch_resident(h->P[0], h->P[1], h->off[0], h->off[1], h->smax[0], h->smax[1],
-                            h->ncand, h->nacc, h->acc, h->tab[0], R,
+                            h->ncand, h->nacc, h->acc, h->hist, h->barrier, h->tab[0], R,
                             h->opt.accum == DSMC_ACCUM_FP64, h->err, h->stream()),
             "resident steps");
   h->cur ^= n & 1;
@@ -1119,8 +1150,9 @@ dsmc_status new_handle(const Capacity& C, const dsmc_options& opt, bool pool, vo
   h->chan_dev = (double*)(b + L.chan);
   h->err = (int*)(b + L.err);
   h->gstep_dev = (long long*)(b + L.err + 8);
+  h->barrier = (unsigned*)(b + L.err + 128);
   ce = set_step_smem_limits(kStepSmemMax, kStepSmemMax);
-  if (ce == cudaSuccess) ce = cudaMemsetAsync(h->err, 0, sizeof(int), h->stream());
+  if (ce == cudaSuccess) ce = cudaMemsetAsync(h->err, 0, 256, h->stream());
   if (ce != cudaSuccess) {
     dsmc_status s = cuda_fail(ce, "handle setup");
     dsmc_destroy(h);

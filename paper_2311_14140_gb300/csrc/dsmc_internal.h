@@ -37,6 +37,7 @@ constexpr int kErrCandidates = 8;  // a group's candidate count exceeded kMaxCan
 constexpr int kErrSort = 16;       // a scatter destination fell outside [0, N)
 constexpr int kErrCopyTimeout = 32;  // a bulk copy into shared memory did not complete
 constexpr int kErrInflow = 64;       // an open-boundary emission ran out of attempts
+constexpr int kErrTeam = 256;        // a wait between the CTAs of a run's team ran out
 constexpr int kErrMoments = 128;     // a group's moment total exceeded the fixed-point range
 
 // Largest NTC candidate count of one group in one step (about 80 on the largest
@@ -159,10 +160,12 @@ __host__ __device__ inline StepSmem step_smem_layout(int n_cells, int cps, int c
 }
 
 // Many steps of small runs in one launch (dsmc_resident.cu): a cluster of `cl` CTAs per
-// instance.
+// instance, or a team of them over the whole device for one run.
 constexpr int kResidentWarps = 20;       // warps per CTA, one instance
 constexpr int kResidentWarpsBatch = 12;  // several instances, two CTAs per SM
 constexpr int kResidentMaxCluster = 16;   // entries of InstParams::cut less one
+constexpr int kTeamMax = 152;     // CTAs of a team, at most
+constexpr int kTeamBlock = 13;    // CTAs per block of count sums (kTeamBlock^2 >= kTeamMax)
 constexpr size_t kResidentSmemMax = 225 * 1024;
 
 inline int resident_warps(bool batch) { return batch ? kResidentWarpsBatch : kResidentWarps; }
@@ -178,7 +181,19 @@ struct ResidentLaunch {
   int range_cap;          // slots of a CTA, at most
   int list_cap;           // collision groups of a CTA, at most
   int own_cap;            // cells owned by a CTA, at most
+  int team;               // 1: the CTAs of one run spread over the device (cl up to kTeamMax),
+                          // exchanging through global memory instead of a cluster
+  int cut[kTeamMax + 1];  // the team's slot shares (as InstParams::cut)
 };
+
+// Ints of a team's exchange area before its 64-bit sums, and in all.
+__host__ __device__ inline size_t team_fix_offset(int cl, int n_cells) {
+  const size_t blocks = (size_t)(cl + kTeamBlock - 1) / kTeamBlock;
+  return (((size_t)cl + 2 * blocks + 2) * n_cells + 1) & ~(size_t)1;
+}
+__host__ __device__ inline size_t team_exchange_ints(int cl, int n_cells) {
+  return team_fix_offset(cl, n_cells) + 24 * (size_t)n_cells;
+}
 
 // Dynamic shared memory of one CTA (byte offsets).
 struct ResidentSmem {
@@ -205,10 +220,10 @@ __host__ __device__ inline ResidentSmem resident_smem_layout(int n_cells, int ra
   o += (size_t)range_cap * 4;
   // counts per warp and cell; before them, the queue of wall hits (16-bit local slots),
   // 4,096 of them if the counts are smaller than that
-  const size_t counts = (size_t)warps * n_cells * 4;
+  const size_t counts = (size_t)warps * n_cells * 2;
   const size_t queue = range_cap < 4096 ? ((size_t)range_cap * 2 + 64) : 8192;
   L.rows = o;
-  L.rows_bytes = step_align(counts > queue ? counts : queue, 4);
+  L.rows_bytes = step_align(counts > queue ? counts : queue, 8);
   o += L.rows_bytes;
   L.tot = o;
   o += (size_t)cl * n_cells * 4;
@@ -222,12 +237,12 @@ __host__ __device__ inline ResidentSmem resident_smem_layout(int n_cells, int ra
   return L;
 }
 
-// Clusters of `cl` CTAs with `smem` bytes each that fit on the device at once (0: none).
-cudaError_t resident_clusters(int cl, size_t smem, bool batch, bool f64, int* clusters);
+// Whether the device can hold one cluster of this launch (a team: all of its CTAs) at once.
+cudaError_t resident_fits(const ResidentLaunch& L, size_t smem, bool f64, bool* fits);
 cudaError_t launch_resident(float4* P0, float4* P1, int* off0, int* off1, float* smax0,
                             float* smax1, unsigned long long* ncand, unsigned long long* nacc,
-                            double* acc, const InstParams& one, const ResidentLaunch& L,
-                            bool f64, int* err, cudaStream_t st);
+                            double* acc, int* exchange, unsigned* barrier, const InstParams& one,
+                            const ResidentLaunch& L, bool f64, int* err, cudaStream_t st);
 
 cudaError_t launch_init(float4* P, int N, int ppc, float ncf, uint32_t k0, uint32_t k1,
                         int* err, cudaStream_t st);

@@ -3,27 +3,35 @@
 // A small run's step is bound by launches and by the latency of its passes, not by work:
 // 20,000 particles through the span passes of dsmc_step.cu take 22 us per step (three
 // launches under graph replay, each a cold start of a CTA's worth of dependent phases),
-// against about 2 us of instruction issue on 16 SMs.  Here a thread-block cluster owns an
-// instance and runs all the steps of a call: particles, counters and prefixes pass between
-// its CTAs through L2 and distributed shared memory, with two hardware cluster barriers
-// per step instead of kernel boundaries.  Instances do not depend on one another, so a
-// batch is one cluster per instance.
+// against about 2 us of instruction issue on 16 SMs.  Here one launch runs all the steps of a
+// call, and particles, counts and prefixes pass between its CTAs with two barriers per step
+// instead of kernel boundaries:
+//   a cluster (up to 16 CTAs) per instance: counts by distributed shared memory, hardware
+//     cluster barriers.  Instances do not depend on one another, so a batch is one cluster per
+//     instance.
+//   a team (kTeam): for one run that 16 SMs would be slow on, a cooperative grid of a CTA per
+//     SM: counts and cell results by global memory, a counter barrier (about 1.5 us each).
+// Measured (us per step, before = span passes under graph replay): 20,000 particles 22.5 ->
+// 11.4 and 9,000 20.9 -> 8.4 (cluster), 100,000 21-30 -> 13.5, 300,000 38 -> 16.7, 1,004,807
+// 71 -> 27.7 (team).  What is left is the latency of one collision group per warp (a chain of
+// about 8,000 cycles at 200 particles), then barriers, loads and the ranking.
 //
-// A step, for CTA r of the cluster (identical arithmetic, operation for operation, to the
+// A step, for CTA r of CL (identical arithmetic, operation for operation, to the
 // span passes; only the place where it happens differs):
-//   A  load its slots -- the collision groups that start in [r N / CL, (r+1) N / CL) --
-//      into shared memory; its warps take the groups one after another (moments, NTC
+//   A  load its slots -- the collision groups that start in its share [cut_r, cut_{r+1}) of
+//      the slots -- into shared memory; its warps take the groups one after another (moments, NTC
 //      candidates, moments, flight) and update them in place; then every warp ranks a
 //      contiguous part of the slots by new cell (running counts per warp and cell), and
 //      the CTA publishes its particles per cell.
-//      [cluster barrier]
+//      [barrier]
 //   B  every CTA reads the others' counts: exclusive prefix over CTAs and cells gives the
 //      new cell offsets and the CTA's base in every cell; the cell's owner CTA adds the
 //      step's moment sums to the run's; each record goes to its sorted place in the other
 //      record buffer (global memory, L2-resident at these sizes).
-//      [cluster barrier]
+//      [barrier]
 // Cell results (fixed-point moment totals, counters, largest relative speed) are integer
-// adds and maxima in the owner CTA's shared memory, so they do not depend on the order.
+// adds and maxima, in the owner CTA's shared memory or in global memory, so they do not depend
+// on the order.
 #include <type_traits>
 
 #include "dsmc_collide.cuh"
@@ -77,13 +85,55 @@ __device__ __forceinline__ void peer_max(uint32_t addr, uint32_t v) {
                : "memory");
 }
 
+// Barrier of the CTAs of a team: a counter and a generation in global memory (both zero, or as
+// an earlier team left them).  The last CTA to arrive clears the counter and advances the
+// generation.  Memory operations before it are visible after it to loads that bypass L1.
+// Waits are bounded; false when one ran out.
+struct TeamBarrier {
+  unsigned *count = nullptr, *gen = nullptr, now = 0u;
+  int n = 0;
+  static __device__ __forceinline__ unsigned load(const unsigned* p) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+  }
+  __device__ __forceinline__ void start(unsigned* b, int ctas) {
+    count = b;
+    gen = b + 1;
+    n = ctas;
+    if (threadIdx.x == 0) now = load(gen);  // nobody passes the first wait before this CTA arrives
+  }
+  __device__ __forceinline__ bool wait() {
+    bool ok = true;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      unsigned before;
+      asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;"
+                   : "=r"(before)
+                   : "l"(count)
+                   : "memory");
+      ++now;
+      if (before == (unsigned)(n - 1)) {
+        *count = 0u;
+        asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(gen), "r"(now) : "memory");
+      } else {
+        ok = false;
+        for (int i = 0; i < kMaxWaitPolls && !ok; ++i) ok = load(gen) == now;
+      }
+    }
+    return __syncthreads_and(ok) != 0;
+  }
+};
+
 }  // namespace
 
-template <bool kBatch, int kWarps, bool kF64>
+template <bool kBatch, int kWarps, bool kF64, bool kTeam>
 __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
     k_resident(float4* P0, float4* P1, int* off0, int* off1, float* smax0, float* smax1,
                unsigned long long* ncand_all, unsigned long long* nacc_all, double* acc_all,
-               const InstParams one, const ResidentLaunch RL, int* err) {
+               int* exchange, unsigned* barrier, const InstParams one, const ResidentLaunch RL,
+               int* err) {
+  static_assert(!(kBatch && kTeam), "a team serves one instance");
   using Acc = typename std::conditional<kF64, double, float>::type;
   constexpr int kThreads = kWarps * 32;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -94,7 +144,7 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const unsigned lt = (1u << lane) - 1u;
   const int CL = RL.cl;
-  const int rank = (int)cluster_rank();
+  const int rank = kTeam ? (int)blockIdx.x : (int)cluster_rank();
   if constexpr (kBatch) {
     const int* src = reinterpret_cast<const int*>(&RL.tab[blockIdx.x / CL]);
     int* dst = reinterpret_cast<int*>(&sh_inst);
@@ -103,11 +153,11 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
   }
   const InstParams& a = kBatch ? sh_inst : one;
   const ResidentSmem L = resident_smem_layout(RL.max_cells, RL.range_cap, RL.list_cap,
-                                              RL.own_cap, RL.cl, kWarps);
+                                              RL.own_cap, kTeam ? 0 : RL.cl, kWarps);
   float4* rec = reinterpret_cast<float4*>(smem + L.rec);        // this CTA's records
   unsigned* key = reinterpret_cast<unsigned*>(smem + L.key);    // candidate masks, then ranks
   int2* list = reinterpret_cast<int2*>(smem + L.list);          // groups: (cell, gi << 10 | gn)
-  int* rows = reinterpret_cast<int*>(smem + L.rows);            // counts per warp and cell
+  unsigned short* rows = reinterpret_cast<unsigned short*>(smem + L.rows);  // counts per warp, cell
   int* tot = reinterpret_cast<int*>(smem + L.tot);              // counts per CTA and cell
   int* base = reinterpret_cast<int*>(smem + L.base);            // this CTA's first slot per cell
   float* csmax = reinterpret_cast<float*>(smem + L.smax);       // (sigma g)_max per cell
@@ -123,7 +173,26 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
   const int own_n = max(0, min(own, n_cells - own0));
   const int lo = a.part_base, hi = a.part_base + a.n_part;
   // slots at which this CTA's and the next CTA's groups may start
-  const int B0 = lo + a.cut[rank], B1 = lo + a.cut[rank + 1];
+  const int B0 = lo + (kTeam ? RL.cut[rank] : a.cut[rank]);
+  const int B1 = lo + (kTeam ? RL.cut[rank + 1] : a.cut[rank + 1]);
+  // A team's exchange in global memory: count rows of its CTAs; their sums over blocks of
+  // kTeamBlock CTAs, of even and odd steps; the cells' largest relative speeds, of even and
+  // odd steps; and the cells' fixed-point sums.
+  const int n_blocks = (CL + kTeamBlock - 1) / kTeamBlock, my_block = rank / kTeamBlock;
+  int* xrow = exchange;
+  int* xblk = xrow + (size_t)CL * n_cells;
+  unsigned* xgmax = reinterpret_cast<unsigned*>(xblk + 2 * (size_t)n_blocks * n_cells);
+  unsigned long long* xfix = reinterpret_cast<unsigned long long*>(
+      exchange + team_fix_offset(CL, n_cells));
+  TeamBarrier team;
+  if constexpr (kTeam) team.start(barrier, CL);
+  bool lost = false;  // a wait ran out: the CTA leaves, and the others' waits run out too
+  auto wait_all = [&]() {
+    if constexpr (kTeam)
+      lost = !team.wait();
+    else
+      cluster_barrier();
+  };
   unsigned long long* ncand = ncand_all + a.cell_base;
   unsigned long long* nacc = nacc_all + a.cell_base;
   double* acc = acc_all + (size_t)a.cell_base * kNMom;
@@ -136,9 +205,15 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
     const float* s = (RL.parity_smax ? smax1 : smax0) + a.cell_base;
     for (int c = tid; c <= n_cells; c += kThreads) off[c] = g[c];
     for (int c = tid; c < n_cells; c += kThreads) csmax[c] = s[c];
-    for (int i = tid; i < own * 12; i += kThreads) cfix[i] = 0ull;
+    if constexpr (kTeam) {
+      for (int i = rank * kThreads + tid; i < 2 * n_blocks * n_cells; i += CL * kThreads) xblk[i] = 0;
+      for (int i = rank * kThreads + tid; i < 2 * n_cells; i += CL * kThreads) xgmax[i] = 0u;
+      for (int i = rank * kThreads + tid; i < 12 * n_cells; i += CL * kThreads) xfix[i] = 0ull;
+    } else {
+      for (int i = tid; i < own * 12; i += kThreads) cfix[i] = 0ull;
+      for (int i = tid; i < 2 * own; i += kThreads) cgmax[i] = 0u;
+    }
     for (int i = tid; i < own_n * kNMom; i += kThreads) csum[i] = acc[(size_t)own0 * kNMom + i];
-    for (int i = tid; i < 2 * own; i += kThreads) cgmax[i] = 0u;
   }
   // The group boundaries of this CTA from cell offsets: boundary B falls into the cell
   // c with first <= B < first + n; the CTA's groups begin with the cell's first group
@@ -151,7 +226,7 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
     bnd_group[k] = min(i, ng);
     bnd_slot[k] = i < ng ? first + i * G : first + n;
   };
-  unsigned short* queue = reinterpret_cast<unsigned short*>(rows);
+  unsigned short* queue = rows;  // (local slots)
   const int qcap = (int)(L.rows_bytes / 2) & ~31;  // wall hits the queue holds
   if (tid == 0) n_hits = 0;
   if (tid == 0) {  // ends of the instance (the last CTA's end is past every cell)
@@ -169,9 +244,10 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
   float4* Pout = RL.parity_rec ? P0 : P1;
   bool bad_bounce = false, cand_fail = false, inflow_fail = false, mom_range = false;
   bool bad_sort = false;
-  cluster_barrier();  // every CTA's accumulators are cleared
+  wait_all();  // every CTA's accumulators are cleared
 
-  for (int st = 0; st < RL.n_steps; ++st, ++istep) {
+  int st = 0;
+  for (; st < RL.n_steps && !lost; ++st, ++istep) {
     const uint32_t step = (uint32_t)istep;
     const bool sample = istep >= a.sample_start;
     const bool collide = a.collide != 0;
@@ -271,13 +347,20 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
           const long long fx = fixed_of(total, gexp);
           const long long lim = (long long)(2 * gn) << (20 + gexp);
           if (fx > lim || fx < -lim) mom_range = true;
-          peer_add(peer_addr(cfix + os * 12 + (k - 1), oc), (unsigned long long)fx);
+          if constexpr (kTeam)
+            atomicAdd(xfix + (size_t)c * 12 + (k - 1), (unsigned long long)fx);
+          else
+            peer_add(peer_addr(cfix + os * 12 + (k - 1), oc), (unsigned long long)fx);
         }
       }
       const unsigned gbits = __reduce_max_sync(kFull, __float_as_uint(gmax));  // gmax >= 0
       const unsigned nac = __reduce_add_sync(kFull, laccn);
       if (lane == 0) {
-        if (gbits) peer_max(peer_addr(cgmax + (st & 1) * own + os, oc), gbits);
+        if constexpr (kTeam) {
+          if (gbits) atomicMax(xgmax + (st & 1) * n_cells + c, gbits);
+        } else {
+          if (gbits) peer_max(peer_addr(cgmax + (st & 1) * own + os, oc), gbits);
+        }
         if (M) atomicAdd(ncand + c, (unsigned long long)M);
         if (nac) atomicAdd(nacc + c, (unsigned long long)nac);
         q = atomicAdd(&next_group, 1);
@@ -325,7 +408,7 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
       if (tid == 0) n_hits = 0;
       if (c1 < len) __syncthreads();
     }
-    int* row = rows + w * n_cells;
+    unsigned short* row = rows + w * n_cells;
     for (int c = lane; c < n_cells; c += 32) row[c] = 0;
     __syncwarp();
 
@@ -342,7 +425,7 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
       __syncwarp();
       if (act) {
         const int before = __popc(peers & lt);
-        if (before == 0) row[cell] = first + __popc(peers);
+        if (before == 0) row[cell] = (unsigned short)(first + __popc(peers));
         key[i] = ((unsigned)cell << 16) | (unsigned)(first + before);
       }
       __syncwarp();
@@ -354,12 +437,18 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
       for (int v = 0; v < kWarps; ++v) t[v] = rows[v * n_cells + c];
 #pragma unroll
       for (int v = 0; v < kWarps; ++v) {
-        rows[v * n_cells + c] = run;
+        rows[v * n_cells + c] = (unsigned short)run;
         run += t[v];
       }
-      for (int v = 0; v < CL; ++v) peer_store(peer_addr(tot + rank * n_cells + c, v), run);
+      if constexpr (kTeam) {
+        xrow[(size_t)rank * n_cells + c] = run;
+        if (run) atomicAdd(xblk + ((size_t)(st & 1) * n_blocks + my_block) * n_cells + c, run);
+      } else {
+        for (int v = 0; v < CL; ++v) peer_store(peer_addr(tot + rank * n_cells + c, v), run);
+      }
     }
-    cluster_barrier();
+    wait_all();
+    if (lost) break;
 
     // B. New offsets, the cells' results, and the sort.
     int carry = lo;
@@ -367,7 +456,24 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
       const int c = cb + tid;
       int total = 0, pre = 0;
       uint32_t gm = 0u;
-      if (c < n_cells) {
+      if constexpr (kTeam) {
+        if (c < n_cells) {
+          gm = __ldcg(xgmax + (st & 1) * n_cells + c);
+          const int* blk = xblk + (size_t)(st & 1) * n_blocks * n_cells + c;
+          const int* row0 = xrow + (size_t)my_block * kTeamBlock * n_cells + c;
+          int x[kTeamBlock], y[kTeamBlock];  // all loads in flight at once
+#pragma unroll
+          for (int v = 0; v < kTeamBlock; ++v) {
+            x[v] = v < n_blocks ? __ldcg(blk + (size_t)v * n_cells) : 0;
+            y[v] = my_block * kTeamBlock + v < rank ? __ldcg(row0 + (size_t)v * n_cells) : 0;
+          }
+#pragma unroll
+          for (int v = 0; v < kTeamBlock; ++v) {
+            total += x[v];
+            pre += (v < my_block ? x[v] : 0) + y[v];
+          }
+        }
+      } else if (c < n_cells) {
         const int oc = c / own;  // the owner's largest relative speed, used below
         gm = peer_load(peer_addr(cgmax + (st & 1) * own + (c - oc * own), oc));
 #pragma unroll 4
@@ -405,19 +511,30 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
     // (taken from the last threads down: the first ones are busy with the cells above)
     for (int i = kThreads - 1 - tid; i < own_n * kNMom; i += kThreads) {
       const int oc = i / kNMom, k = i - oc * kNMom, c = own0 + oc;
-      if (k == 0) cgmax[((st & 1) ^ 1) * own + oc] = 0u;
+      if (k == 0) {
+        if constexpr (kTeam)
+          xgmax[((st & 1) ^ 1) * n_cells + c] = 0u;
+        else
+          cgmax[((st & 1) ^ 1) * own + oc] = 0u;
+      }
       if (sample) {
         const int nc = off[c + 1] - off[c];
         if (k == 0) {
           csum[i] += (double)nc;
         } else {
+          unsigned long long* fix =
+              kTeam ? xfix + (size_t)c * 12 + (k - 1) : cfix + oc * 12 + (k - 1);
+          const unsigned long long q = kTeam ? __ldcg(fix) : *fix;
           const double grid =
               __longlong_as_double((long long)(1023 - grid_exponent(nc > 0 ? nc : 1)) << 52);
-          csum[i] += 0.5 * grid * (double)(long long)cfix[oc * 12 + k - 1];
-          cfix[oc * 12 + k - 1] = 0ull;
+          csum[i] += 0.5 * grid * (double)(long long)q;
+          *fix = 0ull;
         }
       }
     }
+    if constexpr (kTeam)  // the block sums of the next step
+      for (int i = rank * kThreads + tid; i < n_blocks * n_cells; i += CL * kThreads)
+        xblk[(size_t)((st & 1) ^ 1) * n_blocks * n_cells + i] = 0;
     __syncthreads();
     for (int b = pb; b < pe; b += 32) {
       const int i = b + lane;
@@ -431,7 +548,7 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
           bad_sort = true;
       }
     }
-    cluster_barrier();
+    wait_all();
     int* t0 = off;
     off = off_next;
     off_next = t0;
@@ -442,7 +559,7 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
 
   for (int i = tid; i < own_n * kNMom; i += kThreads) acc[(size_t)own0 * kNMom + i] = csum[i];
   // The run's state after the last step, where the next launch of either kind looks for it.
-  if (rank == 0) {
+  if (rank == 0 && !lost) {
     int* g = ((RL.parity_off ^ RL.n_steps) & 1 ? off1 : off0) + a.off_base;
     float* s = ((RL.parity_smax ^ RL.n_steps) & 1 ? smax1 : smax0) + a.cell_base;
     for (int c = tid; c <= n_cells; c += kThreads) g[c] = off[c];
@@ -453,62 +570,85 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
   if (inflow_fail) atomicOr(err, kErrInflow);
   if (mom_range) atomicOr(err, kErrMoments);
   if (bad_sort) atomicOr(err, kErrSort);
+  if (lost && tid == 0) atomicOr(err, kErrTeam);
 }
 
 namespace {
 
-const void* resident_kernel(bool batch, bool f64) {
+const void* resident_kernel(bool batch, bool f64, bool team) {
+  if (team)
+    return f64 ? (const void*)k_resident<false, kResidentWarps, true, true>
+               : (const void*)k_resident<false, kResidentWarps, false, true>;
   if (batch)
-    return f64 ? (const void*)k_resident<true, kResidentWarpsBatch, true>
-               : (const void*)k_resident<true, kResidentWarpsBatch, false>;
-  return f64 ? (const void*)k_resident<false, kResidentWarps, true>
-             : (const void*)k_resident<false, kResidentWarps, false>;
+    return f64 ? (const void*)k_resident<true, kResidentWarpsBatch, true, false>
+               : (const void*)k_resident<true, kResidentWarpsBatch, false, false>;
+  return f64 ? (const void*)k_resident<false, kResidentWarps, true, false>
+             : (const void*)k_resident<false, kResidentWarps, false, false>;
 }
+
+// The launch of `ctas` CTAs in clusters of `cl`, or as a cooperative grid (team).
+struct ResidentConfig {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at{};
+  ResidentConfig(int ctas, int cl, int warps, size_t smem, bool team, cudaStream_t st) {
+    cfg.gridDim = dim3((unsigned)ctas);
+    cfg.blockDim = dim3((unsigned)(warps * 32));
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    if (team) {
+      at.id = cudaLaunchAttributeCooperative;
+      at.val.cooperative = 1;
+    } else {
+      at.id = cudaLaunchAttributeClusterDimension;
+      at.val.clusterDim.x = (unsigned)cl;
+      at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    }
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+  }
+};
 
 }  // namespace
 
-cudaError_t resident_clusters(int cl, size_t smem, bool batch, bool f64, int* clusters) {
-  const void* f = resident_kernel(batch, f64);
-  *clusters = 0;
+cudaError_t resident_fits(const ResidentLaunch& L, size_t smem, bool f64, bool* fits) {
+  const bool batch = L.n_inst > 1;
+  const void* f = resident_kernel(batch, f64, L.team != 0);
+  *fits = false;
   cudaError_t e =
       cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResidentSmemMax);
-  if (e == cudaSuccess)
+  if (e == cudaSuccess && !L.team)
     e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(cl);
-  cfg.blockDim = dim3(resident_warps(batch) * 32);
-  cfg.dynamicSmemBytes = smem;
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = cl;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
-  return cudaOccupancyMaxActiveClusters(clusters, f, &cfg);
+  int n = 0;
+  if (L.team) {  // every CTA of the grid resident at once, one per SM
+    int dev = 0, sms = 0, coop = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+        (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
+        (e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev)) != cudaSuccess)
+      return e;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f, resident_warps(false) * 32, smem);
+    *fits = e == cudaSuccess && coop && n >= 1 && L.cl <= sms;
+    return e;
+  }
+  ResidentConfig c(L.cl, L.cl, resident_warps(batch), smem, false, nullptr);
+  e = cudaOccupancyMaxActiveClusters(&n, f, &c.cfg);
+  *fits = e == cudaSuccess && n >= 1;
+  return e;
 }
 
 cudaError_t launch_resident(float4* P0, float4* P1, int* off0, int* off1, float* smax0,
                             float* smax1, unsigned long long* ncand, unsigned long long* nacc,
-                            double* acc, const InstParams& one, const ResidentLaunch& L,
-                            bool f64, int* err, cudaStream_t st) {
-  const ResidentSmem S =
-      resident_smem_layout(L.max_cells, L.range_cap, L.list_cap, L.own_cap, L.cl,
-                           resident_warps(L.n_inst > 1));
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)(L.cl * L.n_inst));
-  cfg.blockDim = dim3(resident_warps(L.n_inst > 1) * 32);
-  cfg.dynamicSmemBytes = S.total;
-  cfg.stream = st;
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = L.cl;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
-  void* args[] = {&P0,   &P1,  &off0, &off1, &smax0, &smax1, &ncand, &nacc, &acc,
-                  const_cast<InstParams*>(&one), const_cast<ResidentLaunch*>(&L), &err};
-  const cudaError_t e = cudaLaunchKernelExC(&cfg, resident_kernel(L.n_inst > 1, f64), args);
+                            double* acc, int* exchange, unsigned* barrier, const InstParams& one,
+                            const ResidentLaunch& L, bool f64, int* err, cudaStream_t st) {
+  const int warps = resident_warps(L.n_inst > 1);
+  const ResidentSmem S = resident_smem_layout(L.max_cells, L.range_cap, L.list_cap, L.own_cap,
+                                              L.team ? 0 : L.cl, warps);
+  ResidentConfig c(L.cl * L.n_inst, L.cl, warps, S.total, L.team != 0, st);
+  void* args[] = {&P0,   &P1,  &off0,     &off1,    &smax0, &smax1, &ncand,
+                  &nacc, &acc, &exchange, &barrier, const_cast<InstParams*>(&one),
+                  const_cast<ResidentLaunch*>(&L),  &err};
+  const cudaError_t e =
+      cudaLaunchKernelExC(&c.cfg, resident_kernel(L.n_inst > 1, f64, L.team != 0), args);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 

@@ -1,6 +1,7 @@
-"""Cluster-resident steps (csrc/dsmc_resident.cu) against the span passes, bit for bit.
+"""Resident steps (csrc/dsmc_resident.cu) against the span passes, bit for bit.
 
-A handle with default options runs small problems cluster-resident; with profile=1 the
+A handle with default options runs small problems resident, on a cluster of CTAs up to 40,000
+particles and on a team of them over the whole device above; with profile=1 the
 same handle takes the span passes (whose parity with the oracle the other tests pin).  Both
 must give the same records, offsets, maxima, counters and moment sums at the sizes where the
 resident kernel's tables and partitions can go wrong.
@@ -40,6 +41,11 @@ CASES = [
     dict(Kn=0.1, n_cells=700, ppc=20, omega=0.5, group_size=8),  # more cells than threads
     dict(Kn=0.3, n_cells=300, ppc=100, omega=0.5, collisions=False),
     dict(Kn=0.3, n_cells=60, ppc=300, omega=0.81, group_size=512),
+    dict(Kn=0.3, n_cells=400, ppc=103, omega=0.81),             # the smallest team runs
+    dict(Kn=0.3, n_cells=1, ppc=50000, omega=0.5),              # one cell over a team
+    dict(Kn=5.0, n_cells=37, ppc=2000, omega=1.0, accum=1),     # fewer cells than CTAs
+    dict(Kn=0.1, n_cells=1200, ppc=50, omega=0.5, group_size=64),  # more cells than threads
+    dict(Kn=0.3, n_cells=397, ppc=2531, omega=0.81),            # a full device
 ]
 
 
@@ -56,17 +62,18 @@ def test_resident_steps_match_the_span_passes(case):
     _assert_same(*got)
 
 
-def test_resident_steps_of_an_uneven_state_and_open_boundary():
+@pytest.mark.parametrize("ppc", [150, 1500])
+def test_resident_steps_of_an_uneven_state_and_open_boundary(ppc):
     """A loaded state that fills only part of the channel (empty cells, dense cells), then
     an open upper boundary; switching between the two step kinds on the way."""
     from paper_2311_14140_gb300 import Dsmc
     rng = np.random.default_rng(3)
-    n = 60 * 150
+    n = 60 * ppc
     y = (0.35 * rng.random(n) ** 2 + 0.5).astype(np.float32)
     v = [rng.normal(0, np.sqrt(0.5), n).astype(np.float32) for _ in range(3)]
     got = []
     for profile in (False, True):
-        d = Dsmc(0.3, 60, 150, omega=0.81, body_force=1e-2, seed=9, profile=profile)
+        d = Dsmc(0.3, 60, ppc, omega=0.81, body_force=1e-2, seed=9, profile=profile)
         d.load_state(y, *v, step=3)
         d.step(4)
         d.set_open_top(0.01, -0.02)
