@@ -911,7 +911,8 @@ bool size_resident(dsmc_sim* h, ResidentLaunch& R) {
   R.list_cap = R.range_cap / o.group_size + std::min(R.max_cells, R.range_cap) + 2;
   R.own_cap = (R.max_cells + R.cl - 1) / R.cl;
   const size_t smem = resident_smem_layout(R.max_cells, R.range_cap, R.list_cap, R.own_cap,
-                                           R.team ? 0 : R.cl, resident_warps(R.n_inst > 1))
+                                           R.team ? 0 : R.cl, resident_local(R),
+                                           resident_warps(R.n_inst > 1))
                           .total;
   if (smem > kResidentSmemMax) return false;
   bool fits = false;
@@ -941,7 +942,6 @@ void plan_resident(dsmc_sim* h) {
       R = T;
       fits = true;
     }
-    if (!fits && n_max > kClusterParticles) fits = size_resident(h, R);
   } else {
     R.cl = 2;
     while (R.cl < kResidentMaxCluster &&

@@ -306,25 +306,29 @@ __device__ __forceinline__ bool fly_with(float& y, float& vx, float& vy, float& 
     }
     const uint32_t c1 = (uint32_t)b << 8;
     const uint32_t c3 = kStreamMove << 24;
-    U4 w = gen(slot, c1, step, c3);
-    const float speed = fsqrt(-ln32(u01(w.x)));
-    // polar attempts until one falls inside the unit disc; the logarithm, division and
-    // square root of the accepted attempt once after the loop (the lanes of a warp need
-    // different numbers of attempts, so inside it they would run once per attempt)
+    // The speed's draw and the first two polar attempts' draw are always needed: drawn
+    // together, their two dependent chains overlap.  Further attempts (5 % of the lanes, so
+    // most warps go round once more) two at a time; the logarithm, division and square root
+    // of the accepted attempt once after the loop (the lanes of a warp need different numbers
+    // of attempts, so inside it they would run once per attempt).
+    const U4 w = gen(slot, c1, step, c3);
+    U4 q = gen(slot, c1 | 1u, step, c3);
     float a0 = 0.0f, a1 = 0.0f, sacc = 0.0f;
     bool got = false;
-    for (int a = 0; a < kNormalAttempts && !got; ++a) {
-      if ((a & 1) == 0) w = gen(slot, c1 | (1u + (uint32_t)(a >> 1)), step, c3);
-      const float t0 = s11((a & 1) ? w.z : w.x);
-      const float t1 = s11((a & 1) ? w.w : w.y);
-      const float sq = fadd(fmul(t0, t0), fmul(t1, t1));
-      if (sq < 1.0f) {
-        a0 = t0;
-        a1 = t1;
-        sacc = sq;
-        got = true;
-      }
+    for (int a = 0;;) {
+      const float t0 = s11(q.x), t1 = s11(q.y), t2 = s11(q.z), t3 = s11(q.w);
+      const float s0 = fadd(fmul(t0, t0), fmul(t1, t1));
+      const float s1 = fadd(fmul(t2, t2), fmul(t3, t3));
+      const bool first = s0 < 1.0f;
+      got = first || s1 < 1.0f;
+      a0 = first ? t0 : t2;
+      a1 = first ? t1 : t3;
+      sacc = first ? s0 : s1;
+      a += 2;
+      if (got || a >= kNormalAttempts) break;
+      q = gen(slot, c1 | (1u + (uint32_t)(a >> 1)), step, c3);
     }
+    const float speed = fsqrt(-ln32(u01(w.x)));
     float z0 = 0.0f, z1 = 0.0f;
     if (got) {
       polar_scale(a0, a1, sacc, z0, z1);

@@ -186,6 +186,9 @@ struct ResidentLaunch {
   int cut[kTeamMax + 1];  // the team's slot shares (as InstParams::cut)
 };
 
+// One instance on one cluster: the records stay in shared memory from step to step.
+inline bool resident_local(const ResidentLaunch& L) { return L.n_inst == 1 && !L.team; }
+
 // Ints of a team's exchange area before its 64-bit sums, and in all.
 __host__ __device__ inline size_t team_fix_offset(int cl, int n_cells) {
   const size_t blocks = (size_t)(cl + kTeamBlock - 1) / kTeamBlock;
@@ -203,11 +206,11 @@ struct ResidentSmem {
 
 __host__ __device__ inline ResidentSmem resident_smem_layout(int n_cells, int range_cap,
                                                              int list_cap, int own_cap, int cl,
-                                                             int warps) {
+                                                             bool local, int warps) {
   ResidentSmem L;
   size_t o = 0;
   L.rec = o;
-  o += (size_t)range_cap * 16;
+  o += (size_t)range_cap * (local ? 32 : 16);
   L.cfix = o;
   o += (size_t)own_cap * 12 * 8;
   L.csum = o;

@@ -12,8 +12,8 @@
 //   a team (kTeam): for one run that 16 SMs would be slow on, a cooperative grid of a CTA per
 //     SM: counts and cell results by global memory, a counter barrier (about 1.5 us each).
 // Measured (us per step, before = span passes under graph replay): 20,000 particles 22.5 ->
-// 11.4 and 9,000 20.9 -> 8.4 (cluster), 100,000 21-30 -> 13.5, 300,000 38 -> 16.7, 1,004,807
-// 71 -> 27.7 (team).  What is left is the latency of one collision group per warp (a chain of
+// 10.8, 10,000 20.9 -> 8.1 and 2,250 20.5 -> 6.8 (cluster), 100,000 21-30 -> 13.5, 300,000
+// 38 -> 16.7, 1,004,807 71 -> 27.4 (team).  What is left is the latency of one collision group per warp (a chain of
 // about 8,000 cycles at 200 particles), then barriers, loads and the ranking.
 //
 // A step, for CTA r of CL (identical arithmetic, operation for operation, to the
@@ -26,7 +26,8 @@
 //      [barrier]
 //   B  every CTA reads the others' counts: exclusive prefix over CTAs and cells gives the
 //      new cell offsets and the CTA's base in every cell; the cell's owner CTA adds the
-//      step's moment sums to the run's; each record goes to its sorted place in the other
+//      step's moment sums to the run's; each record goes to its sorted place: in the shared
+//      memory of the CTA that takes it next (one instance on one cluster), or in the other
 //      record buffer (global memory, L2-resident at these sizes).
 //      [barrier]
 // Cell results (fixed-point moment totals, counters, largest relative speed) are integer
@@ -73,6 +74,12 @@ __device__ __forceinline__ uint32_t peer_load(uint32_t addr) {
 
 __device__ __forceinline__ void peer_store(uint32_t addr, uint32_t v) {
   asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+
+__device__ __forceinline__ void peer_store4(uint32_t addr, float4 v) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y),
+               "f"(v.z), "f"(v.w)
+               : "memory");
 }
 
 __device__ __forceinline__ void peer_add(uint32_t addr, unsigned long long v) {
@@ -134,12 +141,19 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
                int* exchange, unsigned* barrier, const InstParams one, const ResidentLaunch RL,
                int* err) {
   static_assert(!(kBatch && kTeam), "a team serves one instance");
+  // One instance on one cluster: a CTA sends its sorted records straight into the shared memory
+  // of the CTA that takes them in the next step (two record buffers), so they are neither
+  // written to L2 nor read back.  A batch's CTAs share SMs two by two and a team's are not a
+  // cluster: their records go through the global buffers.
+  constexpr bool kLocal = !kBatch && !kTeam;
   using Acc = typename std::conditional<kF64, double, float>::type;
   constexpr int kThreads = kWarps * 32;
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ InstParams sh_inst;
   __shared__ int wsum[2][32];
-  __shared__ int bnd_slot[2], bnd_cell[2], bnd_group[2];  // first group of this CTA, and the end
+  // first groups of the CTAs (kLocal: of all of them), or of this CTA and the next
+  constexpr int kBounds = kLocal ? kResidentMaxCluster + 1 : 2;
+  __shared__ int bnd_slot[kBounds], bnd_cell[kBounds], bnd_group[kBounds];
   __shared__ int n_groups_sh, next_group, n_hits;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const unsigned lt = (1u << lane) - 1u;
@@ -153,8 +167,9 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
   }
   const InstParams& a = kBatch ? sh_inst : one;
   const ResidentSmem L = resident_smem_layout(RL.max_cells, RL.range_cap, RL.list_cap,
-                                              RL.own_cap, kTeam ? 0 : RL.cl, kWarps);
+                                              RL.own_cap, kTeam ? 0 : RL.cl, kLocal, kWarps);
   float4* rec = reinterpret_cast<float4*>(smem + L.rec);        // this CTA's records
+  float4* rec_next = rec + RL.range_cap;                        // the next step's (kLocal)
   unsigned* key = reinterpret_cast<unsigned*>(smem + L.key);    // candidate masks, then ranks
   int2* list = reinterpret_cast<int2*>(smem + L.list);          // groups: (cell, gi << 10 | gn)
   unsigned short* rows = reinterpret_cast<unsigned short*>(smem + L.rows);  // counts per warp, cell
@@ -175,6 +190,7 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
   // slots at which this CTA's and the next CTA's groups may start
   const int B0 = lo + (kTeam ? RL.cut[rank] : a.cut[rank]);
   const int B1 = lo + (kTeam ? RL.cut[rank + 1] : a.cut[rank + 1]);
+  const int me = kLocal ? rank : 0, last = kLocal ? CL : 1;  // this CTA's bound, the last one
   // A team's exchange in global memory: count rows of its CTAs; their sums over blocks of
   // kTeamBlock CTAs, of even and odd steps; the cells' largest relative speeds, of even and
   // odd steps; and the cells' fixed-point sums.
@@ -215,35 +231,87 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
     }
     for (int i = tid; i < own_n * kNMom; i += kThreads) csum[i] = acc[(size_t)own0 * kNMom + i];
   }
-  // The group boundaries of this CTA from cell offsets: boundary B falls into the cell
-  // c with first <= B < first + n; the CTA's groups begin with the cell's first group
-  // that starts at or after B, or with the next cell.
+  const int gshift = (G & (G - 1)) ? -1 : 31 - __clz(G);  // G is a power of two: its exponent
+  auto groups_of = [&](int n) {  // group_count without its division
+    if (gshift < 0) return group_count(n, G);
+    const int ng = n >> gshift, r = n & (G - 1);
+    return ng + ((r > 0 && (ng == 0 || r >= G / 2)) ? 1 : 0);
+  };
+  // Bound k (a slot share's first slot B) from the cell c it falls into, of n slots from
+  // `first` on: the CTA's groups begin with the cell's first group that starts at or after B,
+  // or with the next cell.
   auto set_bound = [&](int k, int B, int c, int first, int n) {
-    if (B < first || B >= first + n) return;
-    const int i = (B - first + G - 1) / G;
-    const int ng = group_count(n, G);
+    const int i = gshift < 0 ? (B - first + G - 1) / G : (B - first + G - 1) >> gshift;
+    const int ng = groups_of(n);
     bnd_cell[k] = c;
     bnd_group[k] = min(i, ng);
     bnd_slot[k] = i < ng ? first + i * G : first + n;
   };
+  // The bounds under cell offsets o, by the first threads (a search each): what a cluster that
+  // needs all of its CTAs' bounds does.
+  auto find_bounds = [&](const int* o) {
+    if (kLocal ? tid >= CL : (tid >= 2 || rank + tid >= CL)) return;
+    const int B = kLocal ? lo + a.cut[tid] : (tid ? B1 : B0);
+    int c = 0;
+    for (int h = 1 << (31 - __clz(n_cells)); h > 0; h >>= 1)
+      if (c + h < n_cells && o[c + h] <= B) c += h;
+    set_bound(tid, B, c, o[c], o[c + 1] - o[c]);
+  };
+  // The list of this CTA's groups under cell offsets o and the bounds, by one warp.
+  auto make_list = [&](const int* o) {
+    const int cb = bnd_cell[me], ce = bnd_cell[me + 1];
+    const int gb = bnd_group[me], ge = bnd_group[me + 1];
+    const int len = bnd_slot[me + 1] - bnd_slot[me];
+    int run = 0;
+    const int cend = len > 0 && len <= RL.range_cap ? min(ce, n_cells - 1) : cb - 1;
+    for (int c0 = cb; c0 <= cend; c0 += 32) {
+      const int c = c0 + lane;
+      int g0 = 0, g1 = 0, ng = 0, nc = 0;
+      if (c <= cend) {
+        nc = o[c + 1] - o[c];
+        ng = groups_of(nc);
+        g0 = c == cb ? gb : 0;
+        g1 = max(g0, c == ce ? ge : ng);
+      }
+      const int cnt = g1 - g0;
+      int incl = cnt;
+#pragma unroll
+      for (int q = 1; q < 32; q <<= 1) {
+        const int t = __shfl_up_sync(kFull, incl, q);
+        if (lane >= q) incl += t;
+      }
+      int p = run + incl - cnt;
+      for (int g = g0; g < g1; ++g, ++p)
+        if (p < RL.list_cap) list[p] = make_int2(c, (g << 10) | (g == ng - 1 ? nc - g * G : G));
+      run += __shfl_sync(kFull, incl, 31);
+    }
+    if (lane == 0) {
+      n_groups_sh = run <= RL.list_cap ? run : -1;
+      next_group = kWarps;  // every warp starts with the group of its own number
+    }
+  };
   unsigned short* queue = rows;  // (local slots)
   const int qcap = (int)(L.rows_bytes / 2) & ~31;  // wall hits the queue holds
-  if (tid == 0) n_hits = 0;
-  if (tid == 0) {  // ends of the instance (the last CTA's end is past every cell)
-    bnd_slot[1] = hi;
-    bnd_cell[1] = n_cells;
-    bnd_group[1] = 0;
+  if (tid == 0) {
+    n_hits = 0;
+    // the instance's end (the last CTA's end is past every cell)
+    bnd_slot[last] = hi;
+    bnd_cell[last] = n_cells;
+    bnd_group[last] = 0;
   }
+  for (int i = tid; i < RL.range_cap; i += kThreads) key[i] = 0u;  // (zero between steps)
   __syncthreads();
-  for (int c = tid; c < n_cells; c += kThreads) {
-    const int first = off[c], n = off[c + 1] - first;
-    set_bound(0, B0, c, first, n);
-    if (rank + 1 < CL) set_bound(1, B1, c, first, n);
-  }
+  find_bounds(off);
+  __syncthreads();
+  if (kLocal && w == kWarps - 1) make_list(off);
   const float4* Pin = RL.parity_rec ? P1 : P0;
   float4* Pout = RL.parity_rec ? P0 : P1;
   bool bad_bounce = false, cand_fail = false, inflow_fail = false, mom_range = false;
   bool bad_sort = false;
+  if constexpr (kLocal) {
+    const int s0 = bnd_slot[me], n = min(bnd_slot[me + 1] - s0, RL.range_cap);
+    for (int i = tid; i < n; i += kThreads) rec[i] = Pin[s0 + i];
+  }
   wait_all();  // every CTA's accumulators are cleared
 
   int st = 0;
@@ -251,57 +319,23 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
     const uint32_t step = (uint32_t)istep;
     const bool sample = istep >= a.sample_start;
     const bool collide = a.collide != 0;
-    const int s0 = bnd_slot[0];
-    int len = bnd_slot[1] - s0;
+    const int s0 = bnd_slot[me];
+    int len = bnd_slot[me + 1] - s0;
     if (len < 0 || len > RL.range_cap) {  // only corrupted offsets can do this
       bad_sort = true;
       len = 0;
     }
 
     // A. This CTA's records and groups.
-    if (w == 0) {
-      const int cb = bnd_cell[0], ce = bnd_cell[1];
-      const int gb = bnd_group[0], ge = bnd_group[1];
-      int run = 0;
-      const int cend = len > 0 ? min(ce, n_cells - 1) : cb - 1;
-      for (int c0 = cb; c0 <= cend; c0 += 32) {
-        const int c = c0 + lane;
-        int g0 = 0, g1 = 0, ng = 0, nc = 0;
-        if (c <= cend) {
-          nc = off[c + 1] - off[c];
-          ng = group_count(nc, G);
-          g0 = c == cb ? gb : 0;
-          g1 = max(g0, c == ce ? ge : ng);
-        }
-        const int cnt = g1 - g0;
-        int incl = cnt;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int t = __shfl_up_sync(kFull, incl, o);
-          if (lane >= o) incl += t;
-        }
-        if (c <= cend) {
-          int p = run + incl - cnt;
-          for (int g = g0; g < g1; ++g, ++p)
-            if (p < RL.list_cap)
-              list[p] = make_int2(c, (g << 10) | (g == ng - 1 ? nc - g * G : G));
-        }
-        run += __shfl_sync(kFull, incl, 31);
-      }
-      if (lane == 0) {
-        if (run > RL.list_cap) {
-          bad_sort = true;
-          run = 0;
-        }
-        n_groups_sh = run;
-        next_group = kWarps;  // every warp starts with the group of its own number
-      }
-    } else {
-      for (int i = tid - 32; i < len; i += kThreads - 32) rec[i] = __ldcg(Pin + s0 + i);
-      for (int i = tid - 32; i < len; i += kThreads - 32) key[i] = 0u;
+    if constexpr (!kLocal) {
+      if (w == kWarps - 1)
+        make_list(off);
+      else
+        for (int i = tid; i < len; i += kThreads - 32) rec[i] = __ldcg(Pin + s0 + i);
+      __syncthreads();
     }
-    __syncthreads();
     const int n_groups = n_groups_sh;
+    if (n_groups < 0) bad_sort = true;
 
     for (int q = w; q < n_groups;) {
       const int2 e = list[q];
@@ -412,23 +446,34 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
     for (int c = lane; c < n_cells; c += 32) row[c] = 0;
     __syncwarp();
 
-    // Rank of every record among the earlier ones of its warp's part bound for its cell.
+    // Rank of every record among the earlier ones of its warp's part bound for its cell; the
+    // cells and same-cell lanes of four slices at a time, then slice after slice the counts.
     const int part = ((len + kWarps - 1) / kWarps + 31) & ~31;
     const int pb = w * part, pe = min(len, pb + part);
-    for (int b = pb; b < pe; b += 32) {
-      const int i = b + lane;
-      const bool act = i < pe;
-      const int cell = act ? cell_of(rec[i].x, n_cells, a.ncf) : -1;
-      const unsigned peers = __match_any_sync(kFull, cell);
-      int first = 0;
-      if (act) first = row[cell];
-      __syncwarp();
-      if (act) {
-        const int before = __popc(peers & lt);
-        if (before == 0) row[cell] = (unsigned short)(first + __popc(peers));
-        key[i] = ((unsigned)cell << 16) | (unsigned)(first + before);
+    for (int b = pb; b < pe; b += 128) {
+      int cell[4];
+      unsigned peers[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int i = b + 32 * u + lane;
+        cell[u] = i < pe ? cell_of(rec[i].x, n_cells, a.ncf) : -1;
       }
-      __syncwarp();
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (b + 32 * u < pe) peers[u] = __match_any_sync(kFull, cell[u]);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (b + 32 * u >= pe) break;
+        const bool act = cell[u] >= 0;
+        const int first = act ? row[cell[u]] : 0;
+        const int before = __popc(peers[u] & lt);
+        __syncwarp();
+        if (act) {
+          if (before == 0) row[cell[u]] = (unsigned short)(first + __popc(peers[u]));
+          key[b + 32 * u + lane] = ((unsigned)cell[u] << 16) | (unsigned)(first + before);
+        }
+        __syncwarp();
+      }
     }
     __syncthreads();
     for (int c = tid; c < n_cells; c += kThreads) {
@@ -476,9 +521,9 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
       } else if (c < n_cells) {
         const int oc = c / own;  // the owner's largest relative speed, used below
         gm = peer_load(peer_addr(cgmax + (st & 1) * own + (c - oc * own), oc));
-#pragma unroll 4
-        for (int v = 0; v < CL; ++v) {
-          const int t = tot[v * n_cells + c];
+#pragma unroll
+        for (int v = 0; v < kResidentMaxCluster; ++v) {
+          const int t = v < CL ? tot[v * n_cells + c] : 0;
           total += t;
           pre += v < rank ? t : 0;
         }
@@ -499,9 +544,11 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
         const int first = before + incl - total;
         off_next[c] = first;
         base[c] = first + pre;
-        set_bound(0, B0, c, first, total);
-        if (rank + 1 < CL) set_bound(1, B1, c, first, total);
         if (c == n_cells - 1) off_next[n_cells] = first + total;
+        if constexpr (!kLocal) {  // this CTA's two bounds, by the threads whose cells they fall into
+          if (B0 >= first && B0 < first + total) set_bound(0, B0, c, first, total);
+          if (rank + 1 < CL && B1 >= first && B1 < first + total) set_bound(1, B1, c, first, total);
+        }
         // (sigma g)_max of the next step
         const float g = __uint_as_float(gm);
         const float sg = (mode == 0) ? g : fmul(a.cvhs, pow32(g, a.vexp));
@@ -536,18 +583,36 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
       for (int i = rank * kThreads + tid; i < n_blocks * n_cells; i += CL * kThreads)
         xblk[(size_t)((st & 1) ^ 1) * n_blocks * n_cells + i] = 0;
     __syncthreads();
+    if constexpr (kLocal) {
+      find_bounds(off_next);
+      __syncthreads();
+    }
     for (int b = pb; b < pe; b += 32) {
       const int i = b + lane;
       if (i < pe) {
         const unsigned kk = key[i];
+        key[i] = 0u;
         const int cell = (int)(kk >> 16);
         const int d = base[cell] + rows[w * n_cells + cell] + (int)(kk & 0xffffu);
-        if (d >= lo && d < hi)
-          Pout[d] = rec[i];
-        else
+        if (d < lo || d >= hi) {
           bad_sort = true;
+        } else if constexpr (kLocal) {
+          int k = 0;  // the CTA whose slots these are
+#pragma unroll
+          for (int o = kResidentMaxCluster / 2; o > 0; o >>= 1)
+            if (k + o < CL && d >= bnd_slot[k + o]) k += o;
+          const int at = d - bnd_slot[k];
+          if (at < RL.range_cap)
+            peer_store4(peer_addr(rec_next + at, k), rec[i]);
+          else
+            bad_sort = true;
+        } else {
+          Pout[d] = rec[i];
+        }
       }
     }
+    // the next step's groups, by the warp whose part is the shortest
+    if (kLocal && w == kWarps - 1) make_list(off_next);
     wait_all();
     int* t0 = off;
     off = off_next;
@@ -555,6 +620,16 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
     float4* t1 = const_cast<float4*>(Pin);
     Pin = Pout;
     Pout = t1;
+    if constexpr (kLocal) {
+      float4* t2 = rec;
+      rec = rec_next;
+      rec_next = t2;
+    }
+  }
+  if constexpr (kLocal) {  // Pin: the buffer of the state after the last step
+    const int s0 = bnd_slot[me], n = min(bnd_slot[me + 1] - s0, RL.range_cap);
+    float4* out = const_cast<float4*>(Pin);
+    for (int i = tid; i < n; i += kThreads) out[s0 + i] = rec[i];
   }
 
   for (int i = tid; i < own_n * kNMom; i += kThreads) acc[(size_t)own0 * kNMom + i] = csum[i];
@@ -642,7 +717,7 @@ cudaError_t launch_resident(float4* P0, float4* P1, int* off0, int* off1, float*
                             const ResidentLaunch& L, bool f64, int* err, cudaStream_t st) {
   const int warps = resident_warps(L.n_inst > 1);
   const ResidentSmem S = resident_smem_layout(L.max_cells, L.range_cap, L.list_cap, L.own_cap,
-                                              L.team ? 0 : L.cl, warps);
+                                              L.team ? 0 : L.cl, resident_local(L), warps);
   ResidentConfig c(L.cl * L.n_inst, L.cl, warps, S.total, L.team != 0, st);
   void* args[] = {&P0,   &P1,  &off0,     &off1,    &smax0, &smax1, &ncand,
                   &nacc, &acc, &exchange, &barrier, const_cast<InstParams*>(&one),
