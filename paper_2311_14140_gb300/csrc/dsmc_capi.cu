@@ -453,7 +453,8 @@ dsmc_status collect_times(dsmc_sim* h) {
 // The step passes must fit one CTA's shared memory with this partition, group size and
 // CTA shape.
 bool step_fits(int max_cells, int max_cps, int G, int warps = kAWarps, int rows = 1) {
-  return step_smem_layout(max_cells, max_cps, G + G / 2 - 1, warps, rows).total <= kStepSmemMax;
+  return step_smem_layout(max_cells, max_cps, G + G / 2 - 1, warps, rows, false).total <=
+         kStepSmemMax;
 }
 
 // The largest cells-per-span any active instance (and `extra`, if given) would use

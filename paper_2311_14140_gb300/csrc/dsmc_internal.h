@@ -114,17 +114,20 @@ struct InstParams {
   int cut[17];
 };
 
+constexpr int kWallQueue = 64;  // a group's slice of hits on top of at most 31 waiting ones
+
 // Dynamic shared memory of one collide/move CTA (byte offsets).
 struct StepSmem {
   size_t hist, cell_acc, cell_cand, cell_accn, cell_gmax, cell_groups, cell_start, cell_smax,
       warps, per_warp, total;
-  size_t w_rec, w_own, w_bar;  // offsets inside one warp's area
+  size_t w_rec, w_own, w_bar, w_wall;  // offsets inside one warp's area
 };
 
 __host__ __device__ inline size_t step_align(size_t o, size_t a) { return (o + a - 1) / a * a; }
 
 __host__ __device__ inline StepSmem step_smem_layout(int n_cells, int cps, int cap,
-                                                     int warps = kAWarps, int rows = 1) {
+                                                     int warps, int rows,
+                                                     bool wall_queue) {
   StepSmem L;
   size_t o = 0;
   L.hist = o;
@@ -152,6 +155,8 @@ __host__ __device__ inline StepSmem step_smem_layout(int n_cells, int cps, int c
   w = step_align(w + (size_t)cap * 4, 8);
   L.w_bar = w;
   w += 8;
+  L.w_wall = w;  // slots of wall hits waiting for their flight
+  if (wall_queue) w += kWallQueue * 4;
   L.per_warp = step_align(w, 128);
   L.warps = o;
   o += (size_t)warps * L.per_warp;

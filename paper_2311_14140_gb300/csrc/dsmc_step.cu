@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(kWarps * 32, (collide_ctas_per_sm<kBatch, kWar
   const int cap = a.cap;
   const int G = a.G;
   const int R = SL.rows;
-  const StepSmem L = step_smem_layout(n_cells, cps, cap, kWarps, R);
+  const StepSmem L = step_smem_layout(n_cells, cps, cap, kWarps, R, kBatch);
   using Acc = typename std::conditional<kF64, double, float>::type;
   int* h = reinterpret_cast<int*>(smem + L.hist);  // the span's rows x n_cells counts
   // per local cell: fixed-point moment sums (slot 0 unused), in a cell's grid
@@ -267,6 +267,23 @@ __global__ void __launch_bounds__(kWarps * 32, (collide_ctas_per_sm<kBatch, kWar
       bulk_load(rec, P + gs_, (uint32_t)gn_ * 16u, bar);
     }
   };
+  // The batched kernel's wall hits wait from group to group in a per-warp queue, so that (but
+  // for the span's last ones) every flight has 32 particles: its groups are small (a cell of
+  // 50 to 400 particles, a fifth of them hits on average) and flights are most of its
+  // instructions.  A waiting particle's record is in its slot in global memory (staging the
+  // records in shared memory costs the 8-warp CTA one of its three places on an SM).
+  int* wall_slot = reinterpret_cast<int*>(wmem + L.w_wall);
+  int n_wall = 0;
+  auto fly_queued = [&](int at) {
+    const int p = wall_slot[at];
+    const float4 r = P[p];
+    float yy = r.x, xx = r.y, uy = r.z, zz = r.w;
+    if (!fly(yy, xx, uy, zz, a.dt, a.F, a.keys, step, (uint32_t)(p - a.part_base), a.open_top,
+             a.u_top, a.p_top, inflow_fail))
+      bad_bounce = true;
+    P[p] = make_float4(yy, xx, uy, zz);
+    count_cell(p, cell_of(yy, n_cells, a.ncf));
+  };
   int q_next = 0;
   if (lane == 0) q_next = atomicAdd(next_group, 1);
   q_next = __shfl_sync(kFull, q_next, 0);
@@ -324,45 +341,70 @@ __global__ void __launch_bounds__(kWarps * 32, (collide_ctas_per_sm<kBatch, kWar
     __syncwarp();
 
     // 4. Moments after the collisions, free flight, store, count the new cell.
-    //    A particle whose flight reaches a wall is queued and flown afterwards, all such
-    //    particles of the group together (the free flight is exactly the first leg of
-    //    the full flight, so the result is the same).
-    int n_wall = 0;
-#pragma unroll kMoveUnroll
-    for (int b = 0; b < gn; b += 32) {
-      const int i = b + lane;
-      bool hits = false;
-      if (i < gn) {
-        const float4 r = rec[i];
-        if (sample) m.add(r.y, r.z, r.w);
-        const float ynew = fadd(r.x, fmul(r.z, a.dt));
-        hits = (ynew < 0.0f) || (ynew > 1.0f);
-        if (!hits) {
+    //    A particle whose flight reaches a wall is queued and flown afterwards, 32 such
+    //    particles at a time (the free flight is exactly the first leg of the full flight, so
+    //    the result is the same).
+    if constexpr (kBatch) {
+      for (int b = 0; b < gn; b += 32) {
+        const int i = b + lane;
+        bool hits = false;
+        if (i < gn) {
+          const float4 r = rec[i];
+          if (sample) m.add(r.y, r.z, r.w);
+          const float ynew = fadd(r.x, fmul(r.z, a.dt));
+          hits = (ynew < 0.0f) || (ynew > 1.0f);
           const float xx = fadd(r.y, fmul(a.F, a.dt));
-          P[gs + i] = make_float4(ynew, xx, r.z, r.w);
-          count_cell(gs + i, cell_of(ynew, n_cells, a.ncf));
+          P[gs + i] = make_float4(hits ? r.x : ynew, hits ? r.y : xx, r.z, r.w);
+          if (!hits) count_cell(gs + i, cell_of(ynew, n_cells, a.ncf));
+        }
+        const unsigned q = __ballot_sync(kFull, hits);
+        if (hits) wall_slot[n_wall + __popc(q & lt)] = gs + i;
+        n_wall += __popc(q);
+        if (n_wall >= 32) {
+          n_wall -= 32;
+          __syncwarp();
+          fly_queued(n_wall + lane);
+          __syncwarp();
         }
       }
-      const unsigned q = __ballot_sync(kFull, hits);
-      if (hits) touch[n_wall + __popc(q & lt)] = (unsigned)i;
-      n_wall += __popc(q);
-    }
-    __syncwarp();
-    for (int b = 0; b < n_wall; b += 32) {
-      if (b + lane < n_wall) {
-        const int i = (int)touch[b + lane];
-        const int p = gs + i;
-        const float4 r = rec[i];
-        float yy = r.x, xx = r.y, uy = r.z, zz = r.w;
-        if (!fly(yy, xx, uy, zz, a.dt, a.F, a.keys, step, (uint32_t)(p - a.part_base),
-                 a.open_top, a.u_top, a.p_top, inflow_fail))
-          bad_bounce = true;
-        P[p] = make_float4(yy, xx, uy, zz);
-        count_cell(p, cell_of(yy, n_cells, a.ncf));
+    } else {
+      int n_hit = 0;
+#pragma unroll 4
+      for (int b = 0; b < gn; b += 32) {
+        const int i = b + lane;
+        bool hits = false;
+        if (i < gn) {
+          const float4 r = rec[i];
+          if (sample) m.add(r.y, r.z, r.w);
+          const float ynew = fadd(r.x, fmul(r.z, a.dt));
+          hits = (ynew < 0.0f) || (ynew > 1.0f);
+          if (!hits) {
+            const float xx = fadd(r.y, fmul(a.F, a.dt));
+            P[gs + i] = make_float4(ynew, xx, r.z, r.w);
+            count_cell(gs + i, cell_of(ynew, n_cells, a.ncf));
+          }
+        }
+        const unsigned q = __ballot_sync(kFull, hits);
+        if (hits) touch[n_hit + __popc(q & lt)] = (unsigned)i;
+        n_hit += __popc(q);
       }
+      __syncwarp();
+      for (int b = 0; b < n_hit; b += 32) {
+        if (b + lane < n_hit) {
+          const int i = (int)touch[b + lane];
+          const int p = gs + i;
+          const float4 r = rec[i];
+          float yy = r.x, xx = r.y, uy = r.z, zz = r.w;
+          if (!fly(yy, xx, uy, zz, a.dt, a.F, a.keys, step, (uint32_t)(p - a.part_base),
+                   a.open_top, a.u_top, a.p_top, inflow_fail))
+            bad_bounce = true;
+          P[p] = make_float4(yy, xx, uy, zz);
+          count_cell(p, cell_of(yy, n_cells, a.ncf));
+        }
+      }
+      __syncwarp();
+      for (int i = lane; i < n_hit; i += 32) touch[i] = 0u;
     }
-    __syncwarp();
-    for (int i = lane; i < n_wall; i += 32) touch[i] = 0u;
     // the records are read for the last time: bring in the next group's
     if (q_next < n_groups) issue_copy(gs_next, gn_next);
     if (!add_group(m, sample, gn, nc, gmax, M, laccn, cfix + (size_t)lc * kNMom, &cgmax[lc],
@@ -370,6 +412,8 @@ __global__ void __launch_bounds__(kWarps * 32, (collide_ctas_per_sm<kBatch, kWar
       mom_range = true;
     __syncwarp();
   }
+  __syncwarp();
+  if (kBatch && lane < n_wall) fly_queued(lane);
   if (bad_bounce) atomicOr(err, kErrBounces);
   if (cand_fail && lane == 0) atomicOr(err, kErrCandidates);
   if (timeout && lane == 0) atomicOr(err, kErrCopyTimeout);
@@ -978,9 +1022,15 @@ cudaError_t launch_collide_move(float4* P, const int* off, const float* smax_in,
                                 unsigned long long* nacc, double* acc, int* hist,
                                 const InstParams& one, const StepLaunch& L, int* err,
                                 cudaStream_t st) {
-  const bool small = L.warps == kAWarpsSmall;
+  const bool batch = L.n_inst > 1;
+  bool small = L.warps == kAWarpsSmall;
+  // an 8-warp CTA that fits without the batch's wall queues (as the host checked) but not with
+  // them gives way to the 4-warp one, which fits at every accepted size
+  if (!small && step_smem_layout(L.max_cells, L.max_cps, L.max_cap, kAWarps, L.rows, batch).total >
+                    kStepSmemMax)
+    small = true;
   const int warps = small ? kAWarpsSmall : kAWarps;
-  const StepSmem S = step_smem_layout(L.max_cells, L.max_cps, L.max_cap, warps, L.rows);
+  const StepSmem S = step_smem_layout(L.max_cells, L.max_cps, L.max_cap, warps, L.rows, batch);
   const dim3 block(warps * 32);
 #define DSMC_COLLIDE(B, W, D)                                                       \
   k_collide_move<B, W, D><<<L.n_spans_total, block, S.total, st>>>(               \
