@@ -275,7 +275,7 @@ DSMC_API dsmc_status dsmc_get_info(dsmc_handle h, dsmc_info* info);
  * seed, step, cells and slots.  Instances may differ in gas, Kn, wall_T, force,
  * n_cells and ppc; options (dt_factor or dt, group size, sampling start, stream) are
  * shared.  Particle slots, cells and sort matrices are concatenated in one device
- * workspace (dsmc_batch_workspace_bytes); every step is the same four launches as
+ * workspace (dsmc_batch_workspace_bytes); every step is the same launches as
  * for one run, over the spans of all instances.  The functions without `_of` act on
  * instance 0, dsmc_step and dsmc_reset_samples on all instances. */
 

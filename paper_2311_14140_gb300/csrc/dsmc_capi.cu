@@ -389,7 +389,7 @@ struct dsmc_sim {
   bool span_passes = false;  // the caller's options name a partition, or it is being tuned
   // CUDA graph of kGraphSteps consecutive steps, replayed by dsmc_step when
   // options.graph is set.  Its kernels read the global step from gstep_dev, which the
-  // last prefix kernel of each step advances.
+  // kernel that forms the cell offsets advances.
   cudaGraphExec_t graph = nullptr;
   bool graph_valid = false, capturing = false;
   int graph_parity = 0;  // buffer parities (cur, ocur, scur) the graph starts from
@@ -627,7 +627,7 @@ StepLaunch step_launch(const dsmc_sim* h, bool count_only) {
 }
 
 // The launches of one pass over the records from buffer `src` to buffer src ^ 1:
-// collide + sample + move + count (or count only), prefix over spans, cell offsets,
+// collide + sample + move + count (or count only), prefix over spans, cell offsets and
 // stable scatter.
 dsmc_status launch_pass(dsmc_sim* h, bool count_only, const StepLaunch& SL,
                         const InstParams& one, int src, int osrc) {
@@ -640,19 +640,15 @@ dsmc_status launch_pass(dsmc_sim* h, bool count_only, const StepLaunch& SL,
                                          h->hist, one, SL, h->err, s);
             }),
             count_only ? "index_count" : "collide_move");
-  if (prefix_small_fits(SL)) {  // both prefix passes in one launch (timed as the scan)
-    DSMC_CUDA(timed(h, K_SCAN, [&] { return launch_prefix_small(h->hist, off_new, one, SL, s); }),
-              "prefix");
-  } else {
-    DSMC_CUDA(timed(h, K_SCAN, [&] { return launch_scan_spans(h->hist, h->count, one, SL, s); }),
-              "scan_hist");
+  DSMC_CUDA(timed(h, K_SCAN, [&] { return launch_scan_spans(h->hist, h->count, one, SL, s); }),
+            "scan_hist");
+  if (!scatter_forms_offsets(SL))
     DSMC_CUDA(timed(h, K_OFFSETS,
                     [&] { return launch_offsets_cells(h->count, off_new, one, SL, s); }),
               "cell_offsets");
-  }
   DSMC_CUDA(timed(h, count_only ? K_INDEX_SCATTER : K_SCATTER_SPANS, [&] {
-              return launch_scatter_spans(h->P[src], h->P[src ^ 1], off_cur, off_new, h->hist,
-                                          one, SL, h->err, s);
+              return launch_scatter_spans(h->P[src], h->P[src ^ 1], off_cur, h->count, off_new,
+                                          h->hist, one, SL, h->err, s);
             }),
             count_only ? "index_scatter" : "scatter_spans");
   return DSMC_OK;

@@ -288,7 +288,7 @@ struct StepLaunch {
                          // gives each row its own warp
   long long gstep;       // global step number
   long long* gstep_dev;  // non-NULL (graph replay): read the step number here instead;
-                         // the cell-offset kernel advances it at the end of the step
+                         // the kernel that forms the cell offsets advances it
   int count_only;
   int accum;  // DSMC_ACCUM_FP32 or DSMC_ACCUM_FP64: per-lane moment sums
 };
@@ -299,18 +299,17 @@ cudaError_t launch_collide_move(float4* P, const int* off, const float* smax_in,
                                 unsigned long long* nacc, double* acc, int* hist,
                                 const InstParams& one, const StepLaunch& L, int* err,
                                 cudaStream_t st);
-cudaError_t launch_scatter_spans(const float4* P, float4* P2, const int* off_cur,
-                                 const int* off_new, const int* hist, const InstParams& one,
-                                 const StepLaunch& L, int* err, cudaStream_t st);
-cudaError_t launch_scan_spans(int* hist, int* count, const InstParams& one, const StepLaunch& L,
-                              cudaStream_t st);
+// The new cell offsets (off_new) from the cells' counts: formed by the scatter, or by
+// launch_offsets_cells before it.
+bool scatter_forms_offsets(const StepLaunch& L);
 cudaError_t launch_offsets_cells(const int* count, int* off_new, const InstParams& one,
                                  const StepLaunch& L, cudaStream_t st);
-// Both prefix passes as one launch, when prefix_small_fits(L) (one instance, few cells
-// and rows).
-bool prefix_small_fits(const StepLaunch& L);
-cudaError_t launch_prefix_small(int* hist, int* off_new, const InstParams& one,
-                                const StepLaunch& L, cudaStream_t st);
+cudaError_t launch_scatter_spans(const float4* P, float4* P2, const int* off_cur,
+                                 const int* count, int* off_new, const int* hist,
+                                 const InstParams& one, const StepLaunch& L, int* err,
+                                 cudaStream_t st);
+cudaError_t launch_scan_spans(int* hist, int* count, const InstParams& one, const StepLaunch& L,
+                              cudaStream_t st);
 cudaError_t launch_set_counter(long long* counter, long long value, cudaStream_t st);
 // Per-cell arrays of newly added instances (table `tab`, n of them): moment sums and
 // collision counters zeroed, (sigma g)_max set to smax0, and cell offsets of whole

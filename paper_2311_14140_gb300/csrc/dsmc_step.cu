@@ -31,9 +31,9 @@
 //   k_scatter_coop   the same scatter with a CTA per span (up to 1,365 cells): all its
 //                    warps rank one round of 256 (or 512) records at a time.
 //
-// Between them, k_scan_spans (or k_scan_cols for instances of few spans) and
-// k_offsets_cells (below) turn the matrix into per-span bases and the new cell offsets;
-// for a small single run k_prefix_small does both in one launch.
+// Between them, k_scan_spans (or k_scan_cols for instances of few spans) turns the matrix into
+// per-span bases and the cells' counts; the new cell offsets come from those, in the
+// CTA-per-span scatter itself or by k_offsets_cells for the other.
 #include <climits>
 #include <type_traits>
 
@@ -622,12 +622,15 @@ __global__ void __launch_bounds__(kBWarpsMax * 32)
 // that leaves room for 4 CTAs per SM.
 constexpr int kCoopWarps = 8;
 constexpr size_t kCoopSmemMax = 48 * 1024;
+constexpr int kCoopPer =  // cells per thread of the largest instance it serves (1,365)
+    ((int)(kCoopSmemMax / sizeof(int) / (kCoopWarps + 1)) + kCoopWarps * 32 - 1) /
+    (kCoopWarps * 32);
 
 template <bool kBatch, int kSlices>
 __global__ void __launch_bounds__(kCoopWarps * 32)
     k_scatter_coop(const float4* __restrict__ P, float4* __restrict__ P2,
-                   const int* __restrict__ off_cur_all, const int* __restrict__ off_new_all,
-                   const int* __restrict__ hist, const InstParams one, const StepLaunch SL,
+                   const int* __restrict__ off_cur_all, const int* __restrict__ count_all,
+                   int* __restrict__ off_new_all, const int* __restrict__ hist, const InstParams one, const StepLaunch SL,
                    int* __restrict__ err) {
   extern __shared__ int sh_coop[];
   const int lane = threadIdx.x & 31;
@@ -638,12 +641,49 @@ __global__ void __launch_bounds__(kCoopWarps * 32)
   const int n_cells = a.n_cells;
   const int span = gspan - a.span_base;
   const int* __restrict__ off_cur = off_cur_all + a.off_base;
-  const int* __restrict__ off_new = off_new_all + a.off_base;
+  const int* __restrict__ count = count_all + a.cell_base;
   int* run = sh_coop;
   int* tab = sh_coop + n_cells;  // tab[w' * n_cells + c] = (round << 8) | count
   const int* row = hist + a.hist_base + ((size_t)span * R + sub) * n_cells;
-  for (int c = threadIdx.x; c < n_cells; c += blockDim.x) run[c] = off_new[c] + row[c];
-  for (int i = threadIdx.x; i < kCoopWarps * n_cells; i += blockDim.x) tab[i] = -1;
+  {
+    // The new cell offsets (prefix of the cells' counts) on the way to the run's first places:
+    // a thread takes kCoopPer consecutive cells.  Every CTA forms them, the instance's first
+    // one writes them down for the next step.
+    __shared__ int wsum[kCoopWarps];
+    int n[kCoopPer], before[kCoopPer], incl = 0;
+    const int cb = threadIdx.x * kCoopPer;
+#pragma unroll
+    for (int k = 0; k < kCoopPer; ++k) {
+      n[k] = cb + k < n_cells ? count[cb + k] : 0;
+      before[k] = cb + k < n_cells ? row[cb + k] : 0;
+    }
+#pragma unroll
+    for (int k = 0; k < kCoopPer; ++k) incl += n[k];
+    const int mine = incl;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(kFull, incl, o);
+      if (lane >= o) incl += t;
+    }
+    if (lane == 31) wsum[w] = incl;
+    for (int i = threadIdx.x; i < kCoopWarps * n_cells; i += blockDim.x) tab[i] = -1;
+    __syncthreads();
+    int at = a.part_base + incl - mine;
+#pragma unroll
+    for (int v = 0; v < kCoopWarps; ++v) at += v < w ? wsum[v] : 0;
+    int* __restrict__ off_new = blockIdx.x == a.span_base * R ? off_new_all + a.off_base : nullptr;
+#pragma unroll
+    for (int k = 0; k < kCoopPer; ++k) {
+      if (cb + k < n_cells) {
+        run[cb + k] = at + before[k];
+        if (off_new) off_new[cb + k] = at;
+      }
+      at += n[k];
+      if (off_new && cb + k == n_cells - 1) off_new[n_cells] = at;
+    }
+    // Graph replay: the step's collide/move pass has finished reading the step number.
+    if (SL.gstep_dev != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *SL.gstep_dev += 1;
+  }
   const int c0 = span * a.cps;
   const int c1 = min(c0 + a.cps, n_cells);
   const int sb0 = off_cur[c0], sb1 = off_cur[c1];
@@ -733,22 +773,26 @@ __global__ void __launch_bounds__(kCoopWarps * 32)
 }
 
 // Per instance and cell c: row r of the sort matrix <- sum over rows r' < r (the spans
-// before), count[c] <- total.  Block (32, 32): x = cell within a chunk of 32, y = one of
-// 32 contiguous row segments; grid (cell chunks, instances).
+// before), count[c] <- total.  Block (kScanCells, kScanSegs): x = cell
+// within a chunk, y = one of the contiguous row segments; grid (cell chunks, instances).  A chunk
+// of 16 cells reads 64 bytes of a row, two sectors; chunks of 32 would leave 2,000 cells 63 CTAs
+// of twice the rows per thread (20.7 us at 2,000 rows).
+constexpr int kScanCells = 16, kScanSegs = 64;
+
 template <bool kBatch>
-__global__ void __launch_bounds__(1024)
+__global__ void __launch_bounds__(kScanCells * kScanSegs)
     k_scan_spans(int* __restrict__ hist, int* __restrict__ count_all, const InstParams one,
                  const StepLaunch SL) {
-  __shared__ int seg_tot[32][33];
+  __shared__ int seg_tot[kScanSegs][kScanCells + 1];
   const InstParams& a = kBatch ? SL.tab[blockIdx.y] : one;
   const int n_cells = a.n_cells;
-  if ((int)blockIdx.x * 32 >= n_cells) return;
+  if ((int)blockIdx.x * kScanCells >= n_cells) return;
   const int n_rows = a.n_spans * SL.rows;
   int* __restrict__ m = hist + a.hist_base;
   int* __restrict__ count = count_all + a.cell_base;
   const int tx = threadIdx.x, ty = threadIdx.y;
-  const int c = blockIdx.x * 32 + tx;
-  const int seg = (n_rows + 31) / 32;
+  const int c = blockIdx.x * kScanCells + tx;
+  const int seg = (n_rows + kScanSegs - 1) / kScanSegs;
   const int r0 = min(n_rows, ty * seg);
   const int r1 = min(n_rows, r0 + seg);
   int s = 0;
@@ -767,7 +811,7 @@ __global__ void __launch_bounds__(1024)
   __syncthreads();
   if (ty == 0) {
     int run = 0;
-    for (int k = 0; k < 32; ++k) {
+    for (int k = 0; k < kScanSegs; ++k) {
       const int v = seg_tot[k][tx];
       seg_tot[k][tx] = run;
       run += v;
@@ -834,108 +878,41 @@ __global__ void __launch_bounds__(kScanColsCells)
 }
 
 // Per instance (one CTA each): off_new[c] = first global slot of cell c,
-// off_new[n_cells] = end of the instance's slots.
+// off_new[n_cells] = end of the instance's slots.  For the scatter with a warp per span, which
+// would take 5 us to form the offsets of 2,000 cells in every warp (k_scatter_coop does so in
+// every CTA, for 0.1 us).
 template <bool kBatch>
 __global__ void __launch_bounds__(1024)
     k_offsets_cells(const int* __restrict__ count_all, int* __restrict__ off_new_all,
                     const InstParams one, const StepLaunch SL) {
-  __shared__ int part[1024];
+  __shared__ int wsum[32];
   const InstParams& a = kBatch ? SL.tab[blockIdx.x] : one;
   const int n_cells = a.n_cells;
   const int* __restrict__ count = count_all + a.cell_base;
   int* __restrict__ offset = off_new_all + a.off_base;
-  const int t = threadIdx.x;
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   const int per = (n_cells + 1023) / 1024;
   const int cb = t * per;
   const int ce = min(n_cells, cb + per);
-  int s = 0;
-  for (int c = cb; c < ce; ++c) s += count[c];
-  part[t] = s;
-  __syncthreads();
-  for (int d = 1; d < 1024; d <<= 1) {  // inclusive Hillis-Steele scan
-    const int v = t >= d ? part[t - d] : 0;
-    __syncthreads();
-    part[t] += v;
-    __syncthreads();
+  int mine = 0;
+  for (int c = cb; c < ce; ++c) mine += count[c];
+  int incl = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(kFull, incl, o);
+    if (lane >= o) incl += v;
   }
-  int run = a.part_base + (t > 0 ? part[t - 1] : 0);
+  if (lane == 31) wsum[w] = incl;
+  __syncthreads();
+  const int before = __reduce_add_sync(kFull, lane < w ? wsum[lane] : 0);
+  int run = a.part_base + before + incl - mine;
   for (int c = cb; c < ce; ++c) {
     offset[c] = run;
     run += count[c];
   }
-  if (t == 1023) offset[n_cells] = a.part_base + part[1023];
+  if (t == 1023) offset[n_cells] = run;
   // Graph replay: the step's collide/move pass has finished reading the step number.
   if (SL.gstep_dev != nullptr && blockIdx.x == 0 && t == 0) *SL.gstep_dev += 1;
-}
-
-// Both prefix passes in one launch for a single instance of at most kPrefixSmallCells
-// cells and kScanColsMaxRows sort rows (a small run, whose step is launch-bound): one
-// CTA, thread c walks cell c's column of the matrix (its exclusive prefix over the spans,
-// 8 rows of loads in flight), then the CTA scans the cells' totals into the new offsets.
-// (For a batch, a CTA per instance this way was slower than the two launches.)
-constexpr int kPrefixSmallCells = 1024;
-
-__global__ void __launch_bounds__(kPrefixSmallCells, 2)
-    k_prefix_small(int* __restrict__ hist, int* __restrict__ off_new_all, const InstParams a,
-                   const StepLaunch SL) {
-  __shared__ int wsum[kPrefixSmallCells / 32];
-  const int n_cells = a.n_cells;
-  const int c = threadIdx.x;
-  const int n_rows = a.n_spans * SL.rows;
-  int run = 0;  // cell c's particles over all rows
-  if (c < n_cells) {
-    int* __restrict__ m = hist + a.hist_base + c;  // m[r n_cells]: row r of this column
-    for (int r = 0; r < n_rows; r += 8) {
-      int v[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u)
-        if (r + u < n_rows) v[u] = m[(size_t)(r + u) * n_cells];
-#pragma unroll
-      for (int u = 0; u < 8; ++u)
-        if (r + u < n_rows) {
-          m[(size_t)(r + u) * n_cells] = run;
-          run += v[u];
-        }
-    }
-  }
-  // exclusive prefix of the totals over the cells: within each warp, then over warps
-  const int lane = c & 31, w = c >> 5;
-  int incl = run;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int t = __shfl_up_sync(kFull, incl, o);
-    if (lane >= o) incl += t;
-  }
-  if (lane == 31) wsum[w] = incl;
-  __syncthreads();
-  if (w == 0) {
-    const int x = wsum[lane];
-    int y = x;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int t = __shfl_up_sync(kFull, y, o);
-      if (lane >= o) y += t;
-    }
-    wsum[lane] = y - x;
-  }
-  __syncthreads();
-  const int excl = wsum[w] + incl - run;
-  int* __restrict__ offset = off_new_all + a.off_base;
-  if (c < n_cells) offset[c] = a.part_base + excl;
-  if (c == n_cells - 1) offset[n_cells] = a.part_base + excl + run;
-  // Graph replay: the step's collide/move pass has finished reading the step number.
-  if (SL.gstep_dev != nullptr && c == 0) *SL.gstep_dev += 1;
-}
-
-bool prefix_small_fits(const StepLaunch& L) {
-  return L.n_inst == 1 && L.max_cells <= kPrefixSmallCells &&
-         (long long)L.max_spans * L.rows <= kScanColsMaxRows;
-}
-
-cudaError_t launch_prefix_small(int* hist, int* off_new, const InstParams& one,
-                                const StepLaunch& L, cudaStream_t st) {
-  k_prefix_small<<<1, kPrefixSmallCells, 0, st>>>(hist, off_new, one, L);
-  return cudaGetLastError();
 }
 
 __global__ void k_set_counter(long long* counter, long long value) { *counter = value; }
@@ -1065,23 +1042,24 @@ int scatter_spans_warps(int n_cells) {
   return w < 1 ? 1 : (int)w;
 }
 
-size_t scatter_coop_smem(int max_cells) {
+static size_t scatter_coop_smem(int max_cells) {
   return (size_t)(kCoopWarps + 1) * (size_t)max_cells * sizeof(int);
 }
 
 cudaError_t launch_scatter_spans(const float4* P, float4* P2, const int* off_cur,
-                                 const int* off_new, const int* hist, const InstParams& one,
-                                 const StepLaunch& L, int* err, cudaStream_t st) {
-  const size_t coop = scatter_coop_smem(L.max_cells);
-  if (coop <= kCoopSmemMax) {  // a CTA per (span, row)
+                                 const int* count, int* off_new, const int* hist,
+                                 const InstParams& one, const StepLaunch& L, int* err,
+                                 cudaStream_t st) {
+  if (scatter_forms_offsets(L)) {  // a CTA per (span, row)
+    const size_t coop = scatter_coop_smem(L.max_cells);
     const int units = L.n_spans_total * L.rows;
     // two slices per warp and round once the rows average 4,096 records (the batch's
     // tuned spans: 0.328 -> 0.30 ms); one for shorter rows (small runs' 1,024-particle
     // spans, where fewer, longer rounds were slower)
     const bool two = L.n_part_total >= 4096LL * units;
 #define DSMC_COOP(B, S)                                                                  \
-  k_scatter_coop<B, S><<<units, kCoopWarps * 32, coop, st>>>(P, P2, off_cur, off_new, hist, \
-                                                             one, L, err)
+  k_scatter_coop<B, S><<<units, kCoopWarps * 32, coop, st>>>(P, P2, off_cur, count, off_new, \
+                                                             hist, one, L, err)
     if (L.n_inst == 1) {
       if (two) DSMC_COOP(false, 2); else DSMC_COOP(false, 1);
     } else {
@@ -1128,12 +1106,17 @@ cudaError_t launch_scan_spans(int* hist, int* count, const InstParams& one, cons
       k_scan_cols<true><<<grid, kScanColsCells, 0, st>>>(hist, count, one, L);
     return cudaGetLastError();
   }
-  const dim3 grid((L.max_cells + 31) / 32, L.n_inst);
+  const dim3 grid((L.max_cells + kScanCells - 1) / kScanCells, L.n_inst);
+  const dim3 block(kScanCells, kScanSegs);
   if (L.n_inst == 1)
-    k_scan_spans<false><<<grid, dim3(32, 32), 0, st>>>(hist, count, one, L);
+    k_scan_spans<false><<<grid, block, 0, st>>>(hist, count, one, L);
   else
-    k_scan_spans<true><<<grid, dim3(32, 32), 0, st>>>(hist, count, one, L);
+    k_scan_spans<true><<<grid, block, 0, st>>>(hist, count, one, L);
   return cudaGetLastError();
+}
+
+bool scatter_forms_offsets(const StepLaunch& L) {
+  return scatter_coop_smem(L.max_cells) <= kCoopSmemMax;
 }
 
 cudaError_t launch_offsets_cells(const int* count, int* off_new, const InstParams& one,
