@@ -104,9 +104,11 @@ typedef struct dsmc_options {
   int profile;            /* 1: time every kernel launch with CUDA events (then
                              dsmc_step synchronises at its end); default 0 */
   int span_particles;     /* particles per span (CTA) of the step passes at the
-                             initial density: 0 keeps the partition in use (at creation
-                             4096, or fewer down to 1024 when the handle holds less than
-                             two such spans per SM; or what dsmc_autotune chose), else
+                             initial density: 0 leaves the partition to the library
+                             (one run: 4096, or fewer down to 1024 when it holds less
+                             than two such spans per SM; batches and pools: 1024 to
+                             8192 by the particles of the active instances; or what
+                             dsmc_autotune chose, or an earlier value), else
                              1024..2^24.
                              Only the work split changes: results are identical for
                              every value.  While this, cta_warps and span_rows are
@@ -117,8 +119,10 @@ typedef struct dsmc_options {
                              a value in any of the three keeps the span passes;
                              default 0 */
   int cta_warps;          /* warps per CTA of the collide/move pass: 0 keeps the shape
-                             in use (8 at creation, 4 for a pool, or what dsmc_autotune
-                             chose), else 4 or 8; results are identical; default 0 */
+                             in use (one run: 8; batches and pools: 8, or 4 from about
+                             40,000 particles per SM on; or what dsmc_autotune chose,
+                             or an earlier value), else 4 or 8; results are identical;
+                             default 0 */
   int span_rows;          /* sort-matrix rows per span, one per equal part of its
                              slots, each scattered by its own warp: 0 keeps the value
                              in use (1 at creation, or what dsmc_autotune chose), else

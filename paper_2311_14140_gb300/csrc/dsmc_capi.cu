@@ -355,6 +355,10 @@ struct dsmc_sim {
   std::vector<int> order;  // active ids in table order
   long long gstep = 0;     // steps this handle has launched
   int span_target = kDefaultSpanParticles;
+  // The split of the span passes follows the instances (choose_split) until the options or the
+  // tuner name one; instances were added or removed since it was made.
+  bool auto_split = true, split_dirty = false;
+  int check_warps = kAWarps;  // warps per CTA that instances' sizes are checked against
   int cta_warps = kAWarps;  // warps per CTA of the collide/move pass
   int span_rows = 1;        // sort-matrix rows per span
   int spans = 0, max_cps = 1, max_cells = 1, max_spans = 1;  // partition in use
@@ -532,6 +536,41 @@ void set_partition(dsmc_sim* h, int target) {
   h->graph_valid = false;
 }
 
+int default_span_particles(long long n);
+
+// Warps per CTA and particles per span for the active instances of a batch or pool, by their
+// particles: 4-warp CTAs and 8,192 particles from about 40,000 particles per SM on (24 million:
+// 657 us per step, 8 warps 688, the former default of 4,096 and 4 warps 692), below that
+// 8-warp CTAs (fewer, larger CTAs leave fewer SMs idle behind the last spans) with spans that
+// give every place on the SMs one, 1,024 to 5,120 particles (0.94 million: 54 us per step
+// against 74; 2.9 million: 101 against 116; 5.8 million: 192 against 190).  One run of its own
+// keeps 8 warps and default_span_particles.
+void choose_split(dsmc_sim* h) {
+  if (!h->pool && h->n_inst() <= 1) return;
+  long long n = 0;
+  for (int id : h->order) n += h->inst[id].N;
+  int warps = kAWarps;
+  long long target = std::min<long long>(5120, std::max<long long>(kMinSpanParticles,
+                                                                   n / (3LL * h->sms)));
+  if (n >= 40000LL * h->sms) {
+    warps = kAWarpsSmall;
+    target = 8192;
+  }
+  int mcps, mcells;
+  partition_extent(h, (int)target, nullptr, &mcps, &mcells);
+  if (!step_fits(mcells, mcps, h->opt.group_size, warps, h->span_rows)) warps = kAWarpsSmall;
+  h->cta_warps = warps;
+  h->span_target = (int)target;
+}
+
+// Brings the partition up to date with the active instances.
+void ensure_partition(dsmc_sim* h) {
+  if (!h->split_dirty) return;
+  h->split_dirty = false;
+  if (h->auto_split) choose_split(h);
+  set_partition(h, h->span_target);
+}
+
 InstParams instance_params(const dsmc_sim* h, int id, int span_base) {
   const Inst& x = h->inst[id];
   InstParams a{};
@@ -578,6 +617,7 @@ InstParams instance_params(const dsmc_sim* h, int id, int span_base) {
 // the device (ordered on the stream before the next launch).  The copies read
 // pageable host memory, which CUDA stages before the call returns.
 dsmc_status upload_tables(dsmc_sim* h) {
+  ensure_partition(h);
   if (h->tab_dirty) {
     h->tab.resize(h->order.size());
     for (int t = 0; t < h->n_inst(); ++t)
@@ -679,6 +719,7 @@ dsmc_status run_index(dsmc_sim* h) {
 // a sort into cells of those instances alone into the current buffers (the other
 // instances are not touched).
 dsmc_status admit_fresh(dsmc_sim* h) {
+  ensure_partition(h);
   std::vector<int> ids;
   for (int id : h->order)
     if (h->inst[id].fresh) ids.push_back(id);
@@ -920,6 +961,7 @@ bool size_resident(dsmc_sim* h, ResidentLaunch& R) {
 }
 
 void plan_resident(dsmc_sim* h) {
+  ensure_partition(h);
   h->res = ResidentLaunch{};
   h->res_dirty = false;
   if (h->pool || h->opt.profile || h->span_passes) return;
@@ -977,7 +1019,7 @@ dsmc_status step_n(dsmc_sim* h, int n_steps) {
   if ((s = admit_fresh(h)) != DSMC_OK) return s;
   int it = 0;
   if (h->n_inst() > 0 && n_steps > 0) {
-    if (h->res_dirty) plan_resident(h);
+    if (h->res_dirty || h->split_dirty) plan_resident(h);
     if (h->res.cl > 0) {
       if ((s = upload_tables(h)) != DSMC_OK) return s;
       while (it < n_steps) {
@@ -1024,7 +1066,7 @@ dsmc_status add_instance(dsmc_sim* h, const dsmc_instance& d, int index, int n_d
                                   "time step undefined: set options.dt for infinite Kn");
   int mcps, mcells;
   partition_extent(h, h->span_target, &x, &mcps, &mcells);
-  if (!step_fits(mcells, mcps, h->opt.group_size, h->cta_warps, h->span_rows))
+  if (!step_fits(mcells, mcps, h->opt.group_size, h->check_warps, h->span_rows))
     return fail(DSMC_E_INVAL, "n_cells and group_size exceed the step's shared memory");
   // Find a free id and room in every array.
   int new_id = -1;
@@ -1064,7 +1106,7 @@ dsmc_status add_instance(dsmc_sim* h, const dsmc_instance& d, int index, int n_d
   }
   h->order.push_back(new_id);
   h->spans_reserved += x.max_spans;
-  set_partition(h, h->span_target);
+  h->split_dirty = true;
   *id = new_id;
   return DSMC_OK;
 }
@@ -1094,10 +1136,9 @@ dsmc_status new_handle(const Capacity& C, const dsmc_options& opt, bool pool, vo
   h->C = C;
   h->L = layout_of(C);
   h->span_target = opt.span_particles ? opt.span_particles : default_span_particles(C.slots);
-  // A pool holds many small instances whose membership changes too often to tune live;
-  // 4-warp CTAs are what dsmc_autotune picks for such batches (8 % more micro-solves/s
-  // than 8-warp CTAs in the request loop).
   h->cta_warps = opt.cta_warps ? opt.cta_warps : (pool ? kAWarpsSmall : kAWarps);
+  h->check_warps = h->cta_warps;
+  h->auto_split = !opt.span_particles && !opt.cta_warps;
   h->span_rows = opt.span_rows ? opt.span_rows : 1;
   h->span_passes = names_partition(opt);
   h->ex_slots.reset(C.slots);
@@ -1346,7 +1387,7 @@ dsmc_status dsmc_pool_remove(dsmc_handle h, int id) {
   x.active = false;
   x.fresh = false;
   h->order.erase(std::find(h->order.begin(), h->order.end(), id));
-  set_partition(h, h->span_target);
+  h->split_dirty = true;
   return DSMC_OK;
 }
 
@@ -1411,8 +1452,11 @@ dsmc_status dsmc_set_options(dsmc_handle h, const dsmc_options* opt) {
       return fail(DSMC_E_INVAL, "time step undefined: set options.dt for infinite Kn");
   }
   // span_particles = 0 and cta_warps = 0 keep the partition and CTA shape in use.
+  ensure_partition(h);
+  if (opt->span_particles || opt->cta_warps) h->auto_split = false;
   const int target_use = opt->span_particles ? opt->span_particles : h->span_target;
-  const int warps_use = opt->cta_warps ? opt->cta_warps : h->cta_warps;
+  const int warps_use = opt->cta_warps ? opt->cta_warps
+                                       : (h->auto_split ? h->check_warps : h->cta_warps);
   const int rows_use = opt->span_rows ? opt->span_rows : h->span_rows;
   int mcps, mcells;
   partition_extent(h, target_use, nullptr, &mcps, &mcells);
@@ -1425,7 +1469,11 @@ dsmc_status dsmc_set_options(dsmc_handle h, const dsmc_options* opt) {
   h->opt = *opt;
   h->span_passes = names_partition(*opt);
   for (int id : h->order) h->inst[id].p = ps[id];
-  h->cta_warps = warps_use;
+  if (h->auto_split)
+    h->split_dirty = true;  // the group size bears on the choice
+  else
+    h->cta_warps = warps_use;
+  if (opt->cta_warps) h->check_warps = warps_use;
   h->span_rows = rows_use;
   if (target_use != h->span_target) set_partition(h, target_use);
   h->tab_dirty = h->res_dirty = true;
@@ -1460,6 +1508,7 @@ dsmc_status dsmc_autotune(dsmc_handle h, int steps_per_trial, int* best_span_par
     cudaEventDestroy(e0);
     return fail(DSMC_E_CUDA, "event");
   }
+  ensure_partition(h);
   int best = h->span_target, best_warps = h->cta_warps, best_rows = h->span_rows;
   double best_ms = -1.0;
   dsmc_status r = DSMC_OK;
@@ -1508,7 +1557,8 @@ dsmc_status dsmc_autotune(dsmc_handle h, int steps_per_trial, int* best_span_par
   h->span_passes = span_passes;
   h->res_dirty = true;
   if (r != DSMC_OK) return r;
-  h->cta_warps = best_warps;
+  h->auto_split = false;
+  h->cta_warps = h->check_warps = best_warps;
   h->span_rows = best_rows;
   set_partition(h, best);
   h->opt.span_particles = best;
@@ -1712,6 +1762,7 @@ dsmc_status dsmc_get_info_of(dsmc_handle h, int id, dsmc_info* info) {
   dsmc_status s = check_index(h, id);
   if (s != DSMC_OK) return s;
   if (!info) return fail(DSMC_E_INVAL, "info: NULL");
+  ensure_partition(h);
   const Inst& x = h->inst[id];
   info->n_particles = x.N;
   info->n_cells = x.n_cells;
