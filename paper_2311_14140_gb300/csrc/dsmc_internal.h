@@ -321,6 +321,24 @@ cudaError_t launch_admit_cells(const InstParams* tab, int n, int* off, float* sm
 // count and of vx, into out[2 id] and out[2 id + 1].
 cudaError_t launch_channel_sums(const InstParams* tab, int n, const double* acc, double* out,
                                 cudaStream_t st);
+// One instance's cell data and the error word in one block (byte offsets).
+struct CellBlock {
+  static constexpr size_t kPerCell = 8 + 8 + 4 + 4 + 8;  // the last 8: the block's three ends
+  size_t ncand, nacc, smax, offset, err, total;
+  __host__ __device__ explicit CellBlock(int n_cells) {
+    const size_t n = (size_t)n_cells;
+    ncand = 0;
+    nacc = 8 * n;
+    smax = 16 * n;
+    offset = 20 * n;
+    err = 24 * n + 4;
+    total = 24 * n + 8;
+  }
+};
+cudaError_t launch_gather_cells(const int* off, int base, const float* smax,
+                                const unsigned long long* ncand, const unsigned long long* nacc,
+                                const int* err, int n_cells, char* block, cudaStream_t st);
+// (NULL arrays are left out)
 cudaError_t launch_unpack(const float4* P, float* y, float* vx, float* vy, float* vz, int N,
                           cudaStream_t st);
 cudaError_t launch_pack(const float* y, const float* vx, const float* vy, const float* vz,

@@ -974,11 +974,30 @@ __global__ void k_unpack(const float4* __restrict__ P, float* __restrict__ y,
                          int N) {
   for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < N; p += gridDim.x * blockDim.x) {
     const float4 r = P[p];
-    y[p] = r.x;
-    vx[p] = r.y;
-    vy[p] = r.z;
-    vz[p] = r.w;
+    if (y) y[p] = r.x;
+    if (vx) vx[p] = r.y;
+    if (vy) vy[p] = r.z;
+    if (vz) vz[p] = r.w;
   }
+}
+
+// An instance's cell data (offsets relative to its first slot) and the error word in one block.
+__global__ void k_gather_cells(const int* __restrict__ off, int base,
+                               const float* __restrict__ smax,
+                               const unsigned long long* __restrict__ ncand,
+                               const unsigned long long* __restrict__ nacc,
+                               const int* __restrict__ err, int n_cells, char* block) {
+  const CellBlock B(n_cells);
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c > n_cells) return;
+  reinterpret_cast<int*>(block + B.offset)[c] = off[c] - base;
+  if (c == n_cells) {
+    *reinterpret_cast<int*>(block + B.err) = *err;
+    return;
+  }
+  reinterpret_cast<unsigned long long*>(block + B.ncand)[c] = ncand[c];
+  reinterpret_cast<unsigned long long*>(block + B.nacc)[c] = nacc[c];
+  reinterpret_cast<float*>(block + B.smax)[c] = smax[c];
 }
 
 // Pack four arrays into records; y is moved onto the nearest wall if outside [0, 1].
@@ -1143,6 +1162,14 @@ cudaError_t launch_admit_cells(const InstParams* tab, int n, int* off, float* sm
 cudaError_t launch_channel_sums(const InstParams* tab, int n, const double* acc, double* out,
                                 cudaStream_t st) {
   k_channel_sums<<<n, 256, 0, st>>>(tab, acc, out);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_gather_cells(const int* off, int base, const float* smax,
+                                const unsigned long long* ncand, const unsigned long long* nacc,
+                                const int* err, int n_cells, char* block, cudaStream_t st) {
+  k_gather_cells<<<(n_cells + 1 + 255) / 256, 256, 0, st>>>(off, base, smax, ncand, nacc, err,
+                                                           n_cells, block);
   return cudaGetLastError();
 }
 
