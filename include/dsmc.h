@@ -106,10 +106,11 @@ typedef struct dsmc_options {
   int span_particles;     /* particles per span (CTA) of the step passes at the
                              initial density: 0 leaves the partition to the library
                              (one run: 4096, or fewer down to 1024 when it holds less
-                             than two such spans per SM; batches and pools: 1024 to
-                             8192 by the particles of the active instances; or what
-                             dsmc_autotune chose, or an earlier value), else
-                             1024..2^24.
+                             than two such spans per SM, and several spans per cell
+                             when there would be too few to fill the SMs; batches and
+                             pools: 1024 to 8192 by the particles of the active
+                             instances; or what dsmc_autotune chose, or an earlier
+                             value), else 1024..2^24.
                              Only the work split changes: results are identical for
                              every value.  While this, cta_warps and span_rows are
                              all 0, steps of one run of up to about 1,300,000
@@ -120,7 +121,7 @@ typedef struct dsmc_options {
                              default 0 */
   int cta_warps;          /* warps per CTA of the collide/move pass: 0 keeps the shape
                              in use (one run: 8; batches and pools: 8, or 4 from about
-                             40,000 particles per SM on; or what dsmc_autotune chose,
+                             46,000 particles per SM on; or what dsmc_autotune chose,
                              or an earlier value), else 4 or 8; results are identical;
                              default 0 */
   int span_rows;          /* sort-matrix rows per span, one per equal part of its

@@ -81,6 +81,22 @@ void make_spans(int n_cells, int ppc, int target, int* cps, int* n_spans) {
   *n_spans = (int)((n_cells + c - 1) / c);
 }
 
+// Spans per cell of one run with few, populous cells: a cell is then shared by several CTAs, so
+// that the run still makes about kPartSpans spans, of about kPartMin particles or more (16
+// collision groups of 256 for a CTA's 8 warps).  us per step, whole cells -> shared: 200 x 50,000 425 ->
+// 186, 100 x 25,000 195 -> 76, 20 x 100,000 587 -> 65, 300 x 6,666 90 -> 69, 700 x 25,000 366 ->
+// 314.  From about 320 cells on the whole cells of less than 10,000 particles keep most places
+// on the SMs busy, and the larger sort matrix and the sums cost more than sharing gives (400 x
+// 5,000 101 -> 113 at Kn = 6, 860 x 9,302 175 -> 176).
+constexpr int kPartSpans = 900, kPartMin = 4096, kPartCells = 320, kPartLarge = 10000;
+
+int cell_parts(int n_cells, int ppc) {
+  if (n_cells > kPartCells && ppc < kPartLarge) return 1;
+  const long long N = (long long)n_cells * ppc;
+  const long long t = std::max<long long>(kPartMin, N / kPartSpans);
+  return (int)std::max<long long>(1, (ppc + t - 1) / t);
+}
+
 // Parameters of the method in binary64, rounded once to binary32 where the kernels
 // use them.
 struct Params {
@@ -216,6 +232,7 @@ struct Inst {
   int part_base = 0, cell_base = 0, off_base = 0;
   long long hist_base = 0;
   int cps = 0, n_spans = 0, span_base = 0;  // partition in use
+  int parts = 1;                            // spans per cell (cps 1)
   long long step = 0, n_samples = 0;
   int open_top = 0;  // y = 1 an open Chapman-Enskog interface
   float u_top = 0.0f, p_top = 0.0f;
@@ -278,12 +295,23 @@ Layout layout_of(const Capacity& C) {
   return L;
 }
 
+// Ints of the sums of n_cells shared cells: 12 64-bit sums and a maximum each.
+long long cell_sums_ints(int n_cells) { return 25LL * n_cells; }
+
+// The rows of the sort matrix reserved for an instance: its finest partition; for one run of its
+// own also the partition that shares cells.
+int reserved_rows(int n_cells, int ppc, bool alone) {
+  const int r = reserved_spans(n_cells, ppc);
+  const int parts = alone ? cell_parts(n_cells, ppc) : 1;
+  return parts > 1 ? std::max(r, n_cells * parts) : r;
+}
+
 // The capacity that holds exactly these instances, placed one after another.
 Capacity capacity_of(const dsmc_instance* d, int n) {
   Capacity C{};
   for (int i = 0; i < n; ++i) {
     const long long N = (long long)d[i].n_cells * d[i].ppc;
-    const int rows = reserved_spans(d[i].n_cells, d[i].ppc);
+    const int rows = reserved_rows(d[i].n_cells, d[i].ppc, n == 1);
     C.slots += padded_slots(N);
     C.cells += d[i].n_cells;
     C.offs += d[i].n_cells + 1;
@@ -296,6 +324,9 @@ Capacity capacity_of(const dsmc_instance* d, int n) {
   if (n == 1 && C.slots <= kTeamParticles)
     C.hist_ints = std::max<long long>(C.hist_ints,
                                       (long long)team_exchange_ints(kTeamMax, d[0].n_cells));
+  // and, behind it all, for the sums of cells that several CTAs share
+  if (n == 1 && cell_parts(d[0].n_cells, d[0].ppc) > 1)
+    C.hist_ints = ((C.hist_ints + 1) & ~1LL) + cell_sums_ints(d[0].n_cells);
   return C;
 }
 
@@ -496,10 +527,11 @@ void set_span_order(dsmc_sim* h) {
     const Inst& x = h->inst[h->order[t]];
     const double dt = x.p.dt;
     for (int k = 0; k < x.n_spans; ++k) {
-      const int c0 = k * x.cps, c1 = std::min(c0 + x.cps, x.n_cells);
+      const int c0 = k / x.parts * x.cps, c1 = std::min(c0 + x.cps, x.n_cells);
       const double yc = 0.5 * (c0 + c1) / x.n_cells;
       const double hits = dt > 0.0 ? 0.5 * (std::erfc(yc / dt) + std::erfc((1.0 - yc) / dt)) : 0.0;
-      cost.emplace_back(-(double)(c1 - c0) * x.ppc * (1.0 + 2.2 * hits), x.span_base + k);
+      cost.emplace_back(-(double)(c1 - c0) * x.ppc / x.parts * (1.0 + 2.2 * hits),
+                        x.span_base + k);
     }
   }
   std::stable_sort(cost.begin(), cost.end(),
@@ -520,6 +552,11 @@ void set_partition(dsmc_sim* h, int target) {
     Inst& x = h->inst[h->order[t]];
     np += x.N;
     make_spans(x.n_cells, x.ppc, target, &x.cps, &x.n_spans);
+    x.parts = h->auto_split && !h->pool && h->C.inst == 1 ? cell_parts(x.n_cells, x.ppc) : 1;
+    if (x.parts > 1) {
+      x.cps = 1;
+      x.n_spans = x.n_cells * x.parts;
+    }
     x.span_base = base;
     base += x.n_spans;
     m = std::max(m, x.cps);
@@ -540,22 +577,43 @@ void set_partition(dsmc_sim* h, int target) {
 int default_span_particles(long long n);
 
 // Warps per CTA and particles per span for the active instances of a batch or pool, by their
-// particles: 4-warp CTAs and 8,192 particles from about 40,000 particles per SM on (24 million:
-// 657 us per step, 8 warps 688, the former default of 4,096 and 4 warps 692), below that
-// 8-warp CTAs (fewer, larger CTAs leave fewer SMs idle behind the last spans) with spans that
-// give every place on the SMs one, 1,024 to 5,120 particles (0.94 million: 54 us per step
-// against 74; 2.9 million: 101 against 116; 5.8 million: 192 against 190).  One run of its own
+// particles (us per step of pools of uneven instances; in brackets the former 4-warp CTAs of
+// 4,096 particles): below 46,000 particles per SM 8-warp CTAs (fewer, larger CTAs leave fewer
+// SMs idle behind the last spans) with spans that give every place on the SMs about one, 1,024
+// to 8,192 particles (0.94 million particles 55 [74], 2.9 million 101 [116], 4.1 million 133
+// [137], 6.9 million 208 [209]); from there 4-warp CTAs with 5,120 (8.9 million 260 [267], 15.8
+// million 433 [452]), from 120,000 per SM on 8,192 (24 million 657 [692]).  One run of its own
 // keeps 8 warps and default_span_particles.
 void choose_split(dsmc_sim* h) {
-  if (!h->pool && h->n_inst() <= 1) return;
+  if (!h->pool && h->n_inst() <= 1) {
+    if (h->n_inst() == 1) {
+      const Inst& x = h->inst[h->order[0]];
+      long long target;
+      if (x.n_cells > kCoopCells) {
+        // a scatter with a warp per span wants about 6.6 of them per SM (3,000 x 500: 334 spans
+        // 106 us per step, 1,000 spans 64; 4,000 x 1,500: 1,334 spans 196, 1,000 spans 185)
+        target = std::min<long long>(5120, x.N / (33LL * h->sms / 5));
+      } else {
+        // whole cells, nearest to 4,096 particles or to one span per place of an 8-warp CTA on
+        // the SMs, rather more than less (600 x 3,500: 300 spans 82 us per step, 600 spans 65;
+        // 1,000 x 2,000: 334 spans 82, 500 spans 70; 700 x 2,857 at Kn = 6: 350 spans 104, 700
+        // spans 115)
+        const long long t = std::min<long long>(kDefaultSpanParticles, x.N / (3LL * h->sms));
+        target = std::max<long long>(1, (10 * t + 6LL * x.ppc) / (10LL * x.ppc)) * x.ppc;
+      }
+      h->span_target = (int)std::min<long long>(kMaxSpanParticles,
+                                                std::max<long long>(kMinSpanParticles, target));
+    }
+    return;
+  }
   long long n = 0;
   for (int id : h->order) n += h->inst[id].N;
   int warps = kAWarps;
-  long long target = std::min<long long>(5120, std::max<long long>(kMinSpanParticles,
-                                                                   n / (3LL * h->sms)));
-  if (n >= 40000LL * h->sms) {
+  long long target =
+      std::min<long long>(8192, std::max<long long>(kMinSpanParticles, 2 * n / (7LL * h->sms)));
+  if (n >= 46000LL * h->sms) {
     warps = kAWarpsSmall;
-    target = 8192;
+    target = n >= 120000LL * h->sms ? 8192 : 5120;
   }
   int mcps, mcells;
   partition_extent(h, (int)target, nullptr, &mcps, &mcells);
@@ -581,6 +639,7 @@ InstParams instance_params(const dsmc_sim* h, int id, int span_base) {
   a.span_base = span_base;
   a.n_spans = x.n_spans;
   a.cps = x.cps;
+  a.parts = x.parts;
   a.part_base = x.part_base;
   a.n_part = (int)x.N;
   a.hist_base = x.hist_base;
@@ -675,13 +734,22 @@ dsmc_status launch_pass(dsmc_sim* h, bool count_only, const StepLaunch& SL,
   cudaStream_t s = h->stream();
   int* off_cur = h->off[osrc];
   int* off_new = h->off[osrc ^ 1];
+  CellSums sums{};
+  if (one.parts > 1) {
+    sums.off = off_cur;
+    sums.smax_in = h->smax[h->scur];
+    sums.smax_out = h->smax[h->scur ^ 1];
+    sums.acc = h->acc;
+    sums.fix = (unsigned long long*)(h->hist + h->C.hist_ints - cell_sums_ints(one.n_cells));
+    sums.gmax = (unsigned*)(sums.fix + (size_t)one.n_cells * 12);
+  }
   DSMC_CUDA(timed(h, count_only ? K_INDEX_COUNT : K_COLLIDE_MOVE, [&] {
               return launch_collide_move(h->P[src], off_cur, h->smax[h->scur],
                                          h->smax[h->scur ^ 1], h->ncand, h->nacc, h->acc,
-                                         h->hist, one, SL, h->err, s);
+                                         h->hist, sums, one, SL, h->err, s);
             }),
             count_only ? "index_count" : "collide_move");
-  DSMC_CUDA(timed(h, K_SCAN, [&] { return launch_scan_spans(h->hist, h->count, one, SL, s); }),
+  DSMC_CUDA(timed(h, K_SCAN, [&] { return launch_scan_spans(h->hist, h->count, sums, one, SL, s); }),
             "scan_hist");
   if (!scatter_forms_offsets(SL))
     DSMC_CUDA(timed(h, K_OFFSETS,
@@ -758,6 +826,10 @@ dsmc_status admit_fresh(dsmc_sim* h) {
   DSMC_CUDA(launch_admit_cells(adm_tab_dev, (int)ids.size(), h->off[oidle], h->smax[h->scur],
                                h->ncand, h->nacc, h->acc, s),
             "admit cells");
+  if (h->adm_tab[0].parts > 1) {
+    const long long n = cell_sums_ints(h->adm_tab[0].n_cells);
+    DSMC_CUDA(cudaMemsetAsync(h->hist + h->C.hist_ints - n, 0, n * sizeof(int), s), "cell sums");
+  }
   StepLaunch SL{};
   SL.n_inst = (int)ids.size();
   SL.tab = adm_tab_dev;
@@ -1145,7 +1217,7 @@ dsmc_status add_instance(dsmc_sim* h, const dsmc_instance& d, int index, int n_d
     }
   if (new_id < 0 && (int)h->inst.size() >= h->C.inst)
     return fail(DSMC_E_NOMEM, "no room: instance table full");
-  x.max_spans = reserved_spans(x.n_cells, x.ppc);
+  x.max_spans = reserved_rows(x.n_cells, x.ppc, !h->pool && h->C.inst == 1);
   if (h->spans_reserved + x.max_spans > h->C.spans)
     return fail(DSMC_E_NOMEM, "no room: span table full");
   x.slot_len = padded_slots(x.N);
@@ -1582,6 +1654,11 @@ dsmc_status dsmc_autotune(dsmc_handle h, int steps_per_trial, int* best_span_par
   dsmc_status r = DSMC_OK;
   const bool span_passes = h->span_passes;
   h->span_passes = h->res_dirty = true;  // the trials are of the span passes
+  // a run whose cells are shared by several CTAs keeps that partition, which the trials'
+  // whole-cell spans cannot reach
+  const bool shared = h->inst[h->order[0]].parts > 1;
+  const int own_target = h->span_target, own_warps = h->cta_warps, own_rows = h->span_rows;
+  h->auto_split = false;
   const int shapes[4][2] = {{kAWarps, 1}, {kAWarps, 2}, {kAWarpsSmall, 1}, {kAWarpsSmall, 2}};
   for (const auto& shape : shapes) {
     const int w = shape[0], rows = shape[1];
@@ -1624,14 +1701,23 @@ dsmc_status dsmc_autotune(dsmc_handle h, int steps_per_trial, int* best_span_par
   cudaEventDestroy(e1);
   h->span_passes = span_passes;
   h->res_dirty = true;
-  if (r != DSMC_OK) return r;
-  h->auto_split = false;
-  h->cta_warps = h->check_warps = best_warps;
-  h->span_rows = best_rows;
-  set_partition(h, best);
-  h->opt.span_particles = best;
-  h->opt.cta_warps = best_warps;
-  h->opt.span_rows = best_rows;
+  if (r != DSMC_OK) {
+    h->auto_split = shared;
+    return r;
+  }
+  if (shared) {
+    h->auto_split = true;
+    h->cta_warps = own_warps;
+    h->span_rows = own_rows;
+    set_partition(h, own_target);
+  } else {
+    h->cta_warps = h->check_warps = best_warps;
+    h->span_rows = best_rows;
+    set_partition(h, best);
+    h->opt.span_particles = best;
+    h->opt.cta_warps = best_warps;
+    h->opt.span_rows = best_rows;
+  }
   if (best_span_particles) *best_span_particles = best;
   if (best_ms_per_step) *best_ms_per_step = best_ms;
   if (h->opt.profile) return collect_times(h);

@@ -25,6 +25,7 @@ constexpr int kMaxSpans = 152 * 16;   // rows of the per-step sort matrix, at mo
 // the batch of small instances keeps 5 CTAs per SM), 4 % faster than 256 on the batch.
 constexpr int kMaxCellsPerSpan = 24;
 constexpr size_t kStepSmemMax = 220 * 1024;
+constexpr int kCoopCells = 1365;  // the scatter takes a CTA per span up to here, then a warp
 constexpr int kSortWarpsMax = 152 * 16;
 constexpr int kSortWarpsPerBlock = 8;
 constexpr size_t kSortSmemMax = 200 * 1024;
@@ -87,6 +88,7 @@ struct InstParams {
   int span_base;   // first global span
   int n_spans;
   int cps;         // cells per span (one collide/move CTA each)
+  int parts;       // spans per cell (cps 1): a cell of many particles is shared by several CTAs
   int part_base;   // first global slot of the instance's particles
   int n_part;
   long long hist_base;  // first entry of the instance's sort matrix (n_spans x n_cells)
@@ -112,6 +114,17 @@ struct InstParams {
   // cluster-resident steps: CTA r takes the groups that start in slots
   // [part_base + cut[r], part_base + cut[r + 1])
   int cut[17];
+};
+
+// What the CTAs that share a cell (InstParams::parts > 1) add up, and what the scan of the sort
+// matrix, after them, makes the cell's results of.
+struct CellSums {
+  const int* off;                // this step's cell offsets
+  const float* smax_in;
+  float* smax_out;
+  double* acc;
+  unsigned long long* fix;       // n_cells x 12 fixed-point moment sums, zero between steps
+  unsigned* gmax;                // largest relative speeds (binary32 bits), zero between steps
 };
 
 constexpr int kWallQueue = 64;  // a group's slice of hits on top of at most 31 waiting ones
@@ -297,8 +310,8 @@ cudaError_t launch_cell_fields(const double* acc, int n_cells, long long n_sampl
 cudaError_t launch_collide_move(float4* P, const int* off, const float* smax_in,
                                 float* smax_out, unsigned long long* ncand,
                                 unsigned long long* nacc, double* acc, int* hist,
-                                const InstParams& one, const StepLaunch& L, int* err,
-                                cudaStream_t st);
+                                const CellSums& sums, const InstParams& one,
+                                const StepLaunch& L, int* err, cudaStream_t st);
 // The new cell offsets (off_new) from the cells' counts: formed by the scatter, or by
 // launch_offsets_cells before it.
 bool scatter_forms_offsets(const StepLaunch& L);
@@ -308,8 +321,8 @@ cudaError_t launch_scatter_spans(const float4* P, float4* P2, const int* off_cur
                                  const int* count, int* off_new, const int* hist,
                                  const InstParams& one, const StepLaunch& L, int* err,
                                  cudaStream_t st);
-cudaError_t launch_scan_spans(int* hist, int* count, const InstParams& one, const StepLaunch& L,
-                              cudaStream_t st);
+cudaError_t launch_scan_spans(int* hist, int* count, const CellSums& sums, const InstParams& one,
+                              const StepLaunch& L, cudaStream_t st);
 cudaError_t launch_set_counter(long long* counter, long long value, cudaStream_t st);
 // Per-cell arrays of newly added instances (table `tab`, n of them): moment sums and
 // collision counters zeroed, (sigma g)_max set to smax0, and cell offsets of whole

@@ -110,6 +110,36 @@ __device__ __forceinline__ const InstParams& stage_instance(const InstParams& on
   }
 }
 
+// Span `span` of an instance: its cells [c0, c1) and slots [sb0, sb1); with several spans per
+// cell also the groups [g0, g1) of the cell that are its share (g1 = -1: all groups).
+struct SpanRange {
+  int c0, c1, sb0, sb1, g0, g1;
+};
+
+__device__ __forceinline__ SpanRange span_range(const InstParams& a, const int* __restrict__ off,
+                                                int span) {
+  SpanRange s;
+  if (a.parts == 1) {
+    s.c0 = span * a.cps;
+    s.c1 = min(s.c0 + a.cps, a.n_cells);
+    s.sb0 = off[s.c0];
+    s.sb1 = off[s.c1];
+    s.g0 = 0;
+    s.g1 = -1;
+  } else {
+    s.c0 = span / a.parts;
+    s.c1 = s.c0 + 1;
+    const int j = span - s.c0 * a.parts;
+    const int first = off[s.c0], end = off[s.c1];
+    const int ng = group_count(end - first, a.G);
+    s.g0 = (int)((long long)ng * j / a.parts);
+    s.g1 = (int)((long long)ng * (j + 1) / a.parts);
+    s.sb0 = s.g0 == ng ? end : first + s.g0 * a.G;
+    s.sb1 = s.g1 == ng ? end : first + s.g1 * a.G;
+  }
+  return s;
+}
+
 // Collision models (a.mode): 0 hard spheres, 1 VHS with 0.5 < omega < 1, 2 omega = 1
 // (sigma g independent of g).  CTAs per SM the register budget is set for: 3 of 8 warps,
 // 6 of 4 warps; the batched 4-warp kernel reads its parameters from shared memory and
@@ -127,8 +157,8 @@ __global__ void __launch_bounds__(kWarps * 32, (collide_ctas_per_sm<kBatch, kWar
                    const float* __restrict__ smax_in_all, float* __restrict__ smax_out_all,
                    unsigned long long* __restrict__ ncand_all,
                    unsigned long long* __restrict__ nacc_all, double* __restrict__ acc_all,
-                   int* __restrict__ hist, const InstParams one, const StepLaunch SL,
-                   int* __restrict__ err) {
+                   int* __restrict__ hist, const CellSums sums, const InstParams one,
+                   const StepLaunch SL, int* __restrict__ err) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ InstParams sh_inst;
   // unrolling the per-particle loops helps the single run; the batched kernel, which
@@ -178,12 +208,12 @@ __global__ void __launch_bounds__(kWarps * 32, (collide_ctas_per_sm<kBatch, kWar
   uint64_t* bar = reinterpret_cast<uint64_t*>(wmem + L.w_bar);
 
   const int span = gspan - a.span_base;  // the instance's span
-  const int c0 = span * cps;
-  const int c1 = min(c0 + cps, n_cells);
+  const SpanRange sr = span_range(a, off, span);
+  const int c0 = sr.c0, c1 = sr.c1;
   const unsigned lt = (1u << lane) - 1u;
   // rows (span R + r) of the sort matrix; row r counts the r-th half of the slots
   int* row = hist + a.hist_base + (size_t)span * R * n_cells;
-  const int sb0 = off[c0], sb1 = off[c1];
+  const int sb0 = sr.sb0, sb1 = sr.sb1;
   const int mid = (R > 1) ? sb0 + ((sb1 - sb0) >> 1) : sb1;  // first slot of the second row
   for (int i = threadIdx.x; i < R * n_cells; i += blockDim.x) h[i] = 0;
   // count one particle of slot p in new cell cn
@@ -230,6 +260,10 @@ __global__ void __launch_bounds__(kWarps * 32, (collide_ctas_per_sm<kBatch, kWar
     if (lane == 0) {
       gfirst[c1 - c0] = base;
       cstart[c1 - c0] = off[c1];
+      if (!kBatch && sr.g1 >= 0) {  // a share of one cell: its groups are numbered from g0
+        gfirst[0] = -sr.g0;
+        gfirst[1] = base - sr.g0;
+      }
       *next_group = 0;
     }
   }
@@ -239,7 +273,7 @@ __global__ void __launch_bounds__(kWarps * 32, (collide_ctas_per_sm<kBatch, kWar
     fence_mbar_init();
   }
   __syncthreads();
-  const int n_groups = gfirst[c1 - c0];
+  const int n_groups = !kBatch && sr.g1 >= 0 ? sr.g1 - sr.g0 : gfirst[c1 - c0];
 
   bool bad_bounce = false, cand_fail = false, timeout = false;
   bool inflow_fail = false, mom_range = false;
@@ -422,6 +456,14 @@ __global__ void __launch_bounds__(kWarps * 32, (collide_ctas_per_sm<kBatch, kWar
   __syncthreads();
 
   write_rows();
+  if (!kBatch && sr.g1 >= 0) {  // the cell's other CTAs add theirs; the scan makes the results
+    if (threadIdx.x < 12 && sample && cfix[threadIdx.x + 1])
+      atomicAdd(sums.fix + (size_t)c0 * 12 + threadIdx.x, cfix[threadIdx.x + 1]);
+    if (threadIdx.x == 12 && cgmax[0]) atomicMax(sums.gmax + c0, cgmax[0]);
+    if (threadIdx.x == 13 && ccand[0]) atomicAdd(ncand + c0, ccand[0]);
+    if (threadIdx.x == 14 && caccn[0]) atomicAdd(nacc + c0, caccn[0]);
+    return;
+  }
   for (int c = c0 + threadIdx.x; c < c1; c += blockDim.x) {
     const int lc = c - c0;
     const float gm = __uint_as_float(cgmax[lc]);
@@ -580,9 +622,8 @@ __global__ void __launch_bounds__(kBWarpsMax * 32)
   const int* row = hist + a.hist_base + ((size_t)span * R + sub) * n_cells;
   for (int c = lane; c < n_cells; c += 32) run[c] = off_new[c] + row[c];
   __syncwarp();
-  const int c0 = span * a.cps;
-  const int c1 = min(c0 + a.cps, n_cells);
-  const int sb0 = off_cur[c0], sb1 = off_cur[c1];
+  const SpanRange sr = span_range(a, off_cur, span);
+  const int sb0 = sr.sb0, sb1 = sr.sb1;
   const int mid = (R > 1) ? sb0 + ((sb1 - sb0) >> 1) : sb1;
   const int b0 = (sub == 0) ? sb0 : mid;
   const int b1 = (sub == 0) ? mid : sb1;
@@ -622,9 +663,8 @@ __global__ void __launch_bounds__(kBWarpsMax * 32)
 // that leaves room for 4 CTAs per SM.
 constexpr int kCoopWarps = 8;
 constexpr size_t kCoopSmemMax = 48 * 1024;
-constexpr int kCoopPer =  // cells per thread of the largest instance it serves (1,365)
-    ((int)(kCoopSmemMax / sizeof(int) / (kCoopWarps + 1)) + kCoopWarps * 32 - 1) /
-    (kCoopWarps * 32);
+static_assert(kCoopCells == (int)(kCoopSmemMax / sizeof(int) / (kCoopWarps + 1)), "");
+constexpr int kCoopPer = (kCoopCells + kCoopWarps * 32 - 1) / (kCoopWarps * 32);  // cells per thread
 
 template <bool kBatch, int kSlices>
 __global__ void __launch_bounds__(kCoopWarps * 32)
@@ -684,9 +724,8 @@ __global__ void __launch_bounds__(kCoopWarps * 32)
     // Graph replay: the step's collide/move pass has finished reading the step number.
     if (SL.gstep_dev != nullptr && blockIdx.x == 0 && threadIdx.x == 0) *SL.gstep_dev += 1;
   }
-  const int c0 = span * a.cps;
-  const int c1 = min(c0 + a.cps, n_cells);
-  const int sb0 = off_cur[c0], sb1 = off_cur[c1];
+  const SpanRange sr = span_range(a, off_cur, span);
+  const int sb0 = sr.sb0, sb1 = sr.sb1;
   const int mid = (R > 1) ? sb0 + ((sb1 - sb0) >> 1) : sb1;
   const int b0 = (sub == 0) ? sb0 : mid;
   const int b1 = (sub == 0) ? mid : sb1;
@@ -772,18 +811,48 @@ __global__ void __launch_bounds__(kCoopWarps * 32)
   if (bad) atomicOr(err, kErrSort);
 }
 
-// Per instance and cell c: row r of the sort matrix <- sum over rows r' < r (the spans
-// before), count[c] <- total.  Block (kScanCells, kScanSegs): x = cell
-// within a chunk, y = one of the contiguous row segments; grid (cell chunks, instances).  A chunk
-// of 16 cells reads 64 bytes of a row, two sectors; chunks of 32 would leave 2,000 cells 63 CTAs
-// of twice the rows per thread (20.7 us at 2,000 rows).
-constexpr int kScanCells = 16, kScanSegs = 64;
+// The results of a step in cell c of an instance whose cells are shared by several CTAs
+// (as the one CTA of a cell writes them otherwise).
+__device__ __forceinline__ void finish_cell(const CellSums& S, const InstParams& a,
+                                            const StepLaunch& SL, int c) {
+  if (a.parts == 1 || SL.count_only) return;
+  const long long istep = (SL.gstep_dev ? *SL.gstep_dev : SL.gstep) - a.step0;
+  const float gm = __uint_as_float(S.gmax[c]);
+  S.gmax[c] = 0u;
+  const float sg = (a.mode == 0) ? gm : fmul(a.cvhs, pow32(gm, a.vexp));
+  S.smax_out[c] = fmaxf(S.smax_in[c], sg);
+  if (istep < a.sample_start) return;
+  const int nc = S.off[c + 1] - S.off[c];
+  double* acc = S.acc + (size_t)c * kNMom;
+  acc[0] += (double)nc;
+  const double grid =
+      __longlong_as_double((long long)(1023 - grid_exponent(nc > 0 ? nc : 1)) << 52);
+  unsigned long long* fix = S.fix + (size_t)c * 12;
+  unsigned long long q[12];
+  double sum[12];  // (all loads on their way before the first use)
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    q[k] = fix[k];
+    sum[k] = acc[k + 1];
+  }
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    acc[k + 1] = sum[k] + 0.5 * grid * (double)(long long)q[k];
+    fix[k] = 0ull;
+  }
+}
 
-template <bool kBatch>
-__global__ void __launch_bounds__(kScanCells * kScanSegs)
-    k_scan_spans(int* __restrict__ hist, int* __restrict__ count_all, const InstParams one,
-                 const StepLaunch SL) {
-  __shared__ int seg_tot[kScanSegs][kScanCells + 1];
+// Per instance and cell c: row r of the sort matrix <- sum over rows r' < r (the spans
+// before), count[c] <- total.  Block (kScanCells, 1024 / kScanCells): x = cell
+// within a chunk, y = one of the contiguous row segments; grid (cell chunks, instances).  Chunks
+// of 16 cells (two sectors of a row) give 2,000 cells 125 CTAs instead of 63 of twice the rows
+// per thread (20.7 -> 14 us at 2,000 rows); with 92 chunks of 32 or more their wider rows win
+// (3,900 cells x 1,950 rows, whole step: 547 us against 520).
+template <bool kBatch, int kScanCells>
+__global__ void __launch_bounds__(1024)
+    k_scan_spans(int* __restrict__ hist, int* __restrict__ count_all, const CellSums sums,
+                 const InstParams one, const StepLaunch SL) {
+  __shared__ int seg_tot[(1024 / kScanCells)][kScanCells + 1];
   const InstParams& a = kBatch ? SL.tab[blockIdx.y] : one;
   const int n_cells = a.n_cells;
   if ((int)blockIdx.x * kScanCells >= n_cells) return;
@@ -792,7 +861,7 @@ __global__ void __launch_bounds__(kScanCells * kScanSegs)
   int* __restrict__ count = count_all + a.cell_base;
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int c = blockIdx.x * kScanCells + tx;
-  const int seg = (n_rows + kScanSegs - 1) / kScanSegs;
+  const int seg = (n_rows + (1024 / kScanCells) - 1) / (1024 / kScanCells);
   const int r0 = min(n_rows, ty * seg);
   const int r1 = min(n_rows, r0 + seg);
   int s = 0;
@@ -811,12 +880,15 @@ __global__ void __launch_bounds__(kScanCells * kScanSegs)
   __syncthreads();
   if (ty == 0) {
     int run = 0;
-    for (int k = 0; k < kScanSegs; ++k) {
+    for (int k = 0; k < (1024 / kScanCells); ++k) {
       const int v = seg_tot[k][tx];
       seg_tot[k][tx] = run;
       run += v;
     }
-    if (c < n_cells) count[c] = run;
+    if (c < n_cells) {
+      count[c] = run;
+      if constexpr (!kBatch) finish_cell(sums, a, SL, c);
+    }
   }
   __syncthreads();
   if (c < n_cells) {
@@ -853,8 +925,8 @@ constexpr int kScanColsDepth = 32;
 
 template <bool kBatch>
 __global__ void __launch_bounds__(kScanColsCells)
-    k_scan_cols(int* __restrict__ hist, int* __restrict__ count_all, const InstParams one,
-                const StepLaunch SL) {
+    k_scan_cols(int* __restrict__ hist, int* __restrict__ count_all, const CellSums sums,
+                const InstParams one, const StepLaunch SL) {
   const InstParams& a = kBatch ? SL.tab[blockIdx.y] : one;
   const int n_cells = a.n_cells;
   const int c = blockIdx.x * kScanColsCells + threadIdx.x;
@@ -875,6 +947,7 @@ __global__ void __launch_bounds__(kScanColsCells)
       }
   }
   count_all[a.cell_base + c] = run;
+  if constexpr (!kBatch) finish_cell(sums, a, SL, c);
 }
 
 // Per instance (one CTA each): off_new[c] = first global slot of cell c,
@@ -1016,8 +1089,8 @@ __global__ void k_pack(const float* __restrict__ y, const float* __restrict__ vx
 cudaError_t launch_collide_move(float4* P, const int* off, const float* smax_in,
                                 float* smax_out, unsigned long long* ncand,
                                 unsigned long long* nacc, double* acc, int* hist,
-                                const InstParams& one, const StepLaunch& L, int* err,
-                                cudaStream_t st) {
+                                const CellSums& sums, const InstParams& one,
+                                const StepLaunch& L, int* err, cudaStream_t st) {
   const bool batch = L.n_inst > 1;
   bool small = L.warps == kAWarpsSmall;
   // an 8-warp CTA that fits without the batch's wall queues (as the host checked) but not with
@@ -1030,7 +1103,7 @@ cudaError_t launch_collide_move(float4* P, const int* off, const float* smax_in,
   const dim3 block(warps * 32);
 #define DSMC_COLLIDE(B, W, D)                                                       \
   k_collide_move<B, W, D><<<L.n_spans_total, block, S.total, st>>>(               \
-      P, off, smax_in, smax_out, ncand, nacc, acc, hist, one, L, err)
+      P, off, smax_in, smax_out, ncand, nacc, acc, hist, sums, one, L, err)
 #define DSMC_COLLIDE_SHAPE(B, D)   \
   do {                             \
     if (small)                     \
@@ -1115,27 +1188,31 @@ cudaError_t launch_scatter_spans(const float4* P, float4* P2, const int* off_cur
   return cudaGetLastError();
 }
 
-cudaError_t launch_scan_spans(int* hist, int* count, const InstParams& one, const StepLaunch& L,
-                              cudaStream_t st) {
+cudaError_t launch_scan_spans(int* hist, int* count, const CellSums& sums, const InstParams& one,
+                              const StepLaunch& L, cudaStream_t st) {
   if ((long long)L.max_spans * L.rows <= kScanColsMaxRows) {
     const dim3 grid((L.max_cells + kScanColsCells - 1) / kScanColsCells, L.n_inst);
     if (L.n_inst == 1)
-      k_scan_cols<false><<<grid, kScanColsCells, 0, st>>>(hist, count, one, L);
+      k_scan_cols<false><<<grid, kScanColsCells, 0, st>>>(hist, count, sums, one, L);
     else
-      k_scan_cols<true><<<grid, kScanColsCells, 0, st>>>(hist, count, one, L);
+      k_scan_cols<true><<<grid, kScanColsCells, 0, st>>>(hist, count, sums, one, L);
     return cudaGetLastError();
   }
-  const dim3 grid((L.max_cells + kScanCells - 1) / kScanCells, L.n_inst);
-  const dim3 block(kScanCells, kScanSegs);
-  if (L.n_inst == 1)
-    k_scan_spans<false><<<grid, block, 0, st>>>(hist, count, one, L);
-  else
-    k_scan_spans<true><<<grid, block, 0, st>>>(hist, count, one, L);
+  const bool wide = L.max_cells >= 92 * 32;
+  const int cells = wide ? 32 : 16;
+  const dim3 grid((L.max_cells + cells - 1) / cells, L.n_inst), block(cells, 1024 / cells);
+#define DSMC_SCAN(B, C) k_scan_spans<B, C><<<grid, block, 0, st>>>(hist, count, sums, one, L)
+  if (L.n_inst == 1) {
+    if (wide) DSMC_SCAN(false, 32); else DSMC_SCAN(false, 16);
+  } else {
+    if (wide) DSMC_SCAN(true, 32); else DSMC_SCAN(true, 16);
+  }
+#undef DSMC_SCAN
   return cudaGetLastError();
 }
 
 bool scatter_forms_offsets(const StepLaunch& L) {
-  return scatter_coop_smem(L.max_cells) <= kCoopSmemMax;
+  return L.max_cells <= kCoopCells;
 }
 
 cudaError_t launch_offsets_cells(const int* count, int* off_new, const InstParams& one,

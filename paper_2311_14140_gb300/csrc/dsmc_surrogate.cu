@@ -574,9 +574,10 @@ static dsmc_status create_surrogate(double Kn, double F, int n_cells, int ppc, d
   else
     dsmc_surrogate_exponents(Kn, s->b);
   const size_t nc = (size_t)n_cells;
-  cudaError_t e = cudaMalloc(&s->stats, kStats * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&s->window, nc * dsmc::kNMom * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&s->basis, (4 * nc + 6) * sizeof(double));
+  // one allocation: statistics, the window's copy and the basis
+  cudaError_t e = cudaMalloc(&s->stats, (kStats + (dsmc::kNMom + 4) * nc + 6) * sizeof(double));
+  s->window = s->stats + kStats;
+  s->basis = s->window + dsmc::kNMom * nc;
   if (e == cudaSuccess) e = cudaMemsetAsync(s->stats, 0, kStats * sizeof(double), s->stream);
   if (e == cudaSuccess) {
     k_basis<<<1, kThreads, 0, s->stream>>>(window_args(s, 1), s->basis, s->basis + 3 * nc);
@@ -606,9 +607,7 @@ dsmc_status dsmc_surrogate_create_region(double Kn, double F, int n_cells, int p
 dsmc_status dsmc_surrogate_destroy(dsmc_surrogate_handle s) {
   if (!s) return DSMC_OK;
   cudaStreamSynchronize(s->stream);
-  cudaFree(s->stats);
-  cudaFree(s->window);
-  cudaFree(s->basis);
+  cudaFree(s->stats);  // (and the window and the basis)
   cudaFree(s->trials);
   delete s;
   return DSMC_OK;
