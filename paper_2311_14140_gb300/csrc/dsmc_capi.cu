@@ -83,9 +83,9 @@ void make_spans(int n_cells, int ppc, int target, int* cps, int* n_spans) {
 
 // Spans per cell of one run with few, populous cells: a cell is then shared by several CTAs, so
 // that the run still makes about kPartSpans spans, of about kPartMin particles or more (16
-// collision groups of 256 for a CTA's 8 warps).  us per step, whole cells -> shared: 200 x 50,000 425 ->
-// 186, 100 x 25,000 195 -> 76, 20 x 100,000 587 -> 65, 300 x 6,666 90 -> 69, 700 x 25,000 366 ->
-// 314.  From about 320 cells on the whole cells of less than 10,000 particles keep most places
+// collision groups of 256 for a CTA's 8 warps).  us per step, whole cells -> shared: 200 x 50,000 465 ->
+// 191, 100 x 25,000 215 -> 79, 20 x 100,000 610 -> 63, 300 x 6,666 89 -> 68, 700 x 25,000 362 ->
+// 312.  From about 320 cells on the whole cells of less than 10,000 particles keep most places
 // on the SMs busy, and the larger sort matrix and the sums cost more than sharing gives (400 x
 // 5,000 101 -> 113 at Kn = 6, 860 x 9,302 175 -> 176).
 constexpr int kPartSpans = 900, kPartMin = 4096, kPartCells = 320, kPartLarge = 10000;
@@ -96,6 +96,13 @@ int cell_parts(int n_cells, int ppc) {
   const long long t = std::max<long long>(kPartMin, N / kPartSpans);
   return (int)std::max<long long>(1, (ppc + t - 1) / t);
 }
+
+// Whole cells that fill one wave of 8-warp CTAs, three per SM, to 4/5 or more leave few places
+// idle and stay whole: shares of them cost a second and third wave where walls or collisions
+// make the groups long (440 x 10,000, whole / shared us per step: Kn = 3 125 / 152, Kn = 6 161 /
+// 186, Kn = 0.1 124 / 111; 350 x 10,000: 123 / 125, 151 / 150, 120 / 93; 470 x 10,000, just over
+// the wave: 162 / 158, 201 / 194, 128 / 115).
+bool fills_wave(int n_cells, int sms) { return n_cells <= 3 * sms && 5 * n_cells >= 12 * sms; }
 
 // Parameters of the method in binary64, rounded once to binary32 where the kernels
 // use them.
@@ -552,7 +559,9 @@ void set_partition(dsmc_sim* h, int target) {
     Inst& x = h->inst[h->order[t]];
     np += x.N;
     make_spans(x.n_cells, x.ppc, target, &x.cps, &x.n_spans);
-    x.parts = h->auto_split && !h->pool && h->C.inst == 1 ? cell_parts(x.n_cells, x.ppc) : 1;
+    x.parts = h->auto_split && !h->pool && h->C.inst == 1 && !fills_wave(x.n_cells, h->sms)
+                  ? cell_parts(x.n_cells, x.ppc)
+                  : 1;
     if (x.parts > 1) {
       x.cps = 1;
       x.n_spans = x.n_cells * x.parts;

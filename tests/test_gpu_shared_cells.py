@@ -73,3 +73,21 @@ def test_shared_cells_under_graph_replay():
     for d in runs:
         d.step(37)
     _same(runs)
+
+
+def test_cells_that_fill_a_wave_stay_whole():
+    """Both ends of the range of cell counts whose whole cells fill three CTAs per SM."""
+    import torch
+
+    from paper_2311_14140_gb300 import Dsmc
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    lo, hi = -(-12 * sms // 5), 3 * sms
+    for n, whole in ((lo - 1, False), (lo, True), (hi, True), (hi + 1, False)):
+        kw = dict(Kn=0.3, n_cells=n, ppc=10000, omega=0.81, seed=4, profile=True)
+        runs = [Dsmc(**kw), Dsmc(span_particles=4096, **kw)]
+        assert (runs[0].info()["n_spans"] == n) is whole
+        for d in runs:
+            d.step(2)
+        _same(runs)
+        for d in runs:
+            d.close()
