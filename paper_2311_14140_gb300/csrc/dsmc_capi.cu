@@ -600,15 +600,24 @@ void choose_split(dsmc_sim* h) {
       long long target;
       if (x.n_cells > kCoopCells) {
         // a scatter with a warp per span wants about 6.6 of them per SM (3,000 x 500: 334 spans
-        // 106 us per step, 1,000 spans 64; 4,000 x 1,500: 1,334 spans 196, 1,000 spans 185)
-        target = std::min<long long>(5120, x.N / (33LL * h->sms / 5));
+        // 106 us per step, 1,000 spans 64); beyond 4,096 particles whole cells up to 6,144 (4,000
+        // x 1,500: 1,334 spans 196, 1,000 spans 185), but no cell more (1,600 x 5,000: 1,600
+        // spans 182, 800 spans 199)
+        const long long t = x.N / (33LL * h->sms / 5);
+        const long long k = std::max((std::min<long long>(4096, t) + x.ppc - 1) / x.ppc,
+                                     std::min<long long>(6144, t) / x.ppc);
+        target = k * x.ppc;
       } else {
-        // whole cells, nearest to 4,096 particles or to one span per place of an 8-warp CTA on
-        // the SMs, rather more than less (600 x 3,500: 300 spans 82 us per step, 600 spans 65;
-        // 1,000 x 2,000: 334 spans 82, 500 spans 70; 700 x 2,857 at Kn = 6: 350 spans 104, 700
-        // spans 115)
-        const long long t = std::min<long long>(kDefaultSpanParticles, x.N / (3LL * h->sms));
-        target = std::max<long long>(1, (10 * t + 6LL * x.ppc) / (10LL * x.ppc)) * x.ppc;
+        // whole cells: the fewest per span whose spans fit 1.2 waves of 8-warp CTAs, three per
+        // SM, and no more than the default's particles need; the few CTAs behind a full wave have
+        // the SMs to themselves and cost little, half a wave more does not (us per step at Kn 2,
+        // cells per span 1 / 2 / 3: 500 x 3,500 71 / 85 / 113, 1,000 x 3,000 111 / 105 / 112,
+        // 800 x 3,000 95 / 83 / 99, 700 x 2,000 68 / 68 / 78; 1,300 x 2,000 107 / 108 / 88)
+        const long long most =
+            std::max<long long>(1, (default_span_particles(x.N) + x.ppc - 1) / x.ppc);
+        long long k = 1;
+        while (k < most && 5 * ((x.n_cells + k - 1) / k) > 18LL * h->sms) ++k;
+        target = k * x.ppc;
       }
       h->span_target = (int)std::min<long long>(kMaxSpanParticles,
                                                 std::max<long long>(kMinSpanParticles, target));
