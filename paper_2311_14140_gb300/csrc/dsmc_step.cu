@@ -848,8 +848,10 @@ __device__ __forceinline__ void finish_cell(const CellSums& S, const InstParams&
 // before), count[c] <- total.  Block (kScanCells, 1024 / kScanCells): x = cell
 // within a chunk, y = one of the contiguous row segments; grid (cell chunks, instances).  Chunks
 // of 16 cells (two sectors of a row) give 2,000 cells 125 CTAs instead of 63 of twice the rows
-// per thread (20.7 -> 14 us at 2,000 rows); with 92 chunks of 32 or more their wider rows win
-// (3,900 cells x 1,950 rows, whole step: 547 us against 520).
+// per thread (20.7 -> 14 us at 2,000 rows).  They are taken while they fit one wave of CTAs (2,800
+// cells x 934 rows: 16-cell chunks 15.8 us, 32 cells 12.5; 2,400 x 1,200: 12.4, 14.3) and do not
+// straddle sectors, or the rows are short (1,403 x 1,403: 23.3, 18.7; 2,900 x 1,450: 37.9, 21.4;
+// but 1,001 x 1,001: 10.2, 12.4).
 template <bool kBatch, int kScanCells>
 __global__ void __launch_bounds__(1024)
     k_scan_spans(int* __restrict__ hist, int* __restrict__ count_all, const CellSums sums,
@@ -1200,7 +1202,7 @@ cudaError_t launch_scan_spans(int* hist, int* count, const CellSums& sums, const
       k_scan_cols<true><<<grid, kScanColsCells, 0, st>>>(hist, count, sums, one, L);
     return cudaGetLastError();
   }
-  const bool wide = L.max_cells >= 92 * 32;
+  const bool wide = L.max_cells > 16 * 152 || (L.max_cells > 1200 && L.max_cells % 16 != 0);
   const int cells = wide ? 32 : 16;
   const dim3 grid((L.max_cells + cells - 1) / cells, L.n_inst), block(cells, 1024 / cells);
 #define DSMC_SCAN(B, C) k_scan_spans<B, C><<<grid, block, 0, st>>>(hist, count, sums, one, L)
