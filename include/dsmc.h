@@ -105,9 +105,9 @@ typedef struct dsmc_options {
                              dsmc_step synchronises at its end); default 0 */
   int span_particles;     /* particles per span (CTA) of the step passes at the
                              initial density: 0 leaves the partition to the library
-                             (one run: 4096, or fewer down to 1024 when it holds less
-                             than two such spans per SM, and several spans per cell
-                             when there would be too few to fill the SMs; batches and
+                             (one run: 4096 to 6144, fewer when its spans then fill
+                             the SMs better, down to 1024 or one cell, and several
+                             spans per cell when there would be too few; batches and
                              pools: 1024 to 8192 by the particles of the active
                              instances; or what dsmc_autotune chose, or an earlier
                              value), else 1024..2^24.

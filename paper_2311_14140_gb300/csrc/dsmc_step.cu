@@ -21,8 +21,9 @@
 //                         in place and count its new cell in the CTA's histogram.
 //                    The histogram becomes the span's row of the sort matrix.  Per-cell
 //                    (sigma g)_max, collision counters and moment sums are written by
-//                    the one CTA that owns the cell.  With `count_only` the pass just
-//                    counts cells of the span's slots (the sort into cells at creation
+//                    the one CTA that owns the cell; where several CTAs share a cell they
+//                    add integers into CellSums and the scan writes the results.  With
+//                    `count_only` the pass just counts cells of the span's slots (the sort into cells at creation
 //                    and after a state load).
 //   k_scatter_spans  one warp per span: re-reads the records in slot order, 16 per lane
 //                    in flight, ranks each record among the same-cell records before it
