@@ -607,6 +607,12 @@ void choose_split(dsmc_sim* h) {
         const long long k = std::max((std::min<long long>(4096, t) + x.ppc - 1) / x.ppc,
                                      std::min<long long>(6144, t) / x.ppc);
         target = k * x.ppc;
+        // more than two and less than three spans per SM are a second wave of few CTAs (so many
+        // cells' histograms leave room for two per SM): the default's two then (3,500 x 113: 292
+        // spans 45 us per step, 350 spans 49; 3,996 x 200: 286 spans 65, 666 spans 59)
+        const long long c = std::max<long long>(k, kMinSpanParticles / x.ppc);
+        const long long spans = x.n_cells / std::max<long long>(1, c);
+        if (spans >= 2LL * h->sms && spans < 3LL * h->sms) target = default_span_particles(x.N);
       } else {
         // whole cells: the fewest per span whose spans fit 1.2 waves of 8-warp CTAs, three per
         // SM, and no more than the default's particles need; the few CTAs behind a full wave have
