@@ -121,7 +121,7 @@ typedef struct dsmc_options {
                              default 0 */
   int cta_warps;          /* warps per CTA of the collide/move pass: 0 keeps the shape
                              in use (one run: 8; batches and pools: 8, or 4 from about
-                             46,000 particles per SM on; or what dsmc_autotune chose,
+                             27,000 particles per SM on; or what dsmc_autotune chose,
                              or an earlier value), else 4 or 8; results are identical;
                              default 0 */
   int span_rows;          /* sort-matrix rows per span, one per equal part of its

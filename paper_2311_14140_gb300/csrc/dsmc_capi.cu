@@ -586,13 +586,14 @@ void set_partition(dsmc_sim* h, int target) {
 int default_span_particles(long long n);
 
 // Warps per CTA and particles per span for the active instances of a batch or pool, by their
-// particles (us per step of pools of uneven instances; in brackets the former 4-warp CTAs of
-// 4,096 particles): below 46,000 particles per SM 8-warp CTAs (fewer, larger CTAs leave fewer
-// SMs idle behind the last spans) with spans that give every place on the SMs about one, 1,024
-// to 8,192 particles (0.94 million particles 55 [74], 2.9 million 101 [116], 4.1 million 133
-// [137], 6.9 million 208 [209]); from there 4-warp CTAs with 5,120 (8.9 million 260 [267], 15.8
-// million 433 [452]), from 120,000 per SM on 8,192 (24 million 657 [692]).  One run of its own
-// keeps 8 warps and default_span_particles.
+// particles (us per step of batches of uneven instances; in brackets the former 4-warp CTAs of
+// 4,096 particles, then 8-warp CTAs of 4,096 / 6,144 and 4-warp CTAs of 4,096 / 5,120 where they
+// lose): below 27,000 particles per SM 8-warp CTAs (fewer, larger CTAs leave fewer SMs idle behind
+// the last spans) with spans of 1,024 to 4,096 particles, about one per place on the SMs (1.2
+// million 68 [80], 2.8 million 115 [119], 3.6 million 142 [150; 4-warp 157]); from there 4-warp
+// CTAs of 4,096 (4.4 million 154 [167; 8-warp 162 / 161],
+// 5.2 million 176 [194; 8-warp 188 / 185]), from 40,000 per SM on 5,120 (6.3 million 209 [232;
+// 4,096 215], 8.5 million 270 [316]), from 120,000 per SM on 8,192 (24 million 657 [692]).
 void choose_split(dsmc_sim* h) {
   if (!h->pool && h->n_inst() <= 1) {
     if (h->n_inst() == 1) {
@@ -634,10 +635,10 @@ void choose_split(dsmc_sim* h) {
   for (int id : h->order) n += h->inst[id].N;
   int warps = kAWarps;
   long long target =
-      std::min<long long>(8192, std::max<long long>(kMinSpanParticles, 2 * n / (7LL * h->sms)));
-  if (n >= 46000LL * h->sms) {
+      std::min<long long>(4096, std::max<long long>(kMinSpanParticles, 2 * n / (7LL * h->sms)));
+  if (n >= 27000LL * h->sms) {
     warps = kAWarpsSmall;
-    target = n >= 120000LL * h->sms ? 8192 : 5120;
+    target = n >= 120000LL * h->sms ? 8192 : n >= 40000LL * h->sms ? 5120 : 4096;
   }
   int mcps, mcells;
   partition_extent(h, (int)target, nullptr, &mcps, &mcells);
