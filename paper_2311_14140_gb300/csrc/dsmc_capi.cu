@@ -1893,25 +1893,27 @@ dsmc_status dsmc_copy_cells_of(dsmc_handle h, int id, int* offset, float* smax,
   std::vector<char> host(B.total);
   DSMC_CUDA(cudaMemcpyAsync(host.data(), block, B.total, cudaMemcpyDeviceToHost, st),
             "copy cells");
-  DSMC_CUDA(cudaStreamSynchronize(st), "stream sync");
-  if ((s = collect_times(h)) != DSMC_OK) return s;
   struct {
     void* to;
     size_t at, bytes;
-  } const parts[4] = {{offset, B.offset, (nc + 1) * sizeof(int)},
-                      {smax, B.smax, nc * sizeof(float)},
-                      {ncand, B.ncand, nc * 8},
-                      {nacc, B.nacc, nc * 8}};
-  for (const auto& q : parts) {
+  } parts[4] = {{offset, B.offset, (nc + 1) * sizeof(int)},
+                {smax, B.smax, nc * sizeof(float)},
+                {ncand, B.ncand, nc * 8},
+                {nacc, B.nacc, nc * 8}};
+  // Device (and managed) arrays get theirs from the block on the handle's stream, like every
+  // other result; host arrays from its host copy.
+  for (auto& q : parts) {
     if (!q.to) continue;
     cudaPointerAttributes at{};
     if (cudaPointerGetAttributes(&at, q.to) != cudaSuccess) cudaGetLastError();
-    if (at.type == cudaMemoryTypeDevice)
-      DSMC_CUDA(cudaMemcpy(q.to, host.data() + q.at, q.bytes, cudaMemcpyHostToDevice),
-                "copy cells");
-    else
-      std::memcpy(q.to, host.data() + q.at, q.bytes);
+    if (at.type != cudaMemoryTypeDevice && at.type != cudaMemoryTypeManaged) continue;
+    DSMC_CUDA(cudaMemcpyAsync(q.to, block + q.at, q.bytes, cudaMemcpyDefault, st), "copy cells");
+    q.to = nullptr;
   }
+  DSMC_CUDA(cudaStreamSynchronize(st), "stream sync");
+  if ((s = collect_times(h)) != DSMC_OK) return s;
+  for (const auto& q : parts)
+    if (q.to) std::memcpy(q.to, host.data() + q.at, q.bytes);
   int v = 0;
   std::memcpy(&v, host.data() + B.err, sizeof(int));
   return check_error_word(h, v);

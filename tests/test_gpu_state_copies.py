@@ -80,3 +80,34 @@ def test_cells_into_device_memory():
     np.testing.assert_array_equal(t[3].numpy(), nacc.astype(np.int64))
     _check(d._lib.dsmc_copy_cells(d._h, None, None, None, None))
     d.close()
+
+
+def test_cells_into_device_memory_on_the_runs_stream():
+    """Device arrays are written on the run's own stream and complete on return: a reader on that
+    (non-blocking) stream finds them, and work on the default stream is not waited for."""
+    import torch
+
+    from paper_2311_14140_gb300 import Dsmc
+    from paper_2311_14140_gb300.dsmc import _check
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        d = Dsmc(0.5, N_CELLS, PPC, omega=0.81, body_force=1e-2, seed=3)
+        d.step(5)
+        want = d.cells()
+        t = [torch.zeros(N_CELLS + 1, dtype=torch.int32, device="cuda"),
+             torch.zeros(N_CELLS, device="cuda"),
+             torch.zeros(N_CELLS, dtype=torch.int64, device="cuda"),
+             torch.zeros(N_CELLS, dtype=torch.int64, device="cuda")]
+        s.synchronize()
+    busy = torch.cuda.Event()
+    torch.cuda._sleep(2_000_000_000)  # about a second on the default stream
+    busy.record()
+    _check(d._lib.dsmc_copy_cells(d._h, *[ctypes.c_void_p(x.data_ptr()) for x in t]))
+    with torch.cuda.stream(s):
+        got = [x.to("cpu") for x in t]
+    waited = busy.query()
+    torch.cuda.synchronize()
+    for g, w in zip(got, want):
+        np.testing.assert_array_equal(g.numpy(), w.astype(g.numpy().dtype))
+    assert not waited
+    d.close()
