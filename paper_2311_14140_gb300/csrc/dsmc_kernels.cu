@@ -27,30 +27,31 @@ namespace dsmc {
 constexpr unsigned kFull = 0xffffffffu;
 
 // ---------------------------------------------------------------------------
-// Initial state, as float4 records (y, vx, vy, vz).
+// Initial state, as float4 records (y, vx, vy, vz).  A thread per record and no stride over the
+// grid: from 2^30 records on, a record's index plus the grid's size passes 2^31.
 __global__ void k_init(float4* __restrict__ P, int N, int ppc, float ncf, uint32_t k0,
                        uint32_t k1, int* __restrict__ err) {
-  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < N; p += gridDim.x * blockDim.x) {
-    const int c = p / ppc;
-    const uint32_t c3 = kStreamInit << 24;
-    U4 w = philox((uint32_t)p, 0u, 0u, c3, k0, k1);
-    const float y = fdiv(fadd((float)c, u01(w.x)), ncf);
-    float z[3];
-    int have = 0;
-    for (int a = 0; a < kNormalAttempts && have < 3; ++a) {
-      if ((a & 1) == 0) w = philox((uint32_t)p, 1u + (uint32_t)(a >> 1), 0u, c3, k0, k1);
-      float z0, z1;
-      const bool ok = (a & 1) ? polar_pair(w.z, w.w, z0, z1) : polar_pair(w.x, w.y, z0, z1);
-      if (!ok) continue;
-      z[have++] = z0;
-      if (have < 3) z[have++] = z1;
-    }
-    if (have < 3) {
-      atomicOr(err, kErrNormals);
-      for (int i = have; i < 3; ++i) z[i] = 0.0f;
-    }
-    P[p] = make_float4(y, z[0], z[1], z[2]);
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= N) return;
+  const int c = p / ppc;
+  const uint32_t c3 = kStreamInit << 24;
+  U4 w = philox((uint32_t)p, 0u, 0u, c3, k0, k1);
+  const float y = fdiv(fadd((float)c, u01(w.x)), ncf);
+  float z[3];
+  int have = 0;
+  for (int a = 0; a < kNormalAttempts && have < 3; ++a) {
+    if ((a & 1) == 0) w = philox((uint32_t)p, 1u + (uint32_t)(a >> 1), 0u, c3, k0, k1);
+    float z0, z1;
+    const bool ok = (a & 1) ? polar_pair(w.z, w.w, z0, z1) : polar_pair(w.x, w.y, z0, z1);
+    if (!ok) continue;
+    z[have++] = z0;
+    if (have < 3) z[have++] = z1;
   }
+  if (have < 3) {
+    atomicOr(err, kErrNormals);
+    for (int i = have; i < 3; ++i) z[i] = 0.0f;
+  }
+  P[p] = make_float4(y, z[0], z[1], z[2]);
 }
 
 // Flight (optional), cell index and a warp-private histogram over the warp's span of

@@ -1046,17 +1046,18 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// Records <-> four arrays (y, vx, vy, vz), for the state accessors.
+// Records <-> four arrays (y, vx, vy, vz), for the state accessors.  A thread per record and no
+// stride over the grid: from 2^30 records on, a record's index plus the grid's size passes 2^31.
 __global__ void k_unpack(const float4* __restrict__ P, float* __restrict__ y,
                          float* __restrict__ vx, float* __restrict__ vy, float* __restrict__ vz,
                          int N) {
-  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < N; p += gridDim.x * blockDim.x) {
-    const float4 r = P[p];
-    if (y) y[p] = r.x;
-    if (vx) vx[p] = r.y;
-    if (vy) vy[p] = r.z;
-    if (vz) vz[p] = r.w;
-  }
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= N) return;
+  const float4 r = P[p];
+  if (y) y[p] = r.x;
+  if (vx) vx[p] = r.y;
+  if (vy) vy[p] = r.z;
+  if (vz) vz[p] = r.w;
 }
 
 // An instance's cell data (offsets relative to its first slot) and the error word in one block.
@@ -1082,11 +1083,11 @@ __global__ void k_gather_cells(const int* __restrict__ off, int base,
 __global__ void k_pack(const float* __restrict__ y, const float* __restrict__ vx,
                        const float* __restrict__ vy, const float* __restrict__ vz,
                        float4* __restrict__ P, int N) {
-  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < N; p += gridDim.x * blockDim.x) {
-    const float v = y[p];
-    const float yc = (v >= 0.0f) ? ((v <= 1.0f) ? v : 1.0f) : 0.0f;
-    P[p] = make_float4(yc, vx[p], vy[p], vz[p]);
-  }
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= N) return;
+  const float v = y[p];
+  const float yc = (v >= 0.0f) ? ((v <= 1.0f) ? v : 1.0f) : 0.0f;
+  P[p] = make_float4(yc, vx[p], vy[p], vz[p]);
 }
 
 // ---------------------------------------------------------------------------
