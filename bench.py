@@ -408,7 +408,7 @@ def run_precision(steps: int) -> dict:
     rel = np.abs(m32 - m64) / scale
     return {"sampled_steps": steps,
             "fp32": {"ms_per_step": ms[0], "accum": "binary32 per-lane sums (default)"},
-            "fp64": {"ms_per_step": ms[1], "accum": "binary64 per-lane sums"},
+            "fp64": {"ms_per_step": ms[1], "accum": "binary64-grade per-lane sums (triples of binary32)"},
             "fp32_vs_fp64_max_rel": float(rel.max()),
             "fp32_vs_fp64_max_rel_by_degree": {str(d): float(rel[:, deg == d].max())
                                                for d in (0, 1, 2, 3)}}

@@ -86,9 +86,10 @@ typedef enum dsmc_status {
  *     28 roundings of relative size 2^-24 on partial sums bounded by the sum of
  *     |products|.  The default.
  *   DSMC_ACCUM_FP64: every product is rounded to binary32 (as a plain CPU DSMC forms
- *     it); a group's products are added with the rounding error of every addition kept
- *     (pairs of binary32, 48 bits), within 2^-40 of the sum of |products| and far inside
- *     the cell's grid; binary64 from the group totals on. */
+ *     it); a group's products are added with the rounding errors of the additions kept
+ *     (triples of binary32): the total is within 2^-52 of the sum of |products|, closer
+ *     than binary64 additions in the same order are bound to be; binary64 from the group
+ *     totals on. */
 typedef enum dsmc_accum { DSMC_ACCUM_FP32 = 0, DSMC_ACCUM_FP64 = 1 } dsmc_accum;
 
 /* Options.  Get the defaults from dsmc_default_options and change fields. */

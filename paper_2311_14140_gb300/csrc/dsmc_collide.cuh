@@ -83,14 +83,15 @@ __device__ __forceinline__ void direction_of(uint32_t w0, uint32_t w1, float& nx
 // LaneSums<float>: the products of the binary32 velocities summed in binary32, the
 // second and third moments by fused multiply-add (one rounding per term).
 // LaneSums<double> (DSMC_ACCUM_FP64): every product rounded to binary32 exactly as the
-// oracle forms it, then summed with its rounding errors kept, as pairs of binary32.  A
-// group's total, before it is rounded to its cell's grid (fixed_of), is then within 2^-40 of
-// the sum of |products| (48 terms per lane), against grid steps of 2^-27 at 25,000 particles
-// per cell and 2^-35 at 50: against exact sums of known velocities (50 to 25,000 particles
-// per cell) the results' error is that of binary64 additions to every digit compared
-// (rms 6.8e-14 to 1.7e-12 of the sum of |products|), because the grid makes it.  The GB300
-// makes 2 binary64 additions per clock and SM against 128 in binary32: a step of 5,000,000
-// particles took 0.678 ms with them and takes 0.161 ms (0.128 with LaneSums<float>).
+// oracle forms it, then summed as an unevaluated triple of binary32 (hi, mid, lo): the rounding
+// errors of the additions to hi go to mid, those of the additions to mid to lo.  With u = 2^-24
+// and k products per lane (48 at most), |mid| <= k u S and |lo| <= k^2 u^2 S, S the sum of
+// |products|, so the additions to lo lose at most k^3 u^3 S < 2^-55 S; binary64 additions lose up
+// to k 2^-53 S.  (A pair without lo loses k^2 / 2 u^2 S, 2^-38 S: 2^-47 S seen with magnitudes
+// spread over 2^14, where binary64 loses 2^-52 S and the cell's grid is 2^-55 S.)  The GB300 makes
+// 2 binary64 additions per clock and SM against 128 in binary32: a step of 1,000 cells x 5,003
+// (Kn = 0.1) took 0.678 ms with them, takes 0.184 ms (0.151 with pairs, 0.120 with
+// LaneSums<float>).
 template <typename T>
 struct LaneSums;
 
@@ -133,9 +134,7 @@ struct LaneSums<float> {
   }
 };
 
-// Exact sums of binary32 values as unevaluated pairs hi + lo, two sums at a time: Knuth's
-// two-sum gives the rounding error of every addition to hi exactly, and lo collects the
-// errors (in binary32: they are 2^-24 of hi, so the pair carries 48 bits).
+// Two sums at a time, in packed binary32 operations.
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) {
   float2 r;
   asm("sub.rn.f32x2 %0, %1, %2;"
@@ -145,23 +144,27 @@ __device__ __forceinline__ float2 sub2(float2 a, float2 b) {
   return r;
 }
 
-struct Pair2 {
-  float2 hi, lo;
+// s = a + b rounded, and its rounding error exactly (Knuth's two-sum).
+__device__ __forceinline__ float2 two_sum2(float2 a, float2 b, float2& s) {
+  s = __fadd2_rn(a, b);
+  const float2 t = sub2(s, a);
+  return __fadd2_rn(sub2(a, sub2(s, t)), sub2(b, t));
+}
+
+struct Triple2 {
+  float2 hi, mid, lo;
   __device__ __forceinline__ void add(float2 p) {
-    const float2 s = __fadd2_rn(hi, p);
-    const float2 t = sub2(s, hi);
-    const float2 e = __fadd2_rn(sub2(hi, sub2(s, t)), sub2(p, t));
-    lo = __fadd2_rn(lo, e);
-    hi = s;
+    const float2 e = two_sum2(hi, p, hi);
+    lo = __fadd2_rn(lo, two_sum2(mid, e, mid));
   }
 };
 
 template <>
 struct LaneSums<double> {
-  Pair2 a, b, c, d, e, f;  // the same places as in LaneSums<float>
+  Triple2 a, b, c, d, e, f;  // the same places as in LaneSums<float>
   __device__ __forceinline__ void zero() {
     const float2 z = make_float2(0.0f, 0.0f);
-    a = b = c = d = e = f = Pair2{z, z};
+    a = b = c = d = e = f = Triple2{z, z, z};
   }
   // (the products by scalar multiplications: a packed product followed by a packed addition
   // was contracted, which adds the exact product instead of the rounded one)
@@ -175,32 +178,46 @@ struct LaneSums<double> {
     e.add(make_float2(fmul(y, z), fmul(z, v2)));
     f.add(make_float2(fmul(x, v2), fmul(y, v2)));
   }
-  // moment k as its pair (hi, lo), in the order of LaneSums<float>::get
-  __device__ __forceinline__ float2 get(int k) const {
+  static __device__ __forceinline__ float3 first(const Triple2& t) {
+    return make_float3(t.hi.x, t.mid.x, t.lo.x);
+  }
+  static __device__ __forceinline__ float3 second(const Triple2& t) {
+    return make_float3(t.hi.y, t.mid.y, t.lo.y);
+  }
+  // moment k as its triple (hi, mid, lo), in the order of LaneSums<float>::get
+  __device__ __forceinline__ float3 get(int k) const {
     switch (k) {
-      case 1: return make_float2(a.hi.x, a.lo.x);
-      case 2: return make_float2(a.hi.y, a.lo.y);
-      case 3: return make_float2(b.hi.x, b.lo.x);
-      case 4: return make_float2(c.hi.x, c.lo.x);
-      case 5: return make_float2(c.hi.y, c.lo.y);
-      case 6: return make_float2(b.hi.y, b.lo.y);
-      case 7: return make_float2(d.hi.x, d.lo.x);
-      case 8: return make_float2(d.hi.y, d.lo.y);
-      case 9: return make_float2(e.hi.x, e.lo.x);
-      case 10: return make_float2(f.hi.x, f.lo.x);
-      case 11: return make_float2(f.hi.y, f.lo.y);
-      case 12: return make_float2(e.hi.y, e.lo.y);
-      default: return make_float2(0.0f, 0.0f);
+      case 1: return first(a);
+      case 2: return second(a);
+      case 3: return first(b);
+      case 4: return first(c);
+      case 5: return second(c);
+      case 6: return second(b);
+      case 7: return first(d);
+      case 8: return second(d);
+      case 9: return first(e);
+      case 10: return first(f);
+      case 11: return second(f);
+      case 12: return second(e);
+      default: return make_float3(0.0f, 0.0f, 0.0f);
     }
   }
 };
 
-// Sum of two pairs: two-sum of the high parts, the errors collected in the low part.
-__device__ __forceinline__ float2 pair_sum(float2 a, float2 b) {
-  const float s = fadd(a.x, b.x);
-  const float t = fsub(s, a.x);
-  const float e = fadd(fsub(a.x, fsub(s, t)), fsub(b.x, t));
-  return make_float2(s, fadd(fadd(a.y, b.y), e));
+// The same for one sum.
+__device__ __forceinline__ float two_sum(float a, float b, float& s) {
+  s = fadd(a, b);
+  const float t = fsub(s, a);
+  return fadd(fsub(a, fsub(s, t)), fsub(b, t));
+}
+
+// Sum of two triples.
+__device__ __forceinline__ float3 triple_sum(float3 a, float3 b) {
+  float hi, m0, mid;
+  const float e = two_sum(a.x, b.x, hi);
+  const float f = two_sum(a.y, b.y, m0);
+  const float g = two_sum(m0, e, mid);
+  return make_float3(hi, mid, fadd(fadd(a.z, b.z), fadd(f, g)));
 }
 
 // Warp sum of a group's lane sums by a transposing butterfly over 16 slots (moments
@@ -227,26 +244,27 @@ __device__ __forceinline__ float group_total(const LaneSums<float>& m, int lane)
   return v[0] + __shfl_xor_sync(kFull, v[0], 1);
 }
 
-// The same for pairs; the pair's value in binary64.
+// The same for triples; the triple's value in binary64.
 __device__ __forceinline__ double group_total(const LaneSums<double>& m, int lane) {
-  float2 v[16];
+  float3 v[16];
 #pragma unroll
   for (int k = 0; k < 16; ++k) v[k] = m.get(k);
-  auto other = [](float2 x, int mask) {
-    return make_float2(__shfl_xor_sync(kFull, x.x, mask), __shfl_xor_sync(kFull, x.y, mask));
+  auto other = [](float3 x, int mask) {
+    return make_float3(__shfl_xor_sync(kFull, x.x, mask), __shfl_xor_sync(kFull, x.y, mask),
+                       __shfl_xor_sync(kFull, x.z, mask));
   };
 #pragma unroll
   for (int half = 8, mask = 16; half >= 1; half >>= 1, mask >>= 1) {
     const bool upper = (lane & mask) != 0;
 #pragma unroll
     for (int k = 0; k < half; ++k) {
-      const float2 send = upper ? v[k] : v[k + half];
-      const float2 keep = upper ? v[k + half] : v[k];
-      v[k] = pair_sum(keep, other(send, mask));
+      const float3 send = upper ? v[k] : v[k + half];
+      const float3 keep = upper ? v[k + half] : v[k];
+      v[k] = triple_sum(keep, other(send, mask));
     }
   }
-  const float2 s = pair_sum(v[0], other(v[0], 1));
-  return (double)s.x + (double)s.y;
+  const float3 s = triple_sum(v[0], other(v[0], 1));
+  return (double)s.x + ((double)s.y + (double)s.z);
 }
 
 // Exact, order-independent combination of group totals.  A cell's group totals are

@@ -145,8 +145,8 @@ __device__ __forceinline__ SpanRange span_range(const InstParams& a, const int* 
 // (sigma g independent of g).  CTAs per SM the register budget is set for: 3 of 8 warps,
 // 6 of 4 warps; the batched 4-warp kernel reads its parameters from shared memory and
 // spills at 6 (85 registers), so it is given 5 (no spills, 10 % faster on the
-// 256-instance batch).  With the error-keeping moment sums (kF64: 24 binary32 values per
-// lane, 114 to 118 registers) two and four.
+// 256-instance batch).  With the error-keeping moment sums (kF64: 36 binary32 values per
+// lane, 124 registers) two and four.
 template <bool kBatch, int kWarps, bool kF64>
 constexpr int collide_ctas_per_sm() {
   return kF64 ? (kWarps == kAWarps ? 2 : 4) : (kWarps == kAWarps ? 3 : (kBatch ? 5 : 6));
