@@ -217,6 +217,18 @@ DSMC_API dsmc_status dsmc_set_options(dsmc_handle h, const dsmc_options* opt);
  * latched by an earlier synchronising call, else DSMC_OK. */
 DSMC_API dsmc_status dsmc_step(dsmc_handle h, int n_steps);
 
+/* How the latest dsmc_step advanced the handle (the results do not depend on it): by the
+ * span passes, several launches per step; or many steps per launch, on a thread-block
+ * cluster per instance or, for one run, on a team of CTAs over the device.  *ctas gets the
+ * CTAs per instance (0 for the span passes).  Either pointer may be NULL. */
+typedef enum dsmc_step_kind {
+  DSMC_STEP_NONE = 0, /* no step yet */
+  DSMC_STEP_SPANS = 1,
+  DSMC_STEP_CLUSTERS = 2,
+  DSMC_STEP_TEAM = 3
+} dsmc_step_kind;
+DSMC_API dsmc_status dsmc_last_step(dsmc_handle h, int* kind, int* ctas);
+
 /* Wait for the handle's stream and check the device error word. */
 DSMC_API dsmc_status dsmc_sync(dsmc_handle h);
 

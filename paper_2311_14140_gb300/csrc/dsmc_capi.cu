@@ -430,6 +430,7 @@ struct dsmc_sim {
   ResidentLaunch res{};
   bool res_dirty = true;
   bool span_passes = false;  // the caller's options name a partition, or it is being tuned
+  int last_kind = DSMC_STEP_NONE, last_ctas = 0;  // of the latest steps
   // CUDA graph of kGraphSteps consecutive steps, replayed by dsmc_step when
   // options.graph is set.  Its kernels read the global step from gstep_dev, which the
   // kernel that forms the cell offsets advances.
@@ -1176,6 +1177,8 @@ dsmc_status step_resident(dsmc_sim* h, int n) {
   h->ocur ^= n & 1;
   h->scur ^= n & 1;
   count_steps(h, n);
+  h->last_kind = R.team ? DSMC_STEP_TEAM : DSMC_STEP_CLUSTERS;
+  h->last_ctas = R.cl;
   return DSMC_OK;
 }
 
@@ -1194,6 +1197,8 @@ dsmc_status step_n(dsmc_sim* h, int n_steps) {
       }
       return DSMC_OK;
     }
+    h->last_kind = DSMC_STEP_SPANS;
+    h->last_ctas = 0;
   }
   if (h->opt.graph && !h->opt.profile && h->n_inst() > 0) {
     while (n_steps - it >= kGraphSteps) {
@@ -1655,6 +1660,14 @@ dsmc_status dsmc_step(dsmc_handle h, int n_steps) {
   s = step_n(h, n_steps);
   if (s != DSMC_OK) return s;
   if (h->opt.profile) return collect_times(h);
+  return DSMC_OK;
+}
+
+dsmc_status dsmc_last_step(dsmc_handle h, int* kind, int* ctas) {
+  dsmc_status s = check_handle(h);
+  if (s != DSMC_OK) return s;
+  if (kind) *kind = h->last_kind;
+  if (ctas) *ctas = h->last_ctas;
   return DSMC_OK;
 }
 

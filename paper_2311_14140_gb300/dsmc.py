@@ -143,6 +143,7 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
                                 c.c_size_t, c.POINTER(H)]),
         "dsmc_set_options": (st, [H, c.POINTER(Options)]),
         "dsmc_step": (st, [H, c.c_int]),
+        "dsmc_last_step": (st, [H, c.POINTER(c.c_int), c.POINTER(c.c_int)]),
         "dsmc_sync": (st, [H]),
         "dsmc_sample_moments": (st, [H, c.c_void_p, c.POINTER(c.c_longlong)]),
         "dsmc_cell_fields": (st, [c.c_void_p, c.c_longlong, c.c_int, c.c_int, c.c_void_p]),
@@ -239,6 +240,16 @@ def _ptr(a) -> Optional[int]:
     return a.data_ptr()
 
 
+STEP_KINDS = (None, "spans", "clusters", "team")
+
+
+def _last_step(handle):
+    """How the latest step call advanced a handle: (kind, CTAs per run)."""
+    kind, ctas = ctypes.c_int(), ctypes.c_int()
+    _check(load_library().dsmc_last_step(handle, ctypes.byref(kind), ctypes.byref(ctas)))
+    return STEP_KINDS[kind.value], ctas.value
+
+
 def default_options() -> Options:
     o = Options()
     _check(load_library().dsmc_default_options(ctypes.byref(o)))
@@ -319,6 +330,10 @@ class Dsmc:
     # stepping -------------------------------------------------------------------
     def step(self, n: int = 1) -> None:
         _check(self._lib.dsmc_step(self._h, int(n)))
+
+    def last_step(self):
+        """How the latest step call advanced the handle (``dsmc_last_step``)."""
+        return _last_step(self._h)
 
     def sync(self) -> None:
         _check(self._lib.dsmc_sync(self._h))
@@ -465,6 +480,10 @@ class _Multi:
 
     def step(self, n: int = 1) -> None:
         _check(self._lib.dsmc_step(self._h, int(n)))
+
+    def last_step(self):
+        """How the latest step call advanced the handle (``dsmc_last_step``)."""
+        return _last_step(self._h)
 
     def sync(self) -> None:
         _check(self._lib.dsmc_sync(self._h))
