@@ -603,8 +603,13 @@ DSMC_API dsmc_status dsmc_cfd_faces(double Kn, double F, int n, int slip, double
  * advance every instance, and since the partition does not change results the run is
  * the same as without tuning.  A handle whose steps run many to a launch (see
  * dsmc_options.span_particles) keeps doing so; the tuner then chooses the partition its
- * span passes would use.  *best_span_particles and *best_ms_per_step (either may
- * be NULL) get the choice and its time per step.  Synchronises. */
+ * span passes would use.  Where several CTAs share a cell, that partition is tried too and
+ * kept, as the library's own choice, if it is the fastest.  *best_span_particles and
+ * *best_ms_per_step (either may be NULL) get the span_particles (as in dsmc_info) and the
+ * time per step of the partition that the handle has afterwards; after an error it has the
+ * one from before.  Options that give the tuner's values back (a copy of the options with
+ * another field changed) name nothing: they leave the kind of steps and the partition as
+ * they are.  Synchronises. */
 DSMC_API dsmc_status dsmc_autotune(dsmc_handle h, int steps_per_trial, int* best_span_particles,
                                    double* best_ms_per_step);
 

@@ -171,6 +171,11 @@ dsmc_status check_options(const dsmc_options* o) {
   return DSMC_OK;
 }
 
+// The options that set the split of the span passes; 0: not named.
+struct Split {
+  int particles = 0, warps = 0, rows = 0;
+};
+
 bool names_partition(const dsmc_options& o) {
   return o.span_particles || o.cta_warps || o.span_rows;
 }
@@ -397,6 +402,9 @@ struct dsmc_sim {
   // The split of the span passes follows the instances (choose_split) until the options or the
   // tuner name one; instances were added or removed since it was made.
   bool auto_split = true, split_dirty = false;
+  // The split dsmc_autotune chose: options that give it back (as a caller does who changes
+  // another option) name nothing by themselves.
+  Split tuned;
   int check_warps = kAWarps;  // warps per CTA that instances' sizes are checked against
   int cta_warps = kAWarps;  // warps per CTA of the collide/move pass
   int span_rows = 1;        // sort-matrix rows per span
@@ -1621,12 +1629,17 @@ dsmc_status dsmc_set_options(dsmc_handle h, const dsmc_options* opt) {
     if (!derive_params(x.omega, x.Kn, x.F, x.ppc, *opt, &ps[id]))
       return fail(DSMC_E_INVAL, "time step undefined: set options.dt for infinite Kn");
   }
-  // span_particles = 0 and cta_warps = 0 keep the partition and CTA shape in use.
+  // 0 keeps the value in use, and so does the tuner's.
   ensure_partition(h);
-  if (opt->span_particles || opt->cta_warps) h->auto_split = false;
+  const Split& tuned = h->tuned;
+  const bool new_particles = opt->span_particles && opt->span_particles != tuned.particles;
+  const bool new_warps = opt->cta_warps && opt->cta_warps != tuned.warps;
+  const bool named = new_particles || new_warps ||
+                     (opt->span_rows && opt->span_rows != tuned.rows);
+  const bool auto_split = h->auto_split && !new_particles && !new_warps;
   const int target_use = opt->span_particles ? opt->span_particles : h->span_target;
   const int warps_use = opt->cta_warps ? opt->cta_warps
-                                       : (h->auto_split ? h->check_warps : h->cta_warps);
+                                       : (auto_split ? h->check_warps : h->cta_warps);
   const int rows_use = opt->span_rows ? opt->span_rows : h->span_rows;
   int mcps, mcells;
   partition_extent(h, target_use, nullptr, &mcps, &mcells);
@@ -1637,15 +1650,23 @@ dsmc_status dsmc_set_options(dsmc_handle h, const dsmc_options* opt) {
     if (s != DSMC_OK) return s;
   }
   h->opt = *opt;
-  h->span_passes = names_partition(*opt);
+  if (named) {
+    h->span_passes = true;
+    h->tuned = Split{};
+  } else if (!names_partition(*opt)) {
+    h->span_passes = false;
+  }
   for (int id : h->order) h->inst[id].p = ps[id];
-  if (h->auto_split)
-    h->split_dirty = true;  // the group size bears on the choice
-  else
-    h->cta_warps = warps_use;
-  if (opt->cta_warps) h->check_warps = warps_use;
+  const bool was_auto = h->auto_split;
+  h->auto_split = auto_split;
+  if (opt->cta_warps && !auto_split) h->check_warps = warps_use;
   h->span_rows = rows_use;
-  if (target_use != h->span_target) set_partition(h, target_use);
+  if (auto_split) {
+    h->split_dirty = true;  // the group size bears on the choice
+  } else {
+    h->cta_warps = warps_use;
+    if (was_auto || target_use != h->span_target) set_partition(h, target_use);
+  }
   h->tab_dirty = h->res_dirty = true;
   drop_graph(h);  // launch shapes or the stream may have changed
   return DSMC_OK;
@@ -1687,15 +1708,30 @@ dsmc_status dsmc_autotune(dsmc_handle h, int steps_per_trial, int* best_span_par
     return fail(DSMC_E_CUDA, "event");
   }
   ensure_partition(h);
-  int best = h->span_target, best_warps = h->cta_warps, best_rows = h->span_rows;
+  const bool own_auto = h->auto_split, span_passes = h->span_passes;
+  const Split own{h->span_target, h->cta_warps, h->span_rows};
+  Split best = own;
+  bool best_own = false;  // the partition in use is the fastest
   double best_ms = -1.0;
   dsmc_status r = DSMC_OK;
-  const bool span_passes = h->span_passes;
   h->span_passes = h->res_dirty = true;  // the trials are of the span passes
-  // a run whose cells are shared by several CTAs keeps that partition, which the trials'
-  // whole-cell spans cannot reach
-  const bool shared = h->inst[h->order[0]].parts > 1;
-  const int own_target = h->span_target, own_warps = h->cta_warps, own_rows = h->span_rows;
+  // One untimed step with a new shape, then the timed trial; whether it is the fastest.
+  auto trial = [&]() {
+    if ((r = step_n(h, 1)) != DSMC_OK) return false;
+    if (cudaEventRecord(e0, st) != cudaSuccess) return r = fail(DSMC_E_CUDA, "event record"), false;
+    if ((r = step_n(h, steps_per_trial)) != DSMC_OK) return false;
+    if (cudaEventRecord(e1, st) != cudaSuccess) return r = fail(DSMC_E_CUDA, "event record"), false;
+    if (cudaEventSynchronize(e1) != cudaSuccess) return r = fail(DSMC_E_CUDA, "event sync"), false;
+    float ms = 0.0f;
+    cudaEventElapsedTime(&ms, e0, e1);
+    const double per = ms / steps_per_trial;
+    if (best_ms >= 0.0 && per >= best_ms) return false;
+    best_ms = per;
+    return true;
+  };
+  // a run whose cells are shared by several CTAs: that partition, which the whole-cell spans
+  // below cannot reach, is the first trial
+  if (h->inst[h->order[0]].parts > 1) best_own = trial();
   h->auto_split = false;
   const int shapes[4][2] = {{kAWarps, 1}, {kAWarps, 2}, {kAWarpsSmall, 1}, {kAWarpsSmall, 2}};
   for (const auto& shape : shapes) {
@@ -1717,20 +1753,9 @@ dsmc_status dsmc_autotune(dsmc_handle h, int steps_per_trial, int* best_span_par
       h->cta_warps = w;
       h->span_rows = rows;
       set_partition(h, target);
-      // one untimed step with the new shape, then the timed trial
-      if ((r = step_n(h, 1)) != DSMC_OK) break;
-      if (cudaEventRecord(e0, st) != cudaSuccess) { r = fail(DSMC_E_CUDA, "event record"); break; }
-      if ((r = step_n(h, steps_per_trial)) != DSMC_OK) break;
-      if (cudaEventRecord(e1, st) != cudaSuccess) { r = fail(DSMC_E_CUDA, "event record"); break; }
-      if (cudaEventSynchronize(e1) != cudaSuccess) { r = fail(DSMC_E_CUDA, "event sync"); break; }
-      float ms = 0.0f;
-      cudaEventElapsedTime(&ms, e0, e1);
-      const double per = ms / steps_per_trial;
-      if (best_ms < 0.0 || per < best_ms) {
-        best_ms = per;
-        best = target;
-        best_warps = w;
-        best_rows = rows;
+      if (trial()) {
+        best = Split{target, w, rows};
+        best_own = false;
       }
     }
     if (r != DSMC_OK) break;
@@ -1739,24 +1764,26 @@ dsmc_status dsmc_autotune(dsmc_handle h, int steps_per_trial, int* best_span_par
   cudaEventDestroy(e1);
   h->span_passes = span_passes;
   h->res_dirty = true;
-  if (r != DSMC_OK) {
-    h->auto_split = shared;
-    return r;
-  }
-  if (shared) {
-    h->auto_split = true;
-    h->cta_warps = own_warps;
-    h->span_rows = own_rows;
-    set_partition(h, own_target);
+  if (r != DSMC_OK || best_own) {  // as before the trials
+    h->auto_split = own_auto;
+    h->cta_warps = own.warps;
+    h->span_rows = own.rows;
+    set_partition(h, own.particles);
+    if (r != DSMC_OK) {
+      cudaGetLastError();
+      return r;
+    }
+    best = own;
   } else {
-    h->cta_warps = h->check_warps = best_warps;
-    h->span_rows = best_rows;
-    set_partition(h, best);
-    h->opt.span_particles = best;
-    h->opt.cta_warps = best_warps;
-    h->opt.span_rows = best_rows;
+    h->cta_warps = h->check_warps = best.warps;
+    h->span_rows = best.rows;
+    set_partition(h, best.particles);
+    h->opt.span_particles = best.particles;
+    h->opt.cta_warps = best.warps;
+    h->opt.span_rows = best.rows;
   }
-  if (best_span_particles) *best_span_particles = best;
+  h->tuned = best;
+  if (best_span_particles) *best_span_particles = best.particles;
   if (best_ms_per_step) *best_ms_per_step = best_ms;
   if (h->opt.profile) return collect_times(h);
   return DSMC_OK;
