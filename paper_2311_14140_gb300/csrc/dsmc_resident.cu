@@ -95,25 +95,31 @@ __device__ __forceinline__ void peer_max(uint32_t addr, uint32_t v) {
 // Barrier of the CTAs of a team: a counter and a generation in global memory (both zero, or as
 // an earlier team left them).  The last CTA to arrive clears the counter and advances the
 // generation.  Memory operations before it are visible after it to loads that bypass L1.
-// Waits are bounded; false when one ran out.
+// Waits are bounded; false when one ran out.  The counter is then out of step for good, so a team
+// whose run's error word has kErrTeam already does not start: its first wait is false at once, and
+// nothing of the run has been written by then (launches may be queued behind the one that failed).
 struct TeamBarrier {
   unsigned *count = nullptr, *gen = nullptr, now = 0u;
   int n = 0;
+  bool dead = false;
   static __device__ __forceinline__ unsigned load(const unsigned* p) {
     unsigned v;
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
   }
-  __device__ __forceinline__ void start(unsigned* b, int ctas) {
+  __device__ __forceinline__ void start(unsigned* b, int ctas, const int* err) {
     count = b;
     gen = b + 1;
     n = ctas;
-    if (threadIdx.x == 0) now = load(gen);  // nobody passes the first wait before this CTA arrives
+    if (threadIdx.x == 0) {
+      now = load(gen);  // nobody passes the first wait before this CTA arrives
+      dead = (*(const volatile int*)err & kErrTeam) != 0;
+    }
   }
   __device__ __forceinline__ bool wait() {
-    bool ok = true;
+    bool ok = !dead;
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0 && ok) {
       unsigned before;
       asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;"
                    : "=r"(before)
@@ -201,7 +207,7 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
   unsigned long long* xfix = reinterpret_cast<unsigned long long*>(
       exchange + team_fix_offset(CL, n_cells));
   TeamBarrier team;
-  if constexpr (kTeam) team.start(barrier, CL);
+  if constexpr (kTeam) team.start(barrier, CL, err);
   bool lost = false;  // a wait ran out: the CTA leaves, and the others' waits run out too
   auto wait_all = [&]() {
     if constexpr (kTeam)
