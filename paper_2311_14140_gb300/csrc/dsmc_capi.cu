@@ -1168,7 +1168,9 @@ void plan_resident(dsmc_sim* h) {
   h->tab_dirty = true;  // the instance table carries the cuts
 }
 
-// n steps of a resident launch.
+// n steps of a resident launch.  Where the launch is refused (a stream that has only some of the
+// SMs, for which the plan's queries do not ask), nothing has run: the handle's steps take the span
+// passes from then on (res.cl = 0).
 dsmc_status step_resident(dsmc_sim* h, int n) {
   ResidentLaunch R = h->res;
   R.tab = h->tab_dev;
@@ -1177,10 +1179,18 @@ dsmc_status step_resident(dsmc_sim* h, int n) {
   R.parity_rec = h->cur;
   R.parity_off = h->ocur;
   R.parity_smax = h->scur;
-  DSMC_CUDA(launch_resident(h->P[0], h->P[1], h->off[0], h->off[1], h->smax[0], h->smax[1],
-                            h->ncand, h->nacc, h->acc, h->hist, h->barrier, h->tab[0], R,
-                            h->opt.accum == DSMC_ACCUM_FP64, h->err, h->stream()),
-            "resident steps");
+  const cudaError_t e =
+      launch_resident(h->P[0], h->P[1], h->off[0], h->off[1], h->smax[0], h->smax[1], h->ncand,
+                      h->nacc, h->acc, h->hist, h->barrier, h->tab[0], R,
+                      h->opt.accum == DSMC_ACCUM_FP64, h->err, h->stream());
+  if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorLaunchOutOfResources ||
+      e == cudaErrorInvalidConfiguration || e == cudaErrorInvalidClusterSize ||
+      e == cudaErrorNotSupported) {
+    cudaGetLastError();
+    h->res.cl = 0;
+    return DSMC_OK;
+  }
+  DSMC_CUDA(e, "resident steps");
   h->cur ^= n & 1;
   h->ocur ^= n & 1;
   h->scur ^= n & 1;
@@ -1198,12 +1208,12 @@ dsmc_status step_n(dsmc_sim* h, int n_steps) {
     if (h->res_dirty || h->split_dirty) plan_resident(h);
     if (h->res.cl > 0) {
       if ((s = upload_tables(h)) != DSMC_OK) return s;
-      while (it < n_steps) {
+      while (it < n_steps && h->res.cl > 0) {
         const int n = std::min(n_steps - it, kResidentSteps);
         if ((s = step_resident(h, n)) != DSMC_OK) return s;
-        it += n;
+        if (h->res.cl > 0) it += n;
       }
-      return DSMC_OK;
+      if (it == n_steps) return DSMC_OK;
     }
     h->last_kind = DSMC_STEP_SPANS;
     h->last_ctas = 0;
