@@ -95,31 +95,25 @@ __device__ __forceinline__ void peer_max(uint32_t addr, uint32_t v) {
 // Barrier of the CTAs of a team: a counter and a generation in global memory (both zero, or as
 // an earlier team left them).  The last CTA to arrive clears the counter and advances the
 // generation.  Memory operations before it are visible after it to loads that bypass L1.
-// Waits are bounded; false when one ran out.  The counter is then out of step for good, so a team
-// whose run's error word has kErrTeam already does not start: its first wait is false at once, and
-// nothing of the run has been written by then (launches may be queued behind the one that failed).
+// Waits are bounded; false when one ran out.  The counter is then out of step for good.
 struct TeamBarrier {
   unsigned *count = nullptr, *gen = nullptr, now = 0u;
   int n = 0;
-  bool dead = false;
   static __device__ __forceinline__ unsigned load(const unsigned* p) {
     unsigned v;
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
   }
-  __device__ __forceinline__ void start(unsigned* b, int ctas, const int* err) {
+  __device__ __forceinline__ void start(unsigned* b, int ctas) {
     count = b;
     gen = b + 1;
     n = ctas;
-    if (threadIdx.x == 0) {
-      now = load(gen);  // nobody passes the first wait before this CTA arrives
-      dead = (*(const volatile int*)err & kErrTeam) != 0;
-    }
+    if (threadIdx.x == 0) now = load(gen);  // nobody passes the first wait before this CTA arrives
   }
   __device__ __forceinline__ bool wait() {
-    bool ok = !dead;
+    bool ok = true;
     __syncthreads();
-    if (threadIdx.x == 0 && ok) {
+    if (threadIdx.x == 0) {
       unsigned before;
       asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;"
                    : "=r"(before)
@@ -160,7 +154,7 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
   // first groups of the CTAs (kLocal: of all of them), or of this CTA and the next
   constexpr int kBounds = kLocal ? kResidentMaxCluster + 1 : 2;
   __shared__ int bnd_slot[kBounds], bnd_cell[kBounds], bnd_group[kBounds];
-  __shared__ int n_groups_sh, next_group, n_hits;
+  __shared__ int n_groups_sh, next_group, n_hits, dead;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const unsigned lt = (1u << lane) - 1u;
   const int CL = RL.cl;
@@ -207,7 +201,7 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
   unsigned long long* xfix = reinterpret_cast<unsigned long long*>(
       exchange + team_fix_offset(CL, n_cells));
   TeamBarrier team;
-  if constexpr (kTeam) team.start(barrier, CL, err);
+  if constexpr (kTeam) team.start(barrier, CL);
   bool lost = false;  // a wait ran out: the CTA leaves, and the others' waits run out too
   auto wait_all = [&]() {
     if constexpr (kTeam)
@@ -300,6 +294,9 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
   const int qcap = (int)(L.rows_bytes / 2) & ~31;  // wall hits the queue holds
   if (tid == 0) {
     n_hits = 0;
+    // A team whose run's error word has kErrTeam already does not start: launches may be queued
+    // behind the one whose wait ran out.
+    dead = kTeam && (*(const volatile int*)err & kErrTeam) != 0;
     // the instance's end (the last CTA's end is past every cell)
     bnd_slot[last] = hi;
     bnd_cell[last] = n_cells;
@@ -318,7 +315,10 @@ __global__ void __launch_bounds__(kWarps * 32, kBatch ? 2 : 1)
     const int s0 = bnd_slot[me], n = min(bnd_slot[me + 1] - s0, RL.range_cap);
     for (int i = tid; i < n; i += kThreads) rec[i] = Pin[s0 + i];
   }
-  wait_all();  // every CTA's accumulators are cleared
+  if (kTeam && dead)
+    lost = true;  // (nothing of the run has been written)
+  else
+    wait_all();  // every CTA's accumulators are cleared
 
   int st = 0;
   for (; st < RL.n_steps && !lost; ++st, ++istep) {
