@@ -103,7 +103,9 @@ typedef struct dsmc_options {
   int group_size;         /* collision group G: even, 2 <= G <= 512; default 256 */
   int collisions;         /* 0 turns collisions off; default 1 */
   int profile;            /* 1: time every kernel launch with CUDA events (then
-                             dsmc_step synchronises at its end); default 0 */
+                             dsmc_step synchronises at its end); steps then take the
+                             span passes at every size (see span_particles), and
+                             the times are theirs; default 0 */
   int span_particles;     /* particles per span (CTA) of the step passes at the
                              initial density: 0 leaves the partition to the library
                              (one run: 4096 to 6144, fewer when its spans then fill
@@ -117,9 +119,12 @@ typedef struct dsmc_options {
                              all 0, steps of one run of up to about 1,300,000
                              particles, or of a batch of up to about 40,000 per
                              instance, may run many at a time in one launch (a
-                             cooperative one, with a CTA on every SM, above 40,000);
-                             a value in any of the three keeps the span passes;
-                             default 0 */
+                             cooperative one, with a CTA on every SM, above 40,000;
+                             such launches of several streams run one after the
+                             other, so while the steps of two other such runs are in
+                             flight on other streams, a call's steps take the span
+                             passes, which overlap); a value in any of the three, or
+                             profile, keeps the span passes; default 0 */
   int cta_warps;          /* warps per CTA of the collide/move pass: 0 keeps the shape
                              in use (one run: 8; batches and pools: 8, or 4 from about
                              27,000 particles per SM on; or what dsmc_autotune chose,

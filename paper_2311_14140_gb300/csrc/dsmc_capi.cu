@@ -7,10 +7,12 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <climits>
 #include <cmath>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <new>
 #include <string>
 #include <vector>
@@ -402,6 +404,7 @@ struct dsmc_sim {
   // The split of the span passes follows the instances (choose_split) until the options or the
   // tuner name one; instances were added or removed since it was made.
   bool auto_split = true, split_dirty = false;
+  bool split_shared = false;  // choose_split's choice for a device shared with other runs
   // The split dsmc_autotune chose: options that give it back (as a caller does who changes
   // another option) name nothing by themselves.
   Split tuned;
@@ -439,6 +442,9 @@ struct dsmc_sim {
   bool res_dirty = true;
   bool span_passes = false;  // the caller's options name a partition, or it is being tuned
   int last_kind = DSMC_STEP_NONE, last_ctas = 0;  // of the latest steps
+  // Behind the latest steps of a run on a team, and their stream (TeamRuns; under its lock).
+  cudaEvent_t stepped = nullptr;
+  void* stepped_stream = nullptr;
   // CUDA graph of kGraphSteps consecutive steps, replayed by dsmc_step when
   // options.graph is set.  Its kernels read the global step from gstep_dev, which the
   // kernel that forms the cell offsets advances.
@@ -568,7 +574,8 @@ void set_partition(dsmc_sim* h, int target) {
     Inst& x = h->inst[h->order[t]];
     np += x.N;
     make_spans(x.n_cells, x.ppc, target, &x.cps, &x.n_spans);
-    x.parts = h->auto_split && !h->pool && h->C.inst == 1 && !fills_wave(x.n_cells, h->sms)
+    x.parts = h->auto_split && !h->split_shared && !h->pool && h->C.inst == 1 &&
+                      !fills_wave(x.n_cells, h->sms)
                   ? cell_parts(x.n_cells, x.ppc)
                   : 1;
     if (x.parts > 1) {
@@ -608,7 +615,11 @@ void choose_split(dsmc_sim* h) {
     if (h->n_inst() == 1) {
       const Inst& x = h->inst[h->order[0]];
       long long target;
-      if (x.n_cells > kCoopCells) {
+      if (h->split_shared) {
+        // steps beside those of other runs: fewer, larger spans than one run needs to fill the SMs
+        // cost least in all (8 runs of 397 x 2,531: 397 spans 27.6 us per step and run, 199 17.7)
+        target = default_span_particles(x.N);
+      } else if (x.n_cells > kCoopCells) {
         // a scatter with a warp per span wants about 6.6 of them per SM (3,000 x 500: 334 spans
         // 106 us per step, 1,000 spans 64); beyond 4,096 particles whole cells up to 6,144 (4,000
         // x 1,500: 1,334 spans 196, 1,000 spans 185), but no cell more (1,600 x 5,000: 1,600
@@ -1078,22 +1089,6 @@ int set_cuts(const Inst& x, int cl, int* cut) {
   return share;
 }
 
-// Decides whether the handle's steps run resident (dsmc_resident.cu) and with how many CTAs
-// per instance.  Options that name a partition of the span passes keep those, as does
-// profiling, which times their kernels; a pool's members come and go between calls.
-//
-// One run: a cluster of 16 CTAs up to kClusterParticles (us per step, cluster / team of 152 /
-// span passes under graph replay: 2,250 particles 7.0 / 10.7 / 20.5, 20,000 11.4 / 13.0 / 22.5,
-// 40,000 13.8 / 13.0 / 23, 80,000 23.1 / 14.9 / 27), from there a team of a CTA per SM (more
-// CTAs were never slower: 100,000 particles 18.4 with 32, 15.2 with 64, 13.7 with 152), as long
-// as its share fits a CTA's shared memory (1,004,807 particles 27.7 against 71; up to about
-// 1,300,000, depending on the cells).
-// A batch: clusters of as many CTAs per instance as give shares of at most kResidentShare
-// particles and fill the SMs twice, as long as an instance then fits 16 CTAs and the launch is
-// not many waves long (64 x 2,250 particles: 11 us per step against 30; 64 x 10,000: 28 / 48;
-// 64 x 20,000: 45 / 70; 128 x 20,000, 1,024 CTAs: 87 / 95; beyond that the span passes,
-// which spread every instance over all SMs, are as fast: 256 x 20,000, 161 / 153;
-// 24 x 100,000, 137 / 85).
 constexpr long long kClusterParticles = 40000;
 constexpr int kResidentShare = 2600;
 
@@ -1123,10 +1118,113 @@ bool size_resident(dsmc_sim* h, ResidentLaunch& R) {
   return false;
 }
 
-void plan_resident(dsmc_sim* h) {
+// The runs of this process whose steps go to a team.  A team has the whole device to itself, so
+// teams of several streams run one after the other where span passes overlap (us per step and run,
+// one after the other / span passes: 200 x 500 on 2 streams 14.0 / 14.4, 3 14.1 / 9.7, 8 13.9 / 4.0;
+// 300 x 1,000 on 2 16.5 / 22, 3 16.5 / 15.4, 8 16.4 / 7.1; 397 x 2,531 on 3 27.6 / 28, 4 27.7 / 22).
+// While the steps of kTeamOthers other runs, on other streams, are in flight, a call's steps take
+// the span passes.  Runs mark their steps with an event only while there are that many of them.
+constexpr int kTeamOthers = 2;
+
+struct TeamRuns {
+  std::mutex lock;
+  std::vector<dsmc_sim*> runs;
+  std::atomic<int> size{0};
+};
+
+TeamRuns& team_runs() {
+  static TeamRuns* const t = new TeamRuns;  // (handles may be destroyed after static objects)
+  return *t;
+}
+
+// Event calls are not allowed while another thread captures a stream in global mode, unless this
+// thread says that they do not concern it.
+struct RelaxedCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+void leave_team_runs(dsmc_sim* h) {
+  TeamRuns& t = team_runs();
+  std::lock_guard<std::mutex> hold(t.lock);
+  t.runs.erase(std::remove(t.runs.begin(), t.runs.end(), h), t.runs.end());
+  t.size = (int)t.runs.size();
+}
+
+void join_team_runs(dsmc_sim* h) {
+  TeamRuns& t = team_runs();
+  std::lock_guard<std::mutex> hold(t.lock);
+  if (std::find(t.runs.begin(), t.runs.end(), h) == t.runs.end()) t.runs.push_back(h);
+  t.size = (int)t.runs.size();
+}
+
+// Whether events may bear on this handle's steps: enough other runs, and no capture of its stream.
+bool team_runs_watched(dsmc_sim* h) {
+  if (team_runs().size <= kTeamOthers) return false;
+  cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(h->stream(), &c) == cudaSuccess) return c == cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return false;
+}
+
+// Whether the device is to be shared: kTeamOthers other runs have steps in flight.
+bool team_runs_crowded(dsmc_sim* h) {
+  TeamRuns& t = team_runs();
+  RelaxedCapture relaxed;
+  std::lock_guard<std::mutex> hold(t.lock);
+  int n = 0;
+  for (dsmc_sim* x : t.runs) {
+    if (x == h || x->device != h->device || !x->stepped || x->stepped_stream == h->opt.stream)
+      continue;
+    if (cudaEventQuery(x->stepped) == cudaErrorNotReady) ++n;
+    cudaGetLastError();
+    if (n >= kTeamOthers) return true;
+  }
+  return false;
+}
+
+// Marks the steps enqueued so far (best effort: a missing mark only leaves the choice as it was).
+void mark_team_steps(dsmc_sim* h) {
+  TeamRuns& t = team_runs();
+  RelaxedCapture relaxed;
+  std::lock_guard<std::mutex> hold(t.lock);
+  if (!h->stepped && cudaEventCreateWithFlags(&h->stepped, cudaEventDisableTiming) != cudaSuccess) {
+    cudaGetLastError();
+    h->stepped = nullptr;
+    return;
+  }
+  h->stepped_stream = h->opt.stream;
+  if (cudaEventRecord(h->stepped, h->stream()) != cudaSuccess) cudaGetLastError();
+}
+
+// The split of a run of its own beside other runs, or alone.  (The plan of resident steps does
+// not depend on it.)
+void use_shared_split(dsmc_sim* h, bool shared) {
+  if (!h->auto_split || h->split_shared == shared) return;
+  h->split_shared = shared;
+  h->split_dirty = true;
   ensure_partition(h);
-  h->res = ResidentLaunch{};
   h->res_dirty = false;
+}
+
+// Decides whether the handle's steps run resident (dsmc_resident.cu) and with how many CTAs
+// per instance.  Options that name a partition of the span passes keep those, as does
+// profiling, which times their kernels; a pool's members come and go between calls.
+//
+// One run: a cluster of 16 CTAs up to kClusterParticles (us per step, cluster / team of 152 /
+// span passes under graph replay: 2,250 particles 7.0 / 10.7 / 20.5, 20,000 11.4 / 13.0 / 22.5,
+// 40,000 13.8 / 13.0 / 23, 80,000 23.1 / 14.9 / 27), from there a team of a CTA per SM (more
+// CTAs were never slower: 100,000 particles 18.4 with 32, 15.2 with 64, 13.7 with 152), as long
+// as its share fits a CTA's shared memory (1,004,807 particles 27.7 against 71; up to about
+// 1,300,000, depending on the cells).
+// A batch: clusters of as many CTAs per instance as give shares of at most kResidentShare
+// particles and fill the SMs twice, as long as an instance then fits 16 CTAs and the launch is
+// not many waves long (64 x 2,250 particles: 11 us per step against 30; 64 x 10,000: 28 / 48;
+// 64 x 20,000: 45 / 70; 128 x 20,000, 1,024 CTAs: 87 / 95; beyond that the span passes,
+// which spread every instance over all SMs, are as fast: 256 x 20,000, 161 / 153;
+// 24 x 100,000, 137 / 85).
+void find_resident(dsmc_sim* h) {
   if (h->pool || h->opt.profile || h->span_passes) return;
   long long n_max = 0;
   for (int id : h->order) n_max = std::max(n_max, h->inst[id].N);
@@ -1162,11 +1260,23 @@ void plan_resident(dsmc_sim* h) {
     std::stable_sort(h->order.begin(), h->order.end(),
                      [&](int x, int y) { return cost(x) > cost(y); });
     set_partition(h, h->span_target);  // places in the table have changed
-    h->res_dirty = false;
   }
   h->res = R;
   h->tab_dirty = true;  // the instance table carries the cuts
 }
+
+void plan_resident(dsmc_sim* h) {
+  ensure_partition(h);
+  if (h->res.team) leave_team_runs(h);
+  h->res = ResidentLaunch{};
+  find_resident(h);
+  if (h->res.team)
+    join_team_runs(h);
+  else
+    use_shared_split(h, false);
+  h->res_dirty = false;
+}
+
 
 // n steps of a resident launch.  Where the launch is refused (a stream that has only some of the
 // SMs, for which the plan's queries do not ask), nothing has run: the handle's steps take the span
@@ -1187,7 +1297,8 @@ dsmc_status step_resident(dsmc_sim* h, int n) {
       e == cudaErrorInvalidConfiguration || e == cudaErrorInvalidClusterSize ||
       e == cudaErrorNotSupported) {
     cudaGetLastError();
-    h->res.cl = 0;
+    if (R.team) leave_team_runs(h);
+    h->res = ResidentLaunch{};
     return DSMC_OK;
   }
   DSMC_CUDA(e, "resident steps");
@@ -1204,16 +1315,23 @@ dsmc_status step_n(dsmc_sim* h, int n_steps) {
   dsmc_status s;
   if ((s = admit_fresh(h)) != DSMC_OK) return s;
   int it = 0;
+  bool watched = false;
   if (h->n_inst() > 0 && n_steps > 0) {
     if (h->res_dirty || h->split_dirty) plan_resident(h);
-    if (h->res.cl > 0) {
+    watched = h->res.team && team_runs_watched(h);
+    const bool crowded = watched && team_runs_crowded(h);
+    if (crowded) use_shared_split(h, true);
+    if (h->res.cl > 0 && !crowded) {
       if ((s = upload_tables(h)) != DSMC_OK) return s;
       while (it < n_steps && h->res.cl > 0) {
         const int n = std::min(n_steps - it, kResidentSteps);
         if ((s = step_resident(h, n)) != DSMC_OK) return s;
         if (h->res.cl > 0) it += n;
       }
-      if (it == n_steps) return DSMC_OK;
+      if (it == n_steps) {
+        if (watched) mark_team_steps(h);
+        return DSMC_OK;
+      }
     }
     h->last_kind = DSMC_STEP_SPANS;
     h->last_ctas = 0;
@@ -1232,6 +1350,7 @@ dsmc_status step_n(dsmc_sim* h, int n_steps) {
   }
   for (; it < n_steps; ++it)
     if ((s = step_once(h)) != DSMC_OK) return s;
+  if (watched) mark_team_steps(h);
   return DSMC_OK;
 }
 
@@ -2091,6 +2210,8 @@ dsmc_status dsmc_destroy(dsmc_handle h) {
   DeviceGuard guard(h->device);
   cudaStreamSynchronize(h->stream());
   drop_graph(h);
+  leave_team_runs(h);
+  if (h->stepped) cudaEventDestroy(h->stepped);
   for (cudaEvent_t e : h->events) cudaEventDestroy(e);
   if (h->owns && h->ws) cudaFree(h->ws);
   delete h;
