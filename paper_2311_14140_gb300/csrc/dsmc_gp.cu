@@ -125,10 +125,14 @@ __global__ void __launch_bounds__(kGpThreads)
   if (t == 0) bad = 0;
   __syncthreads();
   {
+    // (a subnormal length scale has no finite reciprocal, and 0 times infinity is no distance)
     const double i1 = 1.0 / g[0], i2 = 1.0 / g[1], s2 = g[2];
+    const bool divide = isinf(i1) || isinf(i2);
     for (int e = t; e < nt; e += kGpThreads) {
       const int i = ij[e].x, j = ij[e].y;
-      const double d1 = (X[2 * i] - X[2 * j]) * i1, d2 = (X[2 * i + 1] - X[2 * j + 1]) * i2;
+      double d1 = X[2 * i] - X[2 * j], d2 = X[2 * i + 1] - X[2 * j + 1];
+      d1 = divide ? d1 / g[0] : d1 * i1;
+      d2 = divide ? d2 / g[1] : d2 * i2;
       const double k = exp(-0.5 * fma(d1, d1, d2 * d2));
       A[tri(i) + j] = i == j ? k + s2 : k;
     }
