@@ -301,30 +301,32 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
-// Mean and standard deviation when no model with random weights is selected (no slip, C0):
-// every trial has the same profile, and the standard deviation is the rounding of the sums
-// over the trials, about 1e-16 of u.  A caller comparing runs sees those digits, so the profile
-// is swept (Thomas) and the trials summed one after another, as for distinct profiles solved
-// trial by trial.
+// Standard deviation when no model with random weights is selected (no slip, C0): every trial has
+// the same profile, and the deviation is the rounding of the sums over the trials, about 1e-16 of
+// u.  Those digits are part of the results that runs of the library are compared by, and they
+// depend on the last bits of u: so u is swept here (Thomas) and the trials are summed one after
+// another, as for profiles solved trial by trial.  (The mean is k_bands's for every fit, whether a
+// standard deviation is asked for or not.)
 __global__ void __launch_bounds__(kThreads)
-    k_same_profiles(double kn, double F, int n, int n_trials, double* __restrict__ u,
-                    double* __restrict__ cp, double* __restrict__ mean, double* __restrict__ sd) {
+    k_same_profiles_sd(double kn, double F, int n, int n_trials, double* __restrict__ u,
+                       double* __restrict__ cp, double* __restrict__ sd) {
   if (threadIdx.x == 0) {
     const double h = 1.0 / n;
     const double src = -h * kSqrtPi * F / kn;
+    const double inner = 1.0 / h, wall = 2.0 / h;  // coefficients of the faces
     double cprev = 0.0, rprev = 0.0;
     for (int i = 0; i < n; ++i) {
-      const double lo = (i > 0) ? 1.0 / h : 0.0;
-      const double up = (i < n - 1) ? 1.0 / h : 0.0;
-      const double d =
-          -((i > 0) ? 1.0 / h : 2.0 / h) - ((i < n - 1) ? 1.0 / h : 2.0 / h);
+      const double lo = (i > 0) ? inner : 0.0;
+      const double up = (i < n - 1) ? inner : 0.0;
+      const double d = -((i > 0) ? inner : wall) - ((i < n - 1) ? inner : wall);
       const double den = d - lo * cprev;
       cprev = up / den;
       rprev = (src - lo * rprev) / den;
       cp[i] = cprev;
       u[i] = rprev;
     }
-    for (int i = n - 2; i >= 0; --i) u[i] -= cp[i] * u[i + 1];
+    double next = u[n - 1];
+    for (int i = n - 2; i >= 0; --i) u[i] = next = u[i] - cp[i] * next;
   }
   __syncthreads();
   for (int i = threadIdx.x; i < n; i += kThreads) {
@@ -333,7 +335,6 @@ __global__ void __launch_bounds__(kThreads)
     for (int t = 0; t < n_trials; ++t) s += x;
     const double m = s / n_trials, d = x - m;
     for (int t = 0; t < n_trials; ++t) v += d * d;
-    mean[i] = m;
     sd[i] = sqrt(v / (n_trials - 1));
   }
 }
@@ -778,19 +779,18 @@ dsmc_status dsmc_surrogate_profile(dsmc_surrogate_handle s, const dsmc_surrogate
   double* modes = weights + (size_t)n_trials * 4;
   double* md = modes + (size_t)n_cfd * 4;
   double* sd = md + n_cfd;
+  SUR_CUDA(cudaMemcpyAsync(zd, z, (size_t)n_trials * 4 * sizeof(double), cudaMemcpyDefault,
+                           s->stream),
+           "copy z");
+  k_modes<<<tm.k + 1 + (n_trials + kThreads - 1) / kThreads, kThreads, 0, s->stream>>>(
+      tm, zd, n_trials, modes, weights);
+  SUR_CUDA(cudaGetLastError(), "modes kernel");
+  k_bands<<<n_cfd, kThreads, 0, s->stream>>>(modes, weights, tm.k, n_trials, n_cfd, md, sd);
+  SUR_CUDA(cudaGetLastError(), "bands kernel");
   if (u_std && n_trials > 1 && tm.sel_v == 0 && tm.k == 0) {
-    k_same_profiles<<<1, kThreads, 0, s->stream>>>(tm.kn, tm.F, n_cfd, n_trials, modes,
-                                                   modes + n_cfd, md, sd);
+    k_same_profiles_sd<<<1, kThreads, 0, s->stream>>>(tm.kn, tm.F, n_cfd, n_trials, modes,
+                                                      modes + n_cfd, sd);
     SUR_CUDA(cudaGetLastError(), "profile kernel");
-  } else {
-    SUR_CUDA(cudaMemcpyAsync(zd, z, (size_t)n_trials * 4 * sizeof(double), cudaMemcpyDefault,
-                             s->stream),
-             "copy z");
-    k_modes<<<tm.k + 1 + (n_trials + kThreads - 1) / kThreads, kThreads, 0, s->stream>>>(
-        tm, zd, n_trials, modes, weights);
-    SUR_CUDA(cudaGetLastError(), "modes kernel");
-    k_bands<<<n_cfd, kThreads, 0, s->stream>>>(modes, weights, tm.k, n_trials, n_cfd, md, sd);
-    SUR_CUDA(cudaGetLastError(), "bands kernel");
   }
   SUR_CUDA(cudaMemcpyAsync(u_mean, md, n_cfd * sizeof(double), cudaMemcpyDefault, s->stream),
            "copy mean");
