@@ -1185,16 +1185,19 @@ bool team_runs_crowded(dsmc_sim* h) {
 }
 
 // Marks the steps enqueued so far (best effort: a missing mark only leaves the choice as it was).
+// The record is made without the lock: it waits where the stream's queue of launches is full.
 void mark_team_steps(dsmc_sim* h) {
-  TeamRuns& t = team_runs();
   RelaxedCapture relaxed;
-  std::lock_guard<std::mutex> hold(t.lock);
-  if (!h->stepped && cudaEventCreateWithFlags(&h->stepped, cudaEventDisableTiming) != cudaSuccess) {
-    cudaGetLastError();
-    h->stepped = nullptr;
-    return;
+  if (!h->stepped || h->stepped_stream != h->opt.stream) {
+    cudaEvent_t e = h->stepped;
+    if (!e && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {
+      cudaGetLastError();
+      return;
+    }
+    std::lock_guard<std::mutex> hold(team_runs().lock);
+    h->stepped = e;
+    h->stepped_stream = h->opt.stream;
   }
-  h->stepped_stream = h->opt.stream;
   if (cudaEventRecord(h->stepped, h->stream()) != cudaSuccess) cudaGetLastError();
 }
 
