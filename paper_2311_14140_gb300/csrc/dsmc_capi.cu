@@ -1280,7 +1280,6 @@ void plan_resident(dsmc_sim* h) {
   h->res_dirty = false;
 }
 
-
 // n steps of a resident launch.  Where the launch is refused (a stream that has only some of the
 // SMs, for which the plan's queries do not ask), nothing has run: the handle's steps take the span
 // passes from then on (res.cl = 0).
